@@ -10,6 +10,7 @@ import concurrent.futures as cf
 import os
 import shutil
 import subprocess
+import sys
 from pathlib import Path
 
 PKG = Path(__file__).resolve().parent
@@ -20,7 +21,7 @@ BUILD = PKG.parent / "_build"
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVFLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC,-O2", "--expt-relaxed-constexpr",
-           "-I", str(CSRC), "-I", str(INCLUDE)]
+           "-I", str(CSRC), "-I", str(INCLUDE), "-I", str(BUILD)]
 SOURCES = ["sweep.cu", "pass_fused.cu", "pass_pair.cu", "measure.cu", "api.cu", "measure_static.cu", "batch.cu",
            "cv_conv.cu", "cv_ops.cu", "gcv.cu", "batch_gcv.cu"]
 
@@ -45,6 +46,9 @@ def build(force: bool = False, verbose: bool = False) -> Path:
         return LIB
     BUILD.mkdir(exist_ok=True)
     nv = nvcc()
+    # the FP64 deviate's table, included by device_common.cuh (about a second)
+    subprocess.run([sys.executable, str(CSRC / "gen_erfcinv_f64.py"),
+                    str(BUILD / "erfcinv_f64_table.inc")], check=True)
 
     def compile_one(src):
         obj = BUILD / (Path(src).stem + ".o")
@@ -72,6 +76,5 @@ def build(force: bool = False, verbose: bool = False) -> Path:
 
 
 if __name__ == "__main__":
-    import sys
     build(force=True, verbose="-v" in sys.argv)
     print(LIB)
