@@ -103,6 +103,13 @@ int coulps_lattice_info(coulps_lattice_t lat, int64_t info[13]);
 
 /* Tile shape of the half-sweep kernel: ty rows of y per CTA, dz planes of z
  * per CTA (0 = keep).  Used by the autotuner; results do not depend on it.
+ * A lattice on which no tile and no fused mode was set runs its compound
+ * sweeps (aligned schedule, profiling off) with each chain held in the shared
+ * memory of a cluster of CTAs wherever that is the faster way (small chains);
+ * any call of coulps_set_tile, coulps_set_pass_tile, coulps_set_pair_tile or
+ * coulps_set_fused that succeeds selects the tiled kernels instead.  Fields
+ * are bitwise the same, samples up to the order of the FP64 sums over the
+ * charges.
  * Errors: EINVAL (ty*W/4 > 256 threads, ty < 1, dz < 1). */
 int coulps_set_tile(coulps_lattice_t lat, int ty, int dz);
 

@@ -77,6 +77,10 @@ struct coulps_lattice {
   // pair CTA) and maps on field / field2 with boxes ty + 8 and ty + 6 rows
   Tile qtile = {0, 0};
   CUtensorMap tm_q1[2], tm_q0[2];
+  // small lattices run resident (resident.cu) unless the caller has chosen a
+  // tile or a fused mode, which names the march kernels
+  ResidentPlan rplan;  // cluster = 0: the march kernels
+  bool pinned = false;
   size_t bytes = 0;
   int n_charge_sets = 0;
   // measured compound sweep captured as a graph
@@ -288,6 +292,38 @@ Tile fill_grid(const Geometry &g, Tile t, int target, int min_dz) {
   return t;
 }
 
+// The resident plan of a lattice: the cluster size with the shortest compound
+// sweep of 1 heatbath : 3 over-relaxation passes; {cluster = 0} if the chain
+// fits no cluster.
+ResidentPlan resident_plan(const Geometry &g) {
+  ResidentPlan best;
+  double t_best = 0.0;
+  for (int C = 1; C <= kMaxCluster && C <= g.Lz; ++C) {
+    ResidentPlan p;
+    if (!resident_shape(g, C, &p)) continue;
+    const double t = resident_time(g, p, 1, 3);
+    if (best.cluster == 0 || t < t_best) {
+      t_best = t;
+      best = p;
+    }
+  }
+  return best;
+}
+
+// Time of a compound sweep by the march kernels (us): launches of 5 us at
+// least each, then the work of their passes.  Fitted to measured sweeps
+// (FP32 1:3: 64^3 x 1 37.4, x 12 62, x 64 163, 72^3 x 30 137; 1:0: 19, 23,
+// 58, 48; FP64 1:3: 64^3 x 1 153, 40^3 x 30 185, 80^3 x 4 329; 1:0: 48, 72,
+// 115), for FP64 on the low side.
+double march_time(const Geometry &g, int n_hb, int n_or) {
+  const double sites = 2.0 * (double)g.colour_elems * g.n_chains;
+  const int trips = (n_or + 1) / 2;
+  if (g.precision == COULPS_F32)
+    return std::max(5.0 * (2 * n_hb + 2) + 9.0 * trips,
+                    15.0 + 5.0 * trips + sites * (2.8e-6 * n_hb + 1.9e-6 * n_or));
+  return std::max(38.0 * n_hb + 19.0 * n_or, sites * (4.0e-5 * n_hb + 2.5e-5 * n_or));
+}
+
 int rebuild_pass_maps(coulps_lattice *L) {
   if (!L->fused) return COULPS_OK;
   for (int b = 0; b < 2; ++b) {
@@ -362,11 +398,27 @@ PassPlan pass_plan(const coulps_lattice *L, int n_hb, int n_or) {
   return P;
 }
 
-// The tile by which the last kernel of a measured compound sweep (aligned
-// schedule) gathers Q and P: the pass pair's, the fused pass's, or the
-// half-sweep's.
+// Whether compound sweeps of this mix run resident now: where that is clearly
+// the shorter way (profiling times the march kernels one by one, the other
+// schedules are theirs).  The same for every number of sweeps, so that a run
+// gives bitwise the same samples however it is divided into calls.  Measured
+// (us per compound sweep, march against resident): FP64 16^3 x 1 94 -> 7.7
+// (1:0 39 -> 2.7), 32^3 x 1 112 -> 28, 40^3 x 30 185 -> 177; FP32 16^3 x 1
+// 31 -> 4.7, 64^3 x 1 37 -> 18, x 30 94 -> 58, x 64 163 -> 112, 80^3 x 12 79 ->
+// 67, and past the line 80^3 x 30 147 -> 166, FP64 64^3 x 4 172 -> 177.
+bool resident_on(const coulps_lattice *L, int n_hb, int n_or) {
+  if (L->rplan.cluster == 0 || L->pinned || L->profiling ||
+      L->schedule != COULPS_SCHEDULE_ALIGNED || n_hb + n_or == 0)
+    return false;
+  return resident_time(L->g, L->rplan, n_hb, n_or) < 0.9 * march_time(L->g, n_hb, n_or);
+}
+
+// The tile by which a measured compound sweep (aligned schedule) gathers Q
+// and P: one column of planes (resident), or that of its last kernel, the
+// pass pair's, the fused pass's, or the half-sweep's.
 Tile fused_gather_tile(const coulps_lattice *L, int n_hb, int n_or) {
   const int n = n_hb + n_or;
+  if (resident_on(L, n_hb, n_or)) return Tile{L->g.Ly, L->g.Lz};
   const PassPlan P = pass_plan(L, n_hb, n_or);
   if (P.head + 2 * P.pairs + P.singles < n || P.pairs + P.singles == 0) return L->tile;
   return P.singles > 0 ? L->ptile : L->qtile;
@@ -580,6 +632,43 @@ int enqueue_part(coulps_lattice *L, cudaStream_t st, int n_hb, int n_or, coulps_
   return COULPS_OK;
 }
 
+// n_sweeps compound sweeps of every chain (each sampled when `fuse` is given)
+// by the resident kernel, in launches of at most kResidentSweeps (a launch of
+// the largest resident lattices then lasts some 0.1 s).
+constexpr int kResidentSweeps = 2048;
+
+int enqueue_resident(coulps_lattice *L, int n_sweeps, int n_hb, int n_or, coulps_charges *fuse) {
+  ResidentArgs a = {};
+  const Geometry &g = L->g;
+  a.field = L->field;
+  a.Lx = g.Lx; a.Ly = g.Ly; a.Lz = g.Lz; a.W = g.W; a.Wq = g.Wq;
+  a.n_chains = g.n_chains;
+  a.n_hb = n_hb;
+  a.n_or = n_or;
+  const PhiloxKeys K = philox_keys((uint32_t)(L->seed & 0xffffffffu), (uint32_t)(L->seed >> 32));
+  for (int i = 0; i < 20; ++i) a.round_keys[i] = K.k[i];
+  a.pass_ptr = L->d_pass;
+  a.chain_elems = g.chain_elems;
+  a.colour_elems = g.colour_elems;
+  a.err = L->d_err;
+  if (fuse) {
+    if (fuse->gather_dirty || fuse->gather_tile.ty != g.Ly || fuse->gather_tile.dz != g.Lz)
+      return COULPS_EINVAL;
+    a.g_off = fuse->d_goff;
+    a.g_ent = fuse->d_gent;
+    a.g_q = fuse->d_gq;
+    a.stats = fuse->d_stats;
+    a.log = fuse->d_log;
+    a.log_cap = fuse->log_cap;
+  }
+  for (int done = 0; done < n_sweeps; done += kResidentSweeps) {
+    a.n_sweeps = std::min(kResidentSweeps, n_sweeps - done);
+    CK(launch_resident(g, L->rplan, a, fuse ? fuse->n : 0, L->stream));
+    CK(launch_advance_pass(L->d_pass, (uint32_t)a.n_sweeps * (uint32_t)(n_hb + n_or), L->stream));
+  }
+  return COULPS_OK;
+}
+
 // One compound sweep of every chain (and its sample when `fuse` is given).
 // With k > 1 streams chain c runs on stream c % k: stream 0 is the lattice's,
 // the others are forked from it at the start and joined back at the end
@@ -587,6 +676,7 @@ int enqueue_part(coulps_lattice *L, cudaStream_t st, int n_hb, int n_or, coulps_
 // kernels can share the GPU; each chain's passes, draws and sample are
 // unchanged.  The pass counter is advanced once, after the join.
 int enqueue_compound(coulps_lattice *L, int n_hb, int n_or, coulps_charges *fuse = nullptr) {
+  if (resident_on(L, n_hb, n_or)) return enqueue_resident(L, 1, n_hb, n_or, fuse);
   const int k = L->split < L->g.n_chains ? L->split : L->g.n_chains;
   if (k >= 2) {
     CK(cudaEventRecord(L->ev_fork, L->stream));
@@ -1133,6 +1223,8 @@ int coulps_set_allocator(coulps_alloc_fn alloc, coulps_free_fn free_fn, void *ct
   return COULPS_OK;
 }
 
+static int set_fused(coulps_lattice *L, int enable);
+
 int coulps_lattice_create(int Lx, int Ly, int Lz, int n_chains, int precision, uint64_t seed,
                           void *stream, coulps_lattice_t *out) {
   if (!out) return COULPS_EINVAL;
@@ -1177,8 +1269,9 @@ int coulps_lattice_create(int Lx, int Ly, int Lz, int n_chains, int precision, u
     coulps_lattice_destroy(L);
     return COULPS_ECUDA;
   }
+  L->rplan = resident_plan(g);
   int st = rebuild_maps(L);
-  if (!st) st = coulps_set_fused(L, 3);
+  if (!st) st = set_fused(L, 3);
   if (st) {
     coulps_lattice_destroy(L);
     return st;
@@ -1189,6 +1282,12 @@ int coulps_lattice_create(int Lx, int Ly, int Lz, int n_chains, int precision, u
 
 int coulps_set_fused(coulps_lattice_t L, int enable) {
   if (!L || enable < 0 || enable > 4) return COULPS_EINVAL;
+  const int st = set_fused(L, enable);
+  if (!st) L->pinned = true;
+  return st;
+}
+
+static int set_fused(coulps_lattice *L, int enable) {
   const size_t fbytes = L->g.chain_elems * L->g.es * (size_t)L->g.n_chains;
   drop_graph(L);
   if (!enable) {
@@ -1223,6 +1322,7 @@ int coulps_set_pair_tile(coulps_lattice_t L, int ty, int dz) {
   if (pair_threads(L->g, t) > max_threads) return COULPS_EINVAL;
   if (pair_smem_bytes(L->g, t, true) > 227 * 1024) return COULPS_EINVAL;
   drop_graph(L);
+  L->pinned = true;
   L->qtile = t;
   return rebuild_pass_maps(L);
 }
@@ -1241,6 +1341,7 @@ int coulps_set_pass_tile(coulps_lattice_t L, int ty, int dz) {
   if (pass_threads(L->g, t) > 512) return COULPS_EINVAL;
   if (pass_smem_bytes(L->g, t, true) > 227 * 1024) return COULPS_EINVAL;
   drop_graph(L);
+  L->pinned = true;
   L->ptile = t;
   return rebuild_pass_maps(L);
 }
@@ -1294,6 +1395,7 @@ int coulps_set_tile(coulps_lattice_t L, int ty, int dz) {
   if ((L->g.W / 4) * t.ty > 256) return COULPS_EINVAL;
   if (halfsweep_smem_bytes(L->g, t, true) > 227 * 1024) return COULPS_EINVAL;
   L->tile = t;
+  L->pinned = true;
   drop_graph(L);
   return rebuild_maps(L);
 }
@@ -1363,6 +1465,11 @@ int coulps_field_set(coulps_lattice_t L, int chain, const double *host) {
 
 int coulps_sweep(coulps_lattice_t L, int n_compound, int n_hb, int n_or) {
   if (!L || n_compound < 0 || n_hb < 0 || n_or < 0) return COULPS_EINVAL;
+  if (resident_on(L, n_hb, n_or)) {
+    const int st = enqueue_resident(L, n_compound, n_hb, n_or, nullptr);
+    if (!st) L->pass += (uint64_t)n_compound * (uint64_t)(n_hb + n_or);
+    return st;
+  }
   for (int k = 0; k < n_compound; ++k) {
     int st = enqueue_compound(L, n_hb, n_or);
     if (st) return st;
@@ -1516,6 +1623,11 @@ int coulps_run(coulps_lattice_t L, coulps_charges_t C, int n_therm, int n_meas, 
   }
   if (fused && n_meas >= 2 && shifted_ok(L, n_hb, n_or)) {
     st = run_shifted(L, C, n_meas, n_hb, n_or);
+    if (!st) L->pass += (uint64_t)n_meas * P;
+    return st;
+  }
+  if (fused && resident_on(L, n_hb, n_or)) {
+    st = enqueue_resident(L, n_meas, n_hb, n_or, C);
     if (!st) L->pass += (uint64_t)n_meas * P;
     return st;
   }

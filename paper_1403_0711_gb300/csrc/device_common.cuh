@@ -328,8 +328,9 @@ __device__ __forceinline__ void chain_QP(const double *__restrict__ partials, in
 // cancelling difference of Eq. (nsum2)), then the running sums, the batch
 // sums (kBatchMin..2*kBatchMin batches; neighbours merge and the batch length
 // doubles when 2*kBatchMin complete) and, if row != nullptr, the log row.
-// Adds the sample e to one chain's running sums and batch means.
-__device__ __forceinline__ void record_value(double *st, double e, int *err) {
+// Adds the sample e to one chain's running sums st[0 .. kStatBatch0) and batch
+// sums (kept apart so that a caller may hold the former in registers).
+__device__ __forceinline__ void record_value(double *st, double *batch, double e, int *err) {
   if (!isfinite(e)) atomicOr(err, kErrNonFinite);
   st[kStatLast] = e;
   st[kStatN] += 1.0;
@@ -339,19 +340,23 @@ __device__ __forceinline__ void record_value(double *st, double e, int *err) {
   st[kStatCurN] += 1.0;
   if (st[kStatCurN] >= st[kStatBatchLen]) {
     int nb = (int)st[kStatNBatch];
-    st[kStatBatch0 + nb] = st[kStatCurSum];
+    batch[nb] = st[kStatCurSum];
     st[kStatCurSum] = 0.0;
     st[kStatCurN] = 0.0;
     ++nb;
     if (nb == 2 * kBatchMin) {
       for (int i = 0; i < kBatchMin; ++i)
-        st[kStatBatch0 + i] = st[kStatBatch0 + 2 * i] + st[kStatBatch0 + 2 * i + 1];
-      for (int i = kBatchMin; i < 2 * kBatchMin; ++i) st[kStatBatch0 + i] = 0.0;
+        batch[i] = batch[2 * i] + batch[2 * i + 1];
+      for (int i = kBatchMin; i < 2 * kBatchMin; ++i) batch[i] = 0.0;
       nb = kBatchMin;
       st[kStatBatchLen] *= 2.0;
     }
     st[kStatNBatch] = (double)nb;
   }
+}
+
+__device__ __forceinline__ void record_value(double *st, double e, int *err) {
+  record_value(st, st + kStatBatch0, e, err);
 }
 
 // Eq. (nsum2) sample e = Q^2 - P, logged to row when it is not null.

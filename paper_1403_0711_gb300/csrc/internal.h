@@ -124,6 +124,43 @@ size_t pair_smem_bytes(const Geometry &g, const Tile &t, bool a_or);
 // largest thread count of a pair CTA (FP32 / FP64)
 constexpr int kPairMaxThreads32 = 512, kPairMaxThreads64 = 256;
 
+// Resident sweeps (resident.cu): n_sweeps compound sweeps of every chain in
+// one launch, a cluster of CTAs holding each chain in shared memory.  With
+// stats each sweep is also sampled: the charges grouped by z plane (entries of
+// plane z: [g_off[z], g_off[z + 1]), packed as in SweepArgs).
+constexpr int kMaxCluster = 16;
+constexpr int kResMaxSmem = 227 * 1024;
+struct ResidentArgs {
+  void *field;
+  int Lx, Ly, Lz, W, Wq, n_chains;
+  int cluster, run, meas_warps;  // set by launch_resident
+  int n_sweeps, n_hb, n_or;
+  uint32_t round_keys[20];
+  const uint32_t *pass_ptr;
+  size_t chain_elems, colour_elems;
+  int *err;
+  const uint32_t *g_off, *g_ent;
+  const double *g_q;
+  double *stats, *log;
+  int64_t log_cap;
+};
+struct ResidentPlan {
+  int cluster = 0;  // CTAs per chain
+  int threads = 0;  // sweeping threads per CTA
+  int run = 1;      // planes a thread marches at a time
+  bool single = false;  // one item per thread, deviates by warps of their own
+  int active = 0;   // clusters the GPU holds at once
+  size_t smem = 0;
+  double steps = 0.0;  // steps of a thread per half-sweep
+};
+// The plan with clusters of C CTAs; false if the chain does not fit them.
+bool resident_shape(const Geometry &g, int C, ResidentPlan *p);
+// Estimated time (us) of a compound sweep of every chain.
+double resident_time(const Geometry &g, const ResidentPlan &p, int n_hb, int n_or);
+// n_q: charges of the measured set (0 without)
+cudaError_t launch_resident(const Geometry &g, const ResidentPlan &p, ResidentArgs a, int64_t n_q,
+                            cudaStream_t s);
+
 // Phase-shifted schedule: chain k belongs to group k % groups; per group the
 // launch does nothing (mode 0), a heatbath (1) or an over-relaxation (2)
 // half-sweep with pass index *pass_ptr + pass_delta, gathering Q, P if
