@@ -2268,28 +2268,25 @@ int coulps_gcv_create(coulps_charges_t C, int n_iter, int R, coulps_gcv_t *out) 
     coulps_gcv_destroy(G);
     return COULPS_ENOMEM;
   }
-  // the charge density from the set's host copy (natural order)
-  std::vector<double> rho;
-  try {
-    rho.assign(n, 0.0);
-  } catch (...) {
-    coulps_gcv_destroy(G);
-    return COULPS_ENOMEM;
+  // the charge density from the set's host copy
+  cudaError_t e = cudaSuccess;
+  if (G->R > 0)
+    e = cudaMemcpyAsync(G->d_k, kt.data(), kt.size() * sizeof(float), cudaMemcpyHostToDevice,
+                        L->stream);
+  if (e == cudaSuccess) {
+    try {
+      e = gcv_solve(g, C->n, C->sites.data(), C->qv.data(), G->d_rho, G->d_u, G->d_h32, G->d_v,
+                    G->d_scratch, G->nblk_red, n_iter, G->d_c0res, L->alloc, L->stream);
+    } catch (...) {  // host memory
+      e = cudaErrorMemoryAllocation;
+    }
   }
-  for (size_t i = 0; i < C->qv.size(); ++i) {
-    const int32_t *s = &C->sites[3 * i];
-    rho[((size_t)s[2] * g.Ly + s[1]) * g.Lx + s[0]] += C->qv[i];
-  }
-  if (cudaMemcpyAsync(G->d_rho, rho.data(), n * sizeof(double), cudaMemcpyHostToDevice,
-                      L->stream) != cudaSuccess ||
-      (G->R > 0 && cudaMemcpyAsync(G->d_k, kt.data(), kt.size() * sizeof(float),
-                                   cudaMemcpyHostToDevice, L->stream) != cudaSuccess) ||
-      gcv_solve(g, G->d_rho, G->d_u, G->d_h32, G->d_v, G->d_scratch, G->nblk_red, n_iter,
-                G->d_c0res, L->stream) != cudaSuccess ||
-      cudaStreamSynchronize(L->stream) != cudaSuccess) {  // rho is pageable host memory
+  const cudaError_t es = cudaStreamSynchronize(L->stream);  // kt is pageable host memory
+  if (e == cudaSuccess) e = es;
+  if (e != cudaSuccess) {
     cudaGetLastError();
     coulps_gcv_destroy(G);
-    return COULPS_ECUDA;
+    return e == cudaErrorMemoryAllocation ? COULPS_ENOMEM : COULPS_ECUDA;
   }
   *out = G;
   return COULPS_OK;

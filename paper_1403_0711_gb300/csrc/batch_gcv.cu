@@ -12,9 +12,8 @@
 // Work per sample, all systems at once: the v . phi sums over fixed-size
 // chunks of the batch's field array (one CTA per chunk, chunks never cross a
 // system), one warp per charge for q phi and q^2 phi w, and one warp per
-// system adding its chunks and charges in a fixed order.  The SOR update is
-// the lattice solver's (same formula, same colour order), so a system's h is
-// the one coulps_gcv_create makes for the same box and charges.
+// system adding its chunks and charges in a fixed order.  The SOR solve is the
+// lattice solver's (sor.cu), so a system's h is the one coulps_gcv_create makes for the same box and charges.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -24,6 +23,7 @@
 #include "batch_internal.h"
 #include "device_common.cuh"
 #include "internal.h"
+#include "sor.cuh"
 
 namespace coulps {
 namespace {
@@ -36,7 +36,6 @@ struct BgcvSystem {
   long long nat_off;       // first site of the system in the natural-order arrays
   long long field_off;     // first element of the system's field in the batch layout
   long long colour_elems;  // Lz Ly W
-  double omega;            // SOR factor of the box
 };
 
 struct BgcvChunk {
@@ -47,25 +46,6 @@ struct BgcvChunk {
 __device__ __forceinline__ double nat_at(const double *u, const BgcvSystem &S, int x, int y, int z) {
   if (x < 0 || y < 0 || z < 0 || x >= S.Lx || y >= S.Ly || z >= S.Lz) return 0.0;
   return u[((size_t)z * S.Ly + y) * S.Lx + x];
-}
-
-// one red/black SOR half-sweep of A u = -rho in every system (blockIdx.y)
-__global__ void bgcv_sor_kernel(double *__restrict__ u, const double *__restrict__ rho,
-                                const BgcvSystem *__restrict__ sys, int colour) {
-  const BgcvSystem S = sys[blockIdx.y];
-  double *us = u + S.nat_off;
-  const double *rs = rho + S.nat_off;
-  const int64_t n = (int64_t)S.Lx * S.Ly * S.Lz;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const int x = (int)(i % S.Lx), y = (int)((i / S.Lx) % S.Ly),
-              z = (int)(i / ((int64_t)S.Lx * S.Ly));
-    if (((x + y + z) & 1) != colour) continue;
-    const double sum = nat_at(us, S, x - 1, y, z) + nat_at(us, S, x + 1, y, z) +
-                       nat_at(us, S, x, y - 1, z) + nat_at(us, S, x, y + 1, z) +
-                       nat_at(us, S, x, y, z - 1) + nat_at(us, S, x, y, z + 1);
-    us[i] = (1.0 - S.omega) * us[i] + S.omega * (sum - rs[i]) / 6.0;
-  }
 }
 
 // block sums of (a, b) in a fixed order; thread 0 returns them
@@ -504,10 +484,6 @@ int coulps_batch_gcv_create(coulps_batch_t B, int n_iter, int R, coulps_batch_gc
     g.nat_off = nat;
     g.field_off = S.field_off;
     g.colour_elems = S.colour_elems;
-    // SOR factor from the Jacobi spectral radius of the Dirichlet box
-    const double rj = (std::cos(M_PI / (S.Lx + 1)) + std::cos(M_PI / (S.Ly + 1)) +
-                       std::cos(M_PI / (S.Lz + 1))) / 3.0;
-    g.omega = 2.0 / (1.0 + std::sqrt(1.0 - rj * rj));
     G->sys.push_back(g);
     nat += (long long)S.Lx * S.Ly * S.Lz;
     G->chunk_begin[s] = (int)G->chunks.size();
@@ -549,12 +525,15 @@ int coulps_batch_gcv_create(coulps_batch_t B, int n_iter, int R, coulps_batch_gc
       !G->d_qpart || !G->d_tg || !G->d_cvstats || !d_rho || !d_u || !d_scale)
     return fail(COULPS_ENOMEM);
   // host side: charge density, per-charge sites, the cube kernel and cP
-  std::vector<double> rho, cP(n_sys, 0.0);
+  std::vector<double> cP(n_sys, 0.0);
+  std::vector<SorBox> boxes;
+  std::vector<SorCharge> charges;
   std::vector<int4> qsite;
   std::vector<float> kt;
   try {
-    rho.assign((size_t)nat, 0.0);
     qsite.resize((size_t)G->n_q);
+    boxes.reserve(n_sys);
+    charges.reserve((size_t)G->n_q);
   } catch (...) {
     return fail(COULPS_ENOMEM);
   }
@@ -570,6 +549,7 @@ int coulps_batch_gcv_create(coulps_batch_t B, int n_iter, int R, coulps_batch_gc
     return fail(COULPS_ENOMEM);
   }
   std::vector<int64_t> perm;
+  long long sor_off = 0;
   for (int s = 0; s < n_sys; ++s) {
     const BgcvSystem &g = G->sys[s];
     perm.clear();
@@ -579,11 +559,11 @@ int coulps_batch_gcv_create(coulps_batch_t B, int n_iter, int R, coulps_batch_gc
       return ((int64_t)p[2] * g.Ly + p[1]) * g.Lx + p[0];
     };
     std::stable_sort(perm.begin(), perm.end(), [&](int64_t a, int64_t b) { return key(a) < key(b); });
-    // rho in the charges' input order (as the single-lattice solver adds them)
-    for (int64_t i = B->offsets[s]; i < B->offsets[s + 1]; ++i) {
-      const int32_t *p = &B->sites[3 * i];
-      rho[g.nat_off + ((size_t)p[2] * g.Ly + p[1]) * g.Lx + p[0]] += B->q[i];
-    }
+    // the box's charges for the solve (as the single-lattice solver takes them)
+    boxes.push_back(sor_box(g.Lx, g.Ly, g.Lz, sor_off, g.nat_off));
+    sor_off += sor_elems(boxes.back());
+    sor_charges(boxes.back(), B->offsets[s + 1] - B->offsets[s],
+                B->sites.data() + 3 * B->offsets[s], B->q.data() + B->offsets[s], charges);
     for (size_t k = 0; k < perm.size(); ++k) {
       const int64_t i = perm[k], o = B->offsets[s] + (int64_t)k;
       const int32_t *p = &B->sites[3 * i];
@@ -607,16 +587,20 @@ int coulps_batch_gcv_create(coulps_batch_t B, int n_iter, int R, coulps_batch_gc
       !up(G->d_qsite, qsite.data(), qsite.size() * sizeof(int4)) ||
       !up(G->d_q, qs.data(), qs.size() * sizeof(double)) ||
       !up(G->d_cP, cP.data(), cP.size() * sizeof(double)) ||
-      !up(d_rho, rho.data(), rho.size() * sizeof(double)) ||
       (G->R > 0 && !up(G->d_k, kt.data(), kt.size() * sizeof(float))))
     return fail(COULPS_ECUDA);
   // SOR on every system at once, then residual and max |u| per system
-  if (cudaMemsetAsync(d_u, 0, (size_t)nat * sizeof(double), st) != cudaSuccess)
-    return fail(COULPS_ECUDA);
+  cudaError_t se;
+  try {
+    se = sor_solve(boxes, charges, n_iter, d_u, d_rho, B->alloc, st);
+  } catch (...) {  // host memory
+    se = cudaErrorMemoryAllocation;
+  }
+  if (se != cudaSuccess) {
+    cudaGetLastError();
+    return fail(se == cudaErrorMemoryAllocation ? COULPS_ENOMEM : COULPS_ECUDA);
+  }
   const dim3 sgrid(32, n_sys);
-  for (int it = 0; it < n_iter; ++it)
-    for (int c = 0; c < 2; ++c)
-      bgcv_sor_kernel<<<sgrid, 256, 0, st>>>(d_u, d_rho, G->d_sys, c);
   bgcv_check_kernel<<<n_sys, kBgcvThreads, 0, st>>>(d_u, d_rho, G->d_sys, G->d_res);
   std::vector<double> res(3 * (size_t)n_sys);
   if (cudaGetLastError() != cudaSuccess ||

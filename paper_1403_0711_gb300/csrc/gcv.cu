@@ -5,7 +5,7 @@
 // h = -G rho it equals Q^2 - rho.G.rho, so e - T g = rho.G.rho - P: the far
 // pairs' part of the variance of the Eq. (nsum2) sample is gone and only that
 // of P = sum_i (q_i phi_i)^2 is left.  h comes from red/black SOR on
-// A h = -rho (once per charge set); the estimator stays unbiased whatever the
+// A h = -rho (sor.cu, once per charge set); the estimator stays unbiased whatever the
 // solver's residual, which only sets how much variance is removed.
 //
 // A second, local term removes most of the variance of P: g^P_x =
@@ -26,6 +26,7 @@
 
 #include "device_common.cuh"
 #include "internal.h"
+#include "sor.cuh"
 
 namespace coulps {
 namespace {
@@ -36,21 +37,6 @@ __device__ __forceinline__ double nat_at(const double *u, int Lx, int Ly, int Lz
                                          int z) {
   if (x < 0 || y < 0 || z < 0 || x >= Lx || y >= Ly || z >= Lz) return 0.0;
   return u[((size_t)z * Ly + y) * Lx + x];
-}
-
-// one red/black SOR half-sweep of A u = -rho (natural order, FP64)
-__global__ void gcv_sor_kernel(double *__restrict__ u, const double *__restrict__ rho, int Lx,
-                               int Ly, int Lz, int colour, double omega) {
-  const int64_t n = (int64_t)Lx * Ly * Lz;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const int x = (int)(i % Lx), y = (int)((i / Lx) % Ly), z = (int)(i / ((int64_t)Lx * Ly));
-    if (((x + y + z) & 1) != colour) continue;
-    const double S = nat_at(u, Lx, Ly, Lz, x - 1, y, z) + nat_at(u, Lx, Ly, Lz, x + 1, y, z) +
-                     nat_at(u, Lx, Ly, Lz, x, y - 1, z) + nat_at(u, Lx, Ly, Lz, x, y + 1, z) +
-                     nat_at(u, Lx, Ly, Lz, x, y, z - 1) + nat_at(u, Lx, Ly, Lz, x, y, z + 1);
-    u[i] = (1.0 - omega) * u[i] + omega * (S - rho[i]) / 6.0;
-  }
 }
 
 __device__ __forceinline__ void block_sum2(double a, double b, double *out) {
@@ -287,21 +273,18 @@ int gcv_blocks(const Geometry &g) {
   return b;
 }
 
-cudaError_t gcv_solve(const Geometry &g, const double *rho_nat, double *u_nat, float *h32,
-                      float *v_layout, double *scratch, int nblk_red, int n_iter, double *res,
-                      cudaStream_t s) {
+cudaError_t gcv_solve(const Geometry &g, int64_t n_q, const int32_t *sites, const double *q,
+                      double *rho_nat, double *u_nat, float *h32, float *v_layout,
+                      double *scratch, int nblk_red, int n_iter, double *res,
+                      const Allocator &alloc, cudaStream_t s) {
   const int64_t n = (int64_t)g.Lx * g.Ly * g.Lz;
   const int threads = 256;
   const int blocks = (int)((n + threads - 1) / threads > 4096 ? 4096 : (n + threads - 1) / threads);
-  // SOR factor from the Jacobi spectral radius of the Dirichlet box
-  const double rj = (std::cos(M_PI / (g.Lx + 1)) + std::cos(M_PI / (g.Ly + 1)) +
-                     std::cos(M_PI / (g.Lz + 1))) / 3.0;
-  const double omega = 2.0 / (1.0 + std::sqrt(1.0 - rj * rj));
-  cudaError_t e = cudaMemsetAsync(u_nat, 0, sizeof(double) * n, s);
+  std::vector<SorBox> boxes{sor_box(g.Lx, g.Ly, g.Lz, 0, 0)};
+  std::vector<SorCharge> charges;
+  sor_charges(boxes[0], n_q, sites, q, charges);
+  cudaError_t e = sor_solve(boxes, charges, n_iter, u_nat, rho_nat, alloc, s);
   if (e != cudaSuccess) return e;
-  for (int it = 0; it < n_iter; ++it)
-    for (int c = 0; c < 2; ++c)
-      gcv_sor_kernel<<<blocks, threads, 0, s>>>(u_nat, rho_nat, g.Lx, g.Ly, g.Lz, c, omega);
   gcv_check_kernel<<<nblk_red, kGcvThreads, 0, s>>>(u_nat, rho_nat, g.Lx, g.Ly, g.Lz, scratch);
   gcv_check_sums_kernel<<<1, 32, 0, s>>>(scratch, nblk_red, res);
   double hres[3] = {0, 0, 0};

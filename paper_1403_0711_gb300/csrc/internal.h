@@ -201,21 +201,23 @@ struct SetTable {
 cudaError_t launch_measure_sets(const Geometry &g, const void *field, const SetTable &t,
                                 int *err, cudaStream_t s);
 
-// Global control variate (gcv.cu).  gcv_solve: red/black SOR on A u = -rho
-// (natural order, FP64, u_nat and rho_nat Lx*Ly*Lz doubles), h32 = u rounded
-// to a fixed-point grid (exact FP32), v_layout = A h32 (exact in FP32) in one
+struct Allocator;
+// Global control variate (gcv.cu).  gcv_solve: red/black SOR on A u = -rho for
+// the n_q charges (host sites and values; u and rho are left in u_nat and
+// rho_nat, natural order, Lx*Ly*Lz doubles), h32 = u rounded to a fixed-point grid (exact FP32), v_layout = A h32 (exact in FP32) in one
 // chain's field layout (chain_elems floats), res[0] = h32 . rho,
 // res[1] = |A u + rho| / |rho|, res[2] = max |u| (res: 3 doubles); scratch
-// >= 4 * nblk_red doubles; synchronises once.  gcv_eval: per chain
+// >= 4 * nblk_red doubles; synchronises.  gcv_eval: per chain
 // T g = res[0] - Q (v . phi) into tg; partials >= 2 * nblk * n_chains
 // doubles, nblk = gcv_blocks(g).
 int gcv_blocks(const Geometry &g);
 // Dirichlet Green function of the (2R+1)^3 cube at its centre (FP32,
 // [dz][dy][dx] from -R; api.cu), the local P term's kernel.
 std::vector<float> cube_green(int R);
-cudaError_t gcv_solve(const Geometry &g, const double *rho_nat, double *u_nat, float *h32,
-                      float *v_layout, double *scratch, int nblk_red, int n_iter, double *res,
-                      cudaStream_t s);
+cudaError_t gcv_solve(const Geometry &g, int64_t n_q, const int32_t *sites, const double *q,
+                      double *rho_nat, double *u_nat, float *h32, float *v_layout,
+                      double *scratch, int nblk_red, int n_iter, double *res,
+                      const Allocator &alloc, cudaStream_t s);
 // With R > 0 also the local term of P (kt: (2R+1)^3 floats, index
 // (dz + R)(2R+1)^2 + (dy + R)(2R+1) + dx + R; cP = kt[centre] sum q^2; ppart
 // >= ceil(n_q / 8) * n_chains doubles).
