@@ -612,6 +612,30 @@ int coulps_cv_conv3d_tanh_rows(const void *in_bf16, const void *wpack, const flo
 int coulps_cv_conv3d_wgrad(const void *a_bf16, const void *dh_bf16, float *dW, int nb, int Lx,
                            int Ly, int Lz, float *scratch, int64_t scratch_floats, void *stream);
 
+/* Steps of a training pass between the convolutions and the batched products,
+ * each bitwise the framework operations that it stands for (device memory,
+ * 16-byte aligned unless said; asynchronous on stream; EINVAL, ECUDA):
+ *   pack_weights_dev  coulps_cv_pack_weights of w[16][16][27] in device memory
+ *                     into 27 * 256 BF16.
+ *   act_forward       a = tanh(h) in BF16 (8-byte aligned), s = 1 - a^2 rounded
+ *                     to a BF16 value, for n floats h, n a multiple of 4.
+ *   act_backward      dh = (da - 2 ds a)(1 - a^2), da BF16, ds FP32; either may
+ *                     be NULL (zero).
+ *   region_gather     left[q][n][c][o] = s[n][q + o][c] for the sites q of the
+ *                     box [lo, hi) (x fastest) of E = e[0] x e[1] x e[2], s of
+ *                     shape [nb][z][y][x][16], 0 outside E, o = 9 dz + 3 dy + dx + 13.
+ *   region_scatter    its transpose, ds[n][p][c] = sum over o = 26, 25, .. 0 of
+ *                     dleft[p - o][n][c][o]; EUNSUPPORTED if the box grown by one
+ *                     has more than 56320 sites. */
+int coulps_cv_pack_weights_dev(const float *w, void *out_bf16, void *stream);
+int coulps_cv_act_forward(const float *h, void *a_bf16, float *s, int64_t n, void *stream);
+int coulps_cv_act_backward(const float *h, const void *da_bf16, const float *ds, float *dh,
+                           int64_t n, void *stream);
+int coulps_cv_region_gather(const float *s, float *left, int nb, const int32_t *e,
+                            const int32_t *lo, const int32_t *hi, void *stream);
+int coulps_cv_region_scatter(const float *dleft, float *ds, int nb, const int32_t *e,
+                             const int32_t *lo, const int32_t *hi, void *stream);
+
 /* coulps_cv_pack_field: the net's input for every chain of an FP32 lattice,
  * on the lattice's stream: act[chain][z][y][x][16] BF16 = (phi, rho, rho phi,
  * 0, ...) and Aphi[chain][z][y][x] = (A phi) = 6 phi - (sum of the six neighbours),

@@ -55,6 +55,8 @@ EXPORTS = (
     "coulps_set_pair_tile", "coulps_pair_tile", "coulps_kernel_times_n",
     "coulps_batch_set_fused", "coulps_batch_set_pass_tiles", "coulps_batch_system_pass_tile",
     "coulps_batch_fused", "coulps_batch_set_pair_tiles", "coulps_batch_system_pair_tile",
+    "coulps_cv_pack_weights_dev", "coulps_cv_act_forward", "coulps_cv_act_backward",
+    "coulps_cv_region_gather", "coulps_cv_region_scatter",
 )
 SCHEDULE_ALIGNED, SCHEDULE_PHASED, SCHEDULE_SHIFTED = 0, 1, 2
 STAT_STRIDE = 72
@@ -189,6 +191,13 @@ def load(path: str | Path | None = None):
         "coulps_set_pair_tile": (i32, [vp, i32, i32]),
         "coulps_pair_tile": (i32, [vp, P(i32)]),
         "coulps_kernel_times_n": (i32, [vp, P(f64), i32]),
+        "coulps_cv_pack_weights_dev": (i32, [vp, vp, vp]),
+        "coulps_cv_act_forward": (i32, [vp, vp, vp, i64, vp]),
+        "coulps_cv_act_backward": (i32, [vp, vp, vp, vp, i64, vp]),
+        "coulps_cv_region_gather": (i32, [vp, vp, i32, P(ctypes.c_int32), P(ctypes.c_int32),
+                                          P(ctypes.c_int32), vp]),
+        "coulps_cv_region_scatter": (i32, [vp, vp, i32, P(ctypes.c_int32), P(ctypes.c_int32),
+                                           P(ctypes.c_int32), vp]),
         "coulps_cv_charge_term": (i32, [vp, vp, vp, vp, vp, i32, i32, P(ctypes.c_int32), i32, vp,
                                         i64, vp, vp]),
     }

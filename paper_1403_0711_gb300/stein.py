@@ -46,6 +46,13 @@ def _stream():
 
 def pack_weights(W: torch.Tensor) -> torch.Tensor:
     """(16,16,3,3,3) float -> packed BF16 bits on the device (coulps_cv_pack_weights)."""
+    if W.is_cuda:
+        w = W.detach().float().contiguous()
+        assert w.numel() == 27 * 256
+        out = torch.empty(27 * 256, dtype=torch.int16, device=W.device)
+        coulps._check(coulps.load().coulps_cv_pack_weights_dev(_vp(w), _vp(out), _stream()),
+                      "coulps_cv_pack_weights_dev")
+        return out
     w = np.ascontiguousarray(W.detach().float().cpu().numpy())
     out = np.zeros(27 * 256, dtype=np.uint16)
     st = coulps.load().coulps_cv_pack_weights(w.ctypes.data_as(ctypes.POINTER(ctypes.c_float)),
@@ -117,6 +124,61 @@ class Conv3dTC(torch.autograd.Function):
         if ctx.needs_input_grad[2]:
             db = dh.sum(dim=(0, 1, 2, 3))
         return da, dW, db
+
+
+class _Act(torch.autograd.Function):
+    """(tanh(h) in BF16, 1 - tanh(h)^2 rounded to BF16 values, gradient passed
+    straight through the rounding), bitwise the operations on CUDA FP32."""
+
+    @staticmethod
+    def forward(ctx, h):
+        h = h.contiguous()
+        a, s = torch.empty_like(h, dtype=torch.bfloat16), torch.empty_like(h)
+        coulps._check(coulps.load().coulps_cv_act_forward(_vp(h), _vp(a), _vp(s), h.numel(),
+                                                          _stream()), "coulps_cv_act_forward")
+        ctx.save_for_backward(h)
+        ctx.set_materialize_grads(False)
+        return a, s
+
+    @staticmethod
+    @torch.autograd.function.once_differentiable
+    def backward(ctx, da, ds):
+        h, = ctx.saved_tensors
+        if da is None and ds is None:
+            return None
+        da = None if da is None else da.contiguous()
+        ds = None if ds is None else ds.contiguous()
+        dh = torch.empty_like(h)
+        coulps._check(coulps.load().coulps_cv_act_backward(
+            _vp(h), None if da is None else _vp(da), None if ds is None else _vp(ds), _vp(dh),
+            h.numel(), _stream()), "coulps_cv_act_backward")
+        return dh
+
+
+class _Neighbours(torch.autograd.Function):
+    """(n, m, 27, 16) neighbours of the sites [lo, hi) of s (n, Z, Y, X, 16), as
+    a view of the [m][n][16][27] layout that the batched product takes."""
+
+    @staticmethod
+    def forward(ctx, s, lo, hi):
+        s = s.contiguous()
+        n, Z, Y, X, _ = s.shape
+        ctx.box = [(ctypes.c_int32 * 3)(*v) for v in ((X, Y, Z), lo, hi)]
+        ctx.shape = s.shape
+        m = (hi[0] - lo[0]) * (hi[1] - lo[1]) * (hi[2] - lo[2])
+        left = torch.empty(m, n, 16, 27, dtype=s.dtype, device=s.device)
+        coulps._check(coulps.load().coulps_cv_region_gather(_vp(s), _vp(left), n, *ctx.box,
+                                                            _stream()), "coulps_cv_region_gather")
+        return left.permute(1, 0, 3, 2)
+
+    @staticmethod
+    @torch.autograd.function.once_differentiable
+    def backward(ctx, d):
+        d = d.permute(1, 0, 3, 2).contiguous()  # [m][n][16][27]: as it comes
+        ds = torch.empty(ctx.shape, dtype=d.dtype, device=d.device)
+        coulps._check(coulps.load().coulps_cv_region_scatter(_vp(d), _vp(ds), ctx.shape[0], *ctx.box,
+                                                             _stream()), "coulps_cv_region_scatter")
+        return ds, None, None
 
 
 def _face_masks():
@@ -473,6 +535,13 @@ def _axis_index(n, lo, hi):
     return out
 
 
+_SCATTER_SITES = 56320  # coulps_cv_region_scatter's most, of the box grown by one
+
+
+def _grown_sites(lo, hi):
+    return (hi[0] - lo[0] + 2) * (hi[1] - lo[1] + 2) * (hi[2] - lo[2] + 2)
+
+
 class LocalSteinCV(SteinCV):
     """SteinCV whose g is the net inside the box R = [lo, hi) (lattice x, y, z
     coordinates, half-open) and 0 elsewhere."""
@@ -529,16 +598,10 @@ class LocalSteinCV(SteinCV):
 
     # -- differentiable T g on E-sized inputs: x0 (n, ez, ey, ex, 16) BF16
     def stein_term(self, x0, Aphi, faces=True):
-        h1 = Conv3dTC.apply(x0, self._w1p(), self.b1)
-        a1 = torch.tanh(h1)
-        s1 = 1.0 - a1 * a1
-        h2 = Conv3dTC.apply(a1.to(torch.bfloat16), self.W2, self.b2)
-        a2 = torch.tanh(h2)
-        s2 = 1.0 - a2 * a2
-        g = Conv3dTC.apply(a2.to(torch.bfloat16), self._w3p(), self._b3p())[..., 0]
         # s rounded like the library kernel's BF16 copies (straight-through)
-        s1 = s1 + (s1.to(torch.bfloat16).float() - s1).detach()
-        s2 = s2 + (s2.to(torch.bfloat16).float() - s2).detach()
+        a1, s1 = _Act.apply(Conv3dTC.apply(x0, self._w1p(), self.b1))
+        a2, s2 = _Act.apply(Conv3dTC.apply(a1, self.W2, self.b2))
+        g = Conv3dTC.apply(a2, self._w3p(), self._b3p())[..., 0]
         div = self.region_divergence(s1, s2) + charge_term(
             charge_matrix(*self.weights()), s1, s2, self._cq, self._crho)
         return div - (g * Aphi * self._rmask).sum(dim=(1, 2, 3))
@@ -546,10 +609,15 @@ class LocalSteinCV(SteinCV):
     def region_divergence(self, s1, s2):
         """sum_{x in R} dg_x/dphi_x from s1, s2 (n, ez, ey, ex, 16): for each q
         next to R, s2[q] . (K_class(q) applied to the 27 neighbours of s1)."""
-        s1p = torch.nn.functional.pad(s1, (0, 0, 1, 1, 1, 1, 1, 1))
         qz, qy, qx = self._q[:, 0], self._q[:, 1], self._q[:, 2]
-        patches = torch.stack([s1p[:, qz + 1 + o[0], qy + 1 + o[1], qx + 1 + o[2]] for o in OFFS],
-                              dim=2)  # (n, m, 27, 16)
+        lo = [max(v - 1, 0) for v in self.r_lo]
+        hi = [min(v + 1, e) for v, e in zip(self.r_hi, self.edims)]
+        if s1.is_cuda and s1.dtype == torch.float32 and _grown_sites(lo, hi) <= _SCATTER_SITES:
+            patches = _Neighbours.apply(s1, lo, hi)  # the same sites in the order of _q
+        else:
+            s1p = torch.nn.functional.pad(s1, (0, 0, 1, 1, 1, 1, 1, 1))
+            patches = torch.stack([s1p[:, qz + 1 + o[0], qy + 1 + o[1], qx + 1 + o[2]]
+                                   for o in OFFS], dim=2)  # (n, m, 27, 16)
         Kq = self.region_kernels()[self._qcls]  # (m, 16 c2, 16 c1, 27)
         d = torch.einsum("nmec,mdce->nmd", patches, Kq)
         return (s2[:, qz, qy, qx] * d).sum(dim=(1, 2))
