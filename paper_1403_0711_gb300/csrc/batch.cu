@@ -98,7 +98,10 @@ constexpr int batch_quads_per_thread() {
 }
 
 template <typename T, bool OR, bool GATHER, int V>
-__global__ void __launch_bounds__(kBatchThreads) batch_halfsweep_kernel(const BatchArgs a) {
+// (two quads per thread: at most 80 registers, six CTAs of 128 threads per SM;
+// unbounded it takes 106 and a compound sweep of 256 systems 600 instead of 588 us)
+__global__ void __launch_bounds__(kBatchThreads, V == 2 ? 3 : 1)
+    batch_halfsweep_kernel(const BatchArgs a) {
   extern __shared__ unsigned char smem_raw[];
   unsigned char *smem = align_smem128(smem_raw);
   const PhiloxKeys &K = *reinterpret_cast<const PhiloxKeys *>(a.round_keys);

@@ -47,8 +47,22 @@ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, const PhiloxKeys &K) {
 
 // Small-side argument u = (t + 1/2) 2^-31 in (0, 1] and the sign of the
 // deviate: w < 2^31 means 2r < 1 and the deviate is -erfc^-1(u)/sqrt(3).
+// (A shift for the sign's mask and one three-input operation.)
 __device__ __forceinline__ uint32_t hb_small_side(uint32_t w) {
-  return ((w >> 31) ? ~w : w) & 0x7fffffffu;
+  return (w ^ (uint32_t)((int32_t)w >> 31)) & 0x7fffffffu;
+}
+// 2^31 - 1 less that
+__device__ __forceinline__ uint32_t hb_large_side(uint32_t w) {
+  return (w ^ ~(uint32_t)((int32_t)w >> 31)) & 0x7fffffffu;
+}
+
+// log2 of a normal number: __log2f's result without its scaling of
+// subnormals (three instructions a call), which the deviate's argument,
+// u (2 - u) >= 2^-32, never needs.
+__device__ __forceinline__ float log2_normal(float x) {
+  float y;
+  asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
 }
 
 // The two polynomials of q in FP32 Horner form; V is float or float2 (two
@@ -108,10 +122,9 @@ __device__ __forceinline__ V erfcinv_q_tail(V z) {  // z = sqrt(v) - 3.6, v >= 9
 // 22%, for one more term in the common polynomial.  Measured against FP64
 // erfc^-1 over the whole range: a few FP32 ulps.
 __device__ __forceinline__ float hb_noise_f32(uint32_t w) {
-  const uint32_t s = hb_small_side(w);
-  const float u = fmaf(__uint2float_rn(s), 0x1p-31f, 0x1p-32f);
-  const float x = fmaf(__uint2float_rn(0x7fffffffu - s), 0x1p-31f, 0x1p-32f);
-  const float v = -__log2f(fmaf(u, x, u));
+  const float u = fmaf(__uint2float_rn(hb_small_side(w)), 0x1p-31f, 0x1p-32f);
+  const float x = fmaf(__uint2float_rn(hb_large_side(w)), 0x1p-31f, 0x1p-32f);
+  const float v = -log2_normal(fmaf(u, x, u));
   float q;
   if (v < 9.0f)
     q = erfcinv_q_main(v - 4.5f);
@@ -122,34 +135,36 @@ __device__ __forceinline__ float hb_noise_f32(uint32_t w) {
   return xs * q;
 }
 
-// hb_noise_f32 of 2 NP words (pairs (w[0], w[1]), (w[2], w[3]), ...) with one
-// vote of the warp's active lanes for the tail over all of them, so the words'
-// independent chains can interleave; bitwise the same per word.
+// hb_noise_f32 of 2 NP words (pairs (w[0], w[1]), (w[2], w[3]), ...) as packed
+// pairs, bitwise the same per word.  All pairs' common polynomials come first
+// (independent chains), then one test of whether any of the thread's words is
+// in the tail: an ordinary branch, taken by a warp 12% of the time with NP = 2.
 template <int NP>
 __device__ __forceinline__ void hb_noise_pairs_f32(const uint32_t (&w)[2 * NP], float2 (&out)[NP]) {
   const float2 scale = make_float2(0x1p-31f, 0x1p-31f), half = make_float2(0x1p-32f, 0x1p-32f);
-  float2 x[NP], v[NP], q[NP];
-  bool tail = false;
+  float2 x[NP], l[NP], q[NP];  // l = log2 = -v
+  float least = 0.f;
 #pragma unroll
   for (int p = 0; p < NP; ++p) {
-    const uint32_t s0 = hb_small_side(w[2 * p]), s1 = hb_small_side(w[2 * p + 1]);
-    const float2 u =
-        __ffma2_rn(make_float2(__uint2float_rn(s0), __uint2float_rn(s1)), scale, half);
-    x[p] = __ffma2_rn(
-        make_float2(__uint2float_rn(0x7fffffffu - s0), __uint2float_rn(0x7fffffffu - s1)), scale,
-        half);
+    const float2 u = __ffma2_rn(make_float2(__uint2float_rn(hb_small_side(w[2 * p])),
+                                            __uint2float_rn(hb_small_side(w[2 * p + 1]))),
+                                scale, half);
+    x[p] = __ffma2_rn(make_float2(__uint2float_rn(hb_large_side(w[2 * p])),
+                                  __uint2float_rn(hb_large_side(w[2 * p + 1]))),
+                      scale, half);
     const float2 t = __ffma2_rn(u, x[p], u);
-    v[p] = make_float2(-__log2f(t.x), -__log2f(t.y));
-    q[p] = erfcinv_q_main(__fadd2_rn(v[p], make_float2(-4.5f, -4.5f)));
-    tail = tail || !(v[p].x < 9.0f) || !(v[p].y < 9.0f);
+    l[p] = make_float2(log2_normal(t.x), log2_normal(t.y));
+    // v - 4.5 = -l - 4.5, rounded once either way
+    q[p] = erfcinv_q_main(__ffma2_rn(l[p], make_float2(-1.f, -1.f), make_float2(-4.5f, -4.5f)));
+    least = fminf(least, fminf(l[p].x, l[p].y));
   }
-  if (__any_sync(__activemask(), tail)) {
+  if (least <= -9.0f) {
 #pragma unroll
     for (int p = 0; p < NP; ++p) {
       const float2 qt = erfcinv_q_tail(
-          __fadd2_rn(make_float2(sqrtf(v[p].x), sqrtf(v[p].y)), make_float2(-3.6f, -3.6f)));
-      q[p].x = v[p].x < 9.0f ? q[p].x : qt.x;
-      q[p].y = v[p].y < 9.0f ? q[p].y : qt.y;
+          __fadd2_rn(make_float2(sqrtf(-l[p].x), sqrtf(-l[p].y)), make_float2(-3.6f, -3.6f)));
+      q[p].x = l[p].x > -9.0f ? q[p].x : qt.x;
+      q[p].y = l[p].y > -9.0f ? q[p].y : qt.y;
     }
   }
 #pragma unroll

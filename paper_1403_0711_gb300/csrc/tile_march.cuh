@@ -105,23 +105,16 @@ __device__ __forceinline__ float2 pset(float c) { return make_float2(c, c); }
 __device__ __forceinline__ double2 pset(double c) { return make_double2(c, c); }
 
 // The heatbath deviates of one quad's four Philox words as two pairs (sites
-// 0, 1 and 2, 3): FP32 as packed pairs, each under its own tail vote of the
-// active lanes (no divergent branch per site), FP64 word by word.  Bitwise
-// those of Noise<T>::of per word.  A warp's vote over 64 words finds a tail
-// word (v >= 7, probability 0.0039 per word) 22% of the time, one over the
-// quad's 128 words 39%: measured at 128^3 x 64 chains, 0.1498 against 0.1538
-// ms per heatbath half-sweep with neighbour sums on packed pairs (before
-// those, the vote per quad measured faster than a vote per site: 0.156
-// against 0.159 ms).
+// 0, 1 and 2, 3): FP32 as packed pairs whose common polynomials run side by
+// side, with one branch for the quad's rare tail words; FP64 word by word.
+// Bitwise those of Noise<T>::of per word.  Measured at 128^3 x 64 chains, per
+// heatbath half-sweep: a warp vote per pair 142.4 us (139.6 with the shorter
+// logarithm and integer steps), this form 139.1.
 template <typename T> struct QuadNoise2;
 template <> struct QuadNoise2<float> {
   __device__ __forceinline__ static void of(uint4 w, float2 (&n)[2]) {
-    const uint32_t u0[2] = {w.x, w.y}, u1[2] = {w.z, w.w};
-    float2 a[1], b[1];
-    hb_noise_pairs_f32<1>(u0, a);
-    hb_noise_pairs_f32<1>(u1, b);
-    n[0] = a[0];
-    n[1] = b[0];
+    const uint32_t u[4] = {w.x, w.y, w.z, w.w};
+    hb_noise_pairs_f32<2>(u, n);
   }
 };
 template <> struct QuadNoise2<double> {
@@ -284,6 +277,25 @@ __device__ bool march_tile(const Job &j, const PhiloxKeys &K, unsigned char *sme
       while (issued < n_planes && issued - STAGES <= last_free) issue(issued++);
   };
 
+  // Everything of the plane loop that does not change from plane to plane is
+  // formed here, and what does advances by additions: byte offsets of this
+  // thread's quad in the slots of planes k and k + 1, the next plane's
+  // mbarrier and its parity, the Philox counter of the quad, the output
+  // pointer.  (Formed anew in every step they cost the heatbath 12 of 204
+  // instructions per quad: 139.1 -> 135.4 us per half-sweep of 128^3 x 64
+  // chains.  It is bound by the two arithmetic pipes and by latency, 17 warps
+  // per SM: 59% of the issue slots are used.)
+  const uint32_t hrow = (uint32_t)(((ty + 1) * W + 4 * qx) * (int)sizeof(T));  // in a halo box
+  const uint32_t ring0 = kHeaderBytes + hrow;
+  const uint32_t ring_end = ring0 + (uint32_t)(STAGES * lay.slot_bytes);
+  const uint32_t wb = (uint32_t)(W * (int)sizeof(T));  // a row
+  // this thread's quad in the own box of a slot, from that in its halo box
+  const uint32_t own_delta = (uint32_t)round_up_int(lay.halo_bytes, 128) - wb;
+  const uint32_t bar0 = smem_addr(bars);
+  uint32_t at_k = ring0 + (uint32_t)(slot_of(0) * lay.slot_bytes);
+  uint32_t at_n = ring0 + (uint32_t)(slot_of(1) * lay.slot_bytes);
+  auto quad_at = [&](uint32_t off) { return reinterpret_cast<const T *>(smem + off); };
+
   T cm[V][4], c0[V][4], cp[V][4];
 #pragma unroll
   for (int v = 0; v < V; ++v)
@@ -293,12 +305,12 @@ __device__ bool march_tile(const Job &j, const PhiloxKeys &K, unsigned char *sme
   if (ok)
 #pragma unroll
     for (int v = 0; v < V; ++v)
-      if (qmem[v]) ld_quad(halo_slot(slot_of(0)) + (ty + 1) * W + 4 * (qx + v), cm[v]);
+      if (qmem[v]) ld_quad(quad_at(at_k) + 4 * v, cm[v]);
   ok = ok && wait_plane(1);
   if (ok)
 #pragma unroll
     for (int v = 0; v < V; ++v)
-      if (qmem[v]) ld_quad(halo_slot(slot_of(1)) + (ty + 1) * W + 4 * (qx + v), c0[v]);
+      if (qmem[v]) ld_quad(quad_at(at_n) + 4 * v, c0[v]);
   if (ok) t0_waited = 1;
   if (!ok) {
     atomicOr(err, kErrTimeout);
@@ -307,9 +319,9 @@ __device__ bool march_tile(const Job &j, const PhiloxKeys &K, unsigned char *sme
   __syncthreads();
   bool aborted = *abort_flag != 0;
 
-  // per-thread constants of the plane loop
   // quad lanes past x = Lx - 1 (kept at 0), row parity 0 / 1, per quad
   uint32_t pad0[V], pad1[V];
+  bool padded = false;
 #pragma unroll
   for (int v = 0; v < V; ++v) {
     pad0[v] = pad1[v] = 0u;
@@ -318,47 +330,57 @@ __device__ bool march_tile(const Job &j, const PhiloxKeys &K, unsigned char *sme
       if (2 * (4 * (qx + v) + i) >= j.Lx()) pad0[v] |= 1u << i;
       if (2 * (4 * (qx + v) + i) + 1 >= j.Lx()) pad1[v] |= 1u << i;
     }
+    padded = padded || pad0[v] != 0u || pad1[v] != 0u;
   }
   const bool lo_ok = qx > 0, hi_ok = 4 * qx + 4 * V < W;
-  const int hrow = (ty + 1) * W + 4 * qx;  // this quad in a halo box (first row y0 - 1)
-  const int orow = ty * W + 4 * qx;        // this quad in an own box (first row y0)
   T *outp = j.out() + ((size_t)j.z0() * j.Ly() + y) * W + 4 * qx;  // plane z0; one plane per step
   const size_t pstride = (size_t)j.Ly() * W;
-  int par = (c + y + j.z0()) & 1;  // the row (y, z) holds x = 2h + par; flips with z
+  bool odd = ((c + y + j.z0()) & 1) != 0;  // the row (y, z) holds x = 2h + odd; flips with z
+  uint32_t quad = ((uint32_t)j.z0() * (uint32_t)j.Ly() + (uint32_t)y) * (uint32_t)j.Wq() + (uint32_t)qx;
+  const uint32_t quad_step = (uint32_t)j.Ly() * (uint32_t)j.Wq();
+  const uint32_t rng_id = j.rng_id(), pass = j.pass();
+  // plane 1 becomes plane k of the first step, plane 2 the one it waits for
+  uint32_t bar_n = bar0 + 8u * (uint32_t)slot_of(2), par_n = (uint32_t)(((gb + 2) / STAGES) & 1);
+  auto advance = [&]() {
+    at_k = at_n;
+    at_n += (uint32_t)lay.slot_bytes;
+    if (at_n == ring_end) at_n = ring0;
+  };
+  advance();
 
   // Plane k (z = z0 + k - 1): M, C, P are the other colour's quads of planes
   // z - 1, z, z + 1 (P loaded here).  The loop calls it with the names
   // rotated, so no register is copied from plane to plane.
   //
-  // Between barriers a thread that finds the abort flag set only skips its
-  // work: whether the CTA stops is decided right after a barrier, where
-  // every thread reads the same flag (a thread leaving early would miss the
-  // barriers the others still reach).
+  // Between barriers a thread whose wait gave up only skips its work: whether
+  // the CTA stops is decided right after a barrier, where every thread reads
+  // the same flag (a thread leaving early would miss the barriers the others
+  // still reach).
   auto step = [&](int k, T(&M)[V][4], T(&C)[V][4], T(&P)[V][4]) -> bool {
-    const bool got = *abort_flag == 0 && wait_plane(k + 1);
-    if (got) t0_waited = k + 1;
-    const T *Pz = halo_slot(slot_of(k)) + hrow;  // row y of plane z
-    if (got) {
+    ok = ok && mbar_wait_bounded(bar_n, par_n);
+    if (ok) {
+      t0_waited = k + 1;
+      const T *Pz = quad_at(at_k);  // row y of plane z
 #pragma unroll
       for (int v = 0; v < V; ++v) {
         if (qmem[v]) {
-          ld_quad(halo_slot(slot_of(k + 1)) + hrow + 4 * v, P[v]);
+          ld_quad(quad_at(at_n) + 4 * v, P[v]);
         } else {
 #pragma unroll
           for (int i = 0; i < 4; ++i) P[v][i] = T(0);
         }
       }
       if (live) {
-        const bool odd = par != 0;
         // the x neighbour beyond this thread's quads (left end when even,
         // right end when odd); between its own quads it is in registers
         const T edge = (odd ? hi_ok : lo_ok) ? Pz[odd ? 4 * V : -1] : T(0);
+        const T *Pm = quad_at(at_k - wb), *Pp = quad_at(at_k + wb);
 #pragma unroll
         for (int v = 0; v < V; ++v) {
           if (!qlive[v]) continue;
           T ym[4], yp[4], xs[4], u[4];
-          ld_quad(Pz + 4 * v - W, ym);
-          ld_quad(Pz + 4 * v + W, yp);
+          ld_quad(Pm + 4 * v, ym);
+          ld_quad(Pp + 4 * v, yp);
           const T e = odd ? (v + 1 < V ? C[v + 1 < V ? v + 1 : v][0] : edge)
                           : (v > 0 ? C[v > 0 ? v - 1 : v][3] : edge);
           x_neighbours(odd, e, C[v], xs);
@@ -372,17 +394,14 @@ __device__ bool march_tile(const Job &j, const PhiloxKeys &K, unsigned char *sme
                               padd(pair_of(ym, h), pair_of(yp, h))),
                          padd(pair_of(C[v], h), pair_of(xs, h)));
           if (!OR) {
-            const uint32_t z = (uint32_t)(j.z0() + k - 1);
-            const uint32_t quad =
-                (z * (uint32_t)j.Ly() + (uint32_t)y) * (uint32_t)j.Wq() + (uint32_t)(qx + v);
-            const uint4 w = philox4x32_10(make_uint4(quad, j.pass(), j.rng_id(), (uint32_t)c), K);
+            const uint4 w = philox4x32_10(make_uint4(quad + (uint32_t)v, pass, rng_id, (uint32_t)c), K);
             P2 n2[2];
             QuadNoise2<T>::of(w, n2);
             u2[0] = pfma(S2[0], pset(Coef<T>::sixth), n2[0]);
             u2[1] = pfma(S2[1], pset(Coef<T>::sixth), n2[1]);
           } else {
             T old[4];
-            ld_quad(own_slot(slot_of(k)) + orow + 4 * v, old);
+            ld_quad(quad_at(at_k + own_delta) + 4 * v, old);
 #pragma unroll
             for (int h = 0; h < 2; ++h)
               u2[h] = pfma(S2[h], pset(Coef<T>::third), pneg(pair_of(old, h)));
@@ -391,8 +410,8 @@ __device__ bool march_tile(const Job &j, const PhiloxKeys &K, unsigned char *sme
           u[1] = u2[0].y;
           u[2] = u2[1].x;
           u[3] = u2[1].y;
-          const uint32_t pm = par ? pad1[v] : pad0[v];
-          if (pm) {
+          if (padded) {
+            const uint32_t pm = odd ? pad1[v] : pad0[v];
 #pragma unroll
             for (int i = 0; i < 4; ++i)
               if ((pm >> i) & 1u) u[i] = T(0);  // keep the row padding at 0
@@ -405,7 +424,14 @@ __device__ bool march_tile(const Job &j, const PhiloxKeys &K, unsigned char *sme
       *abort_flag = 1;
     }
     outp += pstride;
-    par ^= 1;
+    odd = !odd;
+    quad += quad_step;
+    advance();
+    bar_n += 8u;
+    if (bar_n == bar0 + 8u * STAGES) {
+      bar_n = bar0;
+      par_n ^= 1u;
+    }
     if (k % GROUP == 0 || k == j.nz()) {
       __syncthreads();
       if (*abort_flag) return false;
