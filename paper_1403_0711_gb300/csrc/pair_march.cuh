@@ -6,8 +6,11 @@
 // (`gbase`).
 #pragma once
 
+#include <type_traits>
+
 #include "device_common.cuh"
 #include "internal.h"
+#include "march_quad.cuh"
 #include "tile_march.cuh"
 
 namespace coulps {
@@ -21,11 +24,19 @@ constexpr int kPairStages = 8;
 constexpr int kPairAbort = 96;
 static_assert(kPairStages <= 12, "mbarriers must end before the abort flag");
 
+// The stages' buffers (3 stages x 2 planes of (TY + 6) x W) lie quad by quad:
+// the six values of one quad side by side and 16 bytes of padding, so that a
+// stage's buffer is an immediate offset of the quad's one address and eight
+// lanes' 16-byte accesses (pitch 28 words, FP64 52 words) fall on different
+// banks.  Over-relaxation pair of 128^3 x 64 chains / 16^3 x 512 chains:
+// 262 / 18.0 us; planes at a distance known only at run time 264 / 18.1; at a
+// fixed 8192 bytes 258 / 28.4 (the small tile then loses CTAs per SM).
+constexpr int pair_quad_pitch(int es) { return 6 * 4 * es + 16; }
+
 struct PairLayout {
   int c1_bytes;   // colour-1 box: (TY + 8) rows x W
   int c0_bytes;   // colour-0 box: (TY + 6) rows x W (pass A over-relaxation only)
   int slot_bytes;
-  int buf_bytes;  // one plane of one stage's rows: (TY + 6) x W
   int total;      // header + ring slots + 3 stages x 2 planes
 };
 
@@ -34,121 +45,8 @@ __host__ __device__ inline PairLayout pair_layout(int TY, int W, int es, bool a_
   L.c1_bytes = (TY + 8) * W * es;
   L.c0_bytes = a_or ? (TY + 6) * W * es : 0;
   L.slot_bytes = round_up_int(L.c1_bytes, 128) + round_up_int(L.c0_bytes, 128);
-  L.buf_bytes = round_up_int((TY + 6) * W * es, 128);
-  L.total = kHeaderBytes + kPairStages * L.slot_bytes + 6 * L.buf_bytes;
+  L.total = kHeaderBytes + kPairStages * L.slot_bytes + (TY + 6) * (W / 4) * pair_quad_pitch(es);
   return L;
-}
-
-template <typename T>
-__device__ __forceinline__ Quad<T> qzero() {
-  Quad<T> q;
-  q.a = pset(T(0));
-  q.b = pset(T(0));
-  return q;
-}
-
-template <typename T>
-__device__ __forceinline__ Quad<T> qload(const T *p);
-template <>
-__device__ __forceinline__ Quad<float> qload<float>(const float *p) {
-  const float4 f = *reinterpret_cast<const float4 *>(p);
-  Quad<float> q;
-  q.a = make_float2(f.x, f.y);
-  q.b = make_float2(f.z, f.w);
-  return q;
-}
-template <>
-__device__ __forceinline__ Quad<double> qload<double>(const double *p) {
-  Quad<double> q;
-  q.a = reinterpret_cast<const double2 *>(p)[0];
-  q.b = reinterpret_cast<const double2 *>(p)[1];
-  return q;
-}
-
-template <typename T>
-__device__ __forceinline__ void qstore(T *p, const Quad<T> &q);
-template <>
-__device__ __forceinline__ void qstore<float>(float *p, const Quad<float> &q) {
-  *reinterpret_cast<float4 *>(p) = make_float4(q.a.x, q.a.y, q.b.x, q.b.y);
-}
-template <>
-__device__ __forceinline__ void qstore<double>(double *p, const Quad<double> &q) {
-  reinterpret_cast<double2 *>(p)[0] = q.a;
-  reinterpret_cast<double2 *>(p)[1] = q.b;
-}
-
-// The heatbath deviates of two quads (two stages' Philox words): FP32 as
-// four packed pairs under one warp vote (every lane of the warp must call
-// it); FP64 word by word.
-template <typename T> struct StageNoise;
-template <> struct StageNoise<float> {
-  __device__ __forceinline__ static void of(uint4 wa, uint4 wb, Quad<float> &na,
-                                            Quad<float> &nb) {
-    const uint32_t w[8] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w};
-    float2 o[4];
-    hb_noise_pairs_f32<4>(w, o);
-    na.a = o[0];
-    na.b = o[1];
-    nb.a = o[2];
-    nb.b = o[3];
-  }
-};
-template <> struct StageNoise<double> {
-  __device__ __forceinline__ static void of(uint4 wa, uint4 wb, Quad<double> &na,
-                                            Quad<double> &nb) {
-    na.a = make_double2(hb_noise_f64(wa.x), hb_noise_f64(wa.y));
-    na.b = make_double2(hb_noise_f64(wa.z), hb_noise_f64(wa.w));
-    nb.a = make_double2(hb_noise_f64(wb.x), hb_noise_f64(wb.y));
-    nb.b = make_double2(hb_noise_f64(wb.z), hb_noise_f64(wb.w));
-  }
-};
-
-// The new values of a quad.  zm, zp: the other colour's quad on planes
-// z -+ 1; ym, yp: rows y -+ 1; c: same row and plane; e: the x neighbour
-// outside c (the previous quad's last site for an even row, the next quad's
-// first for an odd row; 0 beyond the box); r: the site's value before the
-// pass (over-relaxation) or the heatbath deviates.  Sums in the order of the
-// half-sweep kernel: S = ((zm + zp) + (ym + yp)) + (c + xs), then
-// S/3 - old or S/6 + deviate by one fma.
-template <typename T, bool OR>
-__device__ __forceinline__ Quad<T> update(const Quad<T> &zm, const Quad<T> &zp, const Quad<T> &ym,
-                                          const Quad<T> &yp, const Quad<T> &c, bool odd, T e,
-                                          const Quad<T> &r) {
-  using P2 = typename Pair2<T>::type;
-  P2 xa, xb;
-  xa.x = odd ? c.a.y : e;
-  xa.y = odd ? c.b.x : c.a.x;
-  xb.x = odd ? c.b.y : c.a.y;
-  xb.y = odd ? e : c.b.x;
-  Quad<T> S, v;
-  S.a = padd(padd(padd(zm.a, zp.a), padd(ym.a, yp.a)), padd(c.a, xa));
-  S.b = padd(padd(padd(zm.b, zp.b), padd(ym.b, yp.b)), padd(c.b, xb));
-  if (OR) {
-    const P2 third = pset(Coef<T>::third);
-    v.a = pfma(S.a, third, pneg(r.a));
-    v.b = pfma(S.b, third, pneg(r.b));
-  } else {
-    const P2 sixth = pset(Coef<T>::sixth);
-    v.a = pfma(S.a, sixth, r.a);
-    v.b = pfma(S.b, sixth, r.b);
-  }
-  return v;
-}
-
-// Zero what is not a site of the box: the whole quad when `valid` is false
-// (a ghost row or plane), else the lanes past x = Lx - 1 (bit i of pm: site i
-// of the quad).  `fast` (warp-uniform): nothing to zero.
-template <typename T>
-__device__ __forceinline__ Quad<T> mask(Quad<T> v, bool fast, bool valid, uint32_t pm) {
-  if (fast) return v;
-  if (!valid) return qzero<T>();
-  if (pm) {
-    if (pm & 1u) v.a.x = T(0);
-    if (pm & 2u) v.a.y = T(0);
-    if (pm & 4u) v.b.x = T(0);
-    if (pm & 8u) v.b.y = T(0);
-  }
-  return v;
 }
 
 // The tile: TY rows from y0 and planes [z0, z0 + nz) of one chain (or
@@ -209,19 +107,13 @@ __device__ bool march_pair(const Job &a, const PhiloxKeys &K, unsigned char *sme
   const PairLayout lay = pair_layout(a.TY(), a.W(), (int)sizeof(T), A_OR);
   uint64_t *bars = reinterpret_cast<uint64_t *>(smem);
   volatile int *abort_flag = reinterpret_cast<volatile int *>(smem + kPairAbort);
-  unsigned char *ring = smem + kHeaderBytes;
-  unsigned char *bufs = ring + kPairStages * lay.slot_bytes;
   const int gb = gbase;
-  auto c1_slot = [&](int j) {
-    return reinterpret_cast<const T *>(ring + ((gb + j) % kPairStages) * lay.slot_bytes);
+  // ring slot of plane j, as a byte offset
+  auto slot_at = [&](int j) {
+    return (uint32_t)(kHeaderBytes + ((gb + j) % kPairStages) * lay.slot_bytes);
   };
-  auto c0_slot = [&](int j) {
-    return reinterpret_cast<const T *>(ring + ((gb + j) % kPairStages) * lay.slot_bytes +
-                                       round_up_int(lay.c1_bytes, 128));
-  };
-  auto buf = [&](int k, int par) {
-    return reinterpret_cast<T *>(bufs + (2 * k + (par & 1)) * lay.buf_bytes);
-  };
+  auto at = [&](uint32_t off) { return reinterpret_cast<T *>(smem + off); };
+  const uint32_t c0_off = (uint32_t)round_up_int(lay.c1_bytes, 128);  // colour-0 box in a slot
 
   const int W = a.W(), TY = a.TY(), QW = a.QW(), Ly = a.Ly(), Lz = a.Lz();
   const int y0 = a.y0(), z0 = a.z0(), nz = a.nz();
@@ -242,10 +134,16 @@ __device__ bool march_pair(const Job &a, const PhiloxKeys &K, unsigned char *sme
 #pragma unroll
   for (int k = 0; k < 4; ++k) warp_in[k] = wr_hi >= k && wr_lo <= rows - 1 - k;
 
-  // offsets: row r in a buffer / colour-0 box, row r + 1 in the colour-1 box
-  const int o_r = r * W + 4 * qx;
-  const int o_m = max(r - 1, 0) * W + 4 * qx;         // clamped for rows no stage reads
-  const int o_p = min(r + 1, rows - 1) * W + 4 * qx;
+  // byte offsets: row r in a colour-0 box = row r + 1 in the colour-1 box less
+  // one row, and this quad's buffers (and its row neighbours', clamped for
+  // rows no stage reads)
+  constexpr uint32_t kQ = (uint32_t)(4 * sizeof(T)), kPitch = pair_quad_pitch((int)sizeof(T));
+  const uint32_t wb = (uint32_t)W * (uint32_t)sizeof(T);
+  const uint32_t o_r = (uint32_t)r * wb + (uint32_t)qx * kQ;
+  const uint32_t bw = (uint32_t)QW * kPitch;
+  const uint32_t b_r = (uint32_t)(kHeaderBytes + kPairStages * lay.slot_bytes) +
+                       (uint32_t)r * bw + (uint32_t)qx * kPitch;
+  const uint32_t b_m = r > 0 ? b_r - bw : b_r, b_p = r + 1 < rows ? b_r + bw : b_r;
   const bool lo_ok = qx > 0, hi_ok = 4 * qx + 4 < W;
   uint32_t pad0 = 0u, pad1 = 0u;
 #pragma unroll
@@ -276,8 +174,9 @@ __device__ bool march_pair(const Job &a, const PhiloxKeys &K, unsigned char *sme
     const uint32_t bar = smem_addr(&bars[(gb + j) % kPairStages]);
     const bool own = A_OR && j >= 2;
     mbar_arrive_expect_tx(bar, lay.c1_bytes + (own ? lay.c0_bytes : 0));
-    tma_load_4d(smem_addr(c1_slot(j)), a.tm_c1(), 0, y0 - 4, z0 - 4 + j, a.map_c1(), bar);
-    if (own) tma_load_4d(smem_addr(c0_slot(j)), a.tm_c0(), 0, y0 - 3, z0 - 5 + j, a.map_c0(), bar);
+    const uint32_t slot = smem_addr(at(slot_at(j)));
+    tma_load_4d(slot, a.tm_c1(), 0, y0 - 4, z0 - 4 + j, a.map_c1(), bar);
+    if (own) tma_load_4d(slot + c0_off, a.tm_c0(), 0, y0 - 3, z0 - 5 + j, a.map_c0(), bar);
   };
   auto wait_plane = [&](int j) -> bool {
     return mbar_wait_bounded(smem_addr(&bars[(gb + j) % kPairStages]),
@@ -317,9 +216,23 @@ __device__ bool march_pair(const Job &a, const PhiloxKeys &K, unsigned char *sme
   Quad<T> R0 = qzero<T>(), R1 = qzero<T>(), R2 = qzero<T>();
   Quad<T> U0 = qzero<T>(), U1 = qzero<T>(), U2 = qzero<T>();
   if (!aborted) {
-    P0 = qload(c1_slot(0) + o_r + W);
-    P1 = qload(c1_slot(1) + o_r + W);
+    P0 = qload<T>(at(slot_at(0) + o_r + wb));
+    P1 = qload<T>(at(slot_at(1) + o_r + wb));
   }
+
+  // What advances from step to step: this thread's row in the ring slots of
+  // planes s + 1 and s + 2, the mbarrier of plane s + 2 and its parity, the
+  // buffers' parity, the row parity, the output pointer of stage 2's plane.
+  const uint32_t ring_o = (uint32_t)kHeaderBytes + o_r;
+  const uint32_t ring_end = ring_o + (uint32_t)(kPairStages * lay.slot_bytes);
+  uint32_t n1 = slot_at(1) + o_r, n2 = slot_at(2) + o_r;
+  const uint32_t bar0 = smem_addr(bars);
+  uint32_t bar_n = bar0 + 8u * (uint32_t)((gb + 2) % kPairStages);
+  uint32_t par_n = (uint32_t)(((gb + 2) / kPairStages) & 1);
+  uint32_t tog = 0u;  // kQ in odd steps: what the step writes
+  bool odd = ((y + z0 - 3) & 1) != 0;  // the same row parity for all four stages
+  T *out = dst0 + (ptrdiff_t)(z0 - 5) * (ptrdiff_t)plane_elems + row_off;  // plane f - 2
+  const ptrdiff_t out3 = (ptrdiff_t)a.colour_elems() - (ptrdiff_t)plane_elems;
 
   // Step s with the windows' names rotated by the caller.  At entry:
   // P0, P1 = old colour 1 at f - 1, f (P2 loaded here: f + 1); Q0, Q1 =
@@ -335,20 +248,22 @@ __device__ bool march_pair(const Job &a, const PhiloxKeys &K, unsigned char *sme
   // others finish.  After the barrier (all warps are through the previous
   // step: its buffer writes are visible and the buffers it read are free)
   // stages 1 .. 3 read the previous step's buffers and write this step's.
-  auto step = [&](int s, Quad<T> &P0, Quad<T> &P1, Quad<T> &P2, Quad<T> &Q0, Quad<T> &Q1,
-                  Quad<T> &Q2, Quad<T> &R0, Quad<T> &R1, Quad<T> &R2, Quad<T> &U0, Quad<T> &U1,
-                  Quad<T> &U2) -> bool {
+  //
+  // STEADY: s >= 6, all four stages run and stage 3's plane is the tile's.
+  auto step = [&](auto steady, int s, Quad<T> &P0, Quad<T> &P1, Quad<T> &P2, Quad<T> &Q0,
+                  Quad<T> &Q1, Quad<T> &Q2, Quad<T> &R0, Quad<T> &R1, Quad<T> &R2, Quad<T> &U0,
+                  Quad<T> &U1, Quad<T> &U2) -> bool {
+    constexpr bool STEADY = decltype(steady)::value;
     const int f = z0 - 3 + s;
-    const bool odd = ((y + f) & 1) != 0;  // the same row parity for all four stages
-    const uint32_t pm = odd ? pad1 : pad0;
-    const int eo = odd ? 4 : -1;
     const bool e_ok = odd ? hi_ok : lo_ok;
-    bool plane_ok[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) plane_ok[k] = f - k >= 0 && f - k < Lz;
-    // the whole warp agrees on the outcome, so it never splits around the
-    // heatbath deviates' warp vote
-    const bool got = __all_sync(0xffffffffu, wait_plane(s + 2));
+    const uint32_t eo = odd ? kQ : 0u - (uint32_t)sizeof(T);
+    const uint32_t beo = odd ? kPitch : 3u * (uint32_t)sizeof(T) - kPitch;
+    // nothing to zero in any stage: the warp is inside the box and without
+    // padding lanes, and so are planes f - 3 .. f
+    const bool fast = warp_full && f >= 3 && f < Lz;
+    bool got = mbar_wait_bounded(bar_n, par_n);
+    // the heatbath deviates take the whole warp through the same path
+    if (!A_OR || !B_OR) got = __all_sync(0xffffffffu, got);
     if (!got) {
       atomicOr(err, kErrTimeout);
       *abort_flag = 1;
@@ -362,7 +277,7 @@ __device__ bool march_pair(const Job &a, const PhiloxKeys &K, unsigned char *sme
             make_uint4((uint32_t)(f - 1) * qplane + qrow, pass_a, rng, 1u), K);
         StageNoise<T>::of(w0, w1, nA0, nA1);
       }
-      if (!B_OR && s >= 4) {
+      if (!B_OR && (STEADY || s >= 4)) {
         const uint4 w2 = philox4x32_10(
             make_uint4((uint32_t)(f - 2) * qplane + qrow, pass_b, rng, 0u), K);
         const uint4 w3 = philox4x32_10(
@@ -370,61 +285,80 @@ __device__ bool march_pair(const Job &a, const PhiloxKeys &K, unsigned char *sme
         StageNoise<T>::of(w2, w3, nB0, nB1);
       }
       // ---- stage 0: colour 0 of pass A at plane f (ring only)
-      const T *C = c1_slot(s + 1);  // old colour 1, plane f (box row r + 1)
-      P2 = qload(c1_slot(s + 2) + o_r + W);
-      const Quad<T> ym = qload(C + o_r), yp = qload(C + o_r + 2 * W);
-      const T e = e_ok ? C[o_r + W + eo] : T(0);
+      P2 = qload<T>(at(n2 + wb));
+      const Quad<T> ym = qload<T>(at(n1)), yp = qload<T>(at(n1 + 2u * wb));
+      const T e = e_ok ? *at(n1 + wb + eo) : T(0);
       Quad<T> r0 = nA0;
-      if (A_OR) r0 = qload(c0_slot(s + 2) + o_r);
-      const Quad<T> v = update<T, A_OR>(P0, P2, ym, yp, P1, odd, e, r0);
-      Q2 = mask(v, warp_full && plane_ok[0], live && plane_ok[0], pm);
+      if (A_OR) r0 = qload<T>(at(n2 + c0_off));
+      Q2 = update<T, A_OR>(P0, P2, ym, yp, P1, odd, e, r0);
+      if (!fast) mask(Q2, live && f >= 0 && f < Lz, odd ? pad1 : pad0);
     }
     __syncthreads();
     if (*abort_flag) return false;
     done = s + 2;
     // ring plane s was last read in the previous step: refill its slot
     if (tid == 0 && issued < n_ring) issue(issued++);
-    if (lane_ok) qstore(buf(0, s) + o_r, Q2);
+    // stage k's plane goes to buffer k of this step's parity; stage k + 1 reads
+    // buffer k of the other one
+    const uint32_t w_r = b_r + tog, d = kQ - tog;
+    const uint32_t r_m = b_m + d, r_p = b_p + d, r_e = b_r + d + beo;
+    if (lane_ok) qstore(at(w_r), Q2);
     // ---- stage 1: colour 1 of pass A at plane f - 1 (old value: P0)
-    if (s >= 2 && warp_in[1]) {
-      const T *B = buf(0, s - 1);  // colour 0 after A, plane f - 1
-      const Quad<T> ym = qload(B + o_m), yp = qload(B + o_p);
-      const T e = e_ok ? B[o_r + eo] : T(0);
-      const Quad<T> v = update<T, A_OR>(Q0, Q2, ym, yp, Q1, odd, e, A_OR ? P0 : nA1);
-      R2 = mask(v, warp_full && plane_ok[1], live && plane_ok[1], pm);
-      if (lane_ok) qstore(buf(1, s) + o_r, R2);
+    if ((STEADY || s >= 2) && warp_in[1]) {
+      const Quad<T> ym = qload<T>(at(r_m)), yp = qload<T>(at(r_p));
+      const T e = e_ok ? *at(r_e) : T(0);
+      R2 = update<T, A_OR>(Q0, Q2, ym, yp, Q1, odd, e, A_OR ? P0 : nA1);
+      if (!fast) mask(R2, live && f >= 1 && f - 1 < Lz, odd ? pad1 : pad0);
+      if (lane_ok) qstore(at(w_r + 2u * kQ), R2);
     }
     // ---- stage 2: colour 0 of pass B at plane f - 2 (old value: Q0)
-    if (s >= 4 && warp_in[2]) {
-      const T *B = buf(1, s - 1);  // colour 1 after A, plane f - 2
-      const Quad<T> ym = qload(B + o_m), yp = qload(B + o_p);
-      const T e = e_ok ? B[o_r + eo] : T(0);
-      const Quad<T> v = update<T, B_OR>(R0, R2, ym, yp, R1, odd, e, B_OR ? Q0 : nB0);
-      const int p = f - 2;
-      U2 = mask(v, warp_full && plane_ok[2], live && plane_ok[2], pm);
-      if (lane_ok) qstore(buf(2, s) + o_r, U2);
-      if (own_row && p >= z0 && p < z0 + nz) qstore(dst0 + (size_t)p * plane_elems + row_off, U2);
+    if ((STEADY || s >= 4) && warp_in[2]) {
+      const Quad<T> ym = qload<T>(at(r_m + 2u * kQ)), yp = qload<T>(at(r_p + 2u * kQ));
+      const T e = e_ok ? *at(r_e + 2u * kQ) : T(0);
+      U2 = update<T, B_OR>(R0, R2, ym, yp, R1, odd, e, B_OR ? Q0 : nB0);
+      if (!fast) mask(U2, live && f >= 2 && f - 2 < Lz, odd ? pad1 : pad0);
+      if (lane_ok) qstore(at(w_r + 4u * kQ), U2);
+      // the tile's planes: s = 5 .. nz + 4
+      if (own_row && (STEADY || s >= 5) && s < nz + 5) qstore(out, U2);
     }
     // ---- stage 3: colour 1 of pass B at plane f - 3 (old value: R0)
-    if (s >= 6 && warp_in[3]) {
-      const T *B = buf(2, s - 1);  // colour 0 after B, plane f - 3
-      const Quad<T> ym = qload(B + o_m), yp = qload(B + o_p);
-      const T e = e_ok ? B[o_r + eo] : T(0);
-      const Quad<T> v = update<T, B_OR>(U0, U2, ym, yp, U1, odd, e, B_OR ? R0 : nB1);
-      const int p = f - 3;
-      if (own_row && p >= z0 && p < z0 + nz)
-        qstore(dst1 + (size_t)p * plane_elems + row_off, mask(v, warp_full, true, pm));
+    if ((STEADY || s >= 6) && warp_in[3]) {
+      const Quad<T> ym = qload<T>(at(r_m + 4u * kQ)), yp = qload<T>(at(r_p + 4u * kQ));
+      const T e = e_ok ? *at(r_e + 4u * kQ) : T(0);
+      Quad<T> v = update<T, B_OR>(U0, U2, ym, yp, U1, odd, e, B_OR ? R0 : nB1);
+      if (!fast) mask(v, true, odd ? pad1 : pad0);
+      if (own_row) qstore(out + out3, v);
     }
+    n1 = n2;
+    n2 += (uint32_t)lay.slot_bytes;
+    if (n2 == ring_end) n2 = ring_o;
+    bar_n += 8u;
+    if (bar_n == bar0 + 8u * kPairStages) {
+      bar_n = bar0;
+      par_n ^= 1u;
+    }
+    tog ^= kQ;
+    odd = !odd;
+    out += plane_elems;
     return true;
   };
 
   const int n_steps = nz + 6;
-  for (int s = 0; s < n_steps && !aborted; s += 3) {
-    if (!step(s, P0, P1, P2, Q0, Q1, Q2, R0, R1, R2, U0, U1, U2)) { aborted = true; break; }
+  using First = std::integral_constant<bool, false>;
+  using Steady = std::integral_constant<bool, true>;
+  int s = 0;
+#pragma unroll 1
+  for (; s < 6 && !aborted; s += 3)
+    aborted = !(step(First(), s, P0, P1, P2, Q0, Q1, Q2, R0, R1, R2, U0, U1, U2) &&
+                step(First(), s + 1, P1, P2, P0, Q1, Q2, Q0, R1, R2, R0, U1, U2, U0) &&
+                step(First(), s + 2, P2, P0, P1, Q2, Q0, Q1, R2, R0, R1, U2, U0, U1));
+#pragma unroll 1
+  for (; s < n_steps && !aborted; s += 3) {
+    if (!step(Steady(), s, P0, P1, P2, Q0, Q1, Q2, R0, R1, R2, U0, U1, U2)) { aborted = true; break; }
     if (s + 1 >= n_steps) break;
-    if (!step(s + 1, P1, P2, P0, Q1, Q2, Q0, R1, R2, R0, U1, U2, U0)) { aborted = true; break; }
+    if (!step(Steady(), s + 1, P1, P2, P0, Q1, Q2, Q0, R1, R2, R0, U1, U2, U0)) { aborted = true; break; }
     if (s + 2 >= n_steps) break;
-    if (!step(s + 2, P2, P0, P1, Q2, Q0, Q1, R2, R0, R1, U2, U0, U1)) { aborted = true; break; }
+    if (!step(Steady(), s + 2, P2, P0, P1, Q2, Q0, Q1, R2, R0, R1, U2, U0, U1)) { aborted = true; break; }
   }
   if (aborted && tid == 0) {
     // leave no copy in flight into this CTA's shared memory

@@ -101,6 +101,9 @@ __device__ __forceinline__ double2 pfma(double2 p, double2 q, double2 r) {
 }
 __device__ __forceinline__ float2 pneg(float2 p) { return make_float2(-p.x, -p.y); }
 __device__ __forceinline__ double2 pneg(double2 p) { return make_double2(-p.x, -p.y); }
+// the same as one packed product by -1 (four sign changes otherwise)
+__device__ __forceinline__ float2 pneg2(float2 p) { return __fmul2_rn(p, make_float2(-1.f, -1.f)); }
+__device__ __forceinline__ double2 pneg2(double2 p) { return pneg(p); }
 __device__ __forceinline__ float2 pset(float c) { return make_float2(c, c); }
 __device__ __forceinline__ double2 pset(double c) { return make_double2(c, c); }
 
