@@ -5,8 +5,11 @@
 // ring's mbarrier phases run on from tile to tile (`gbase`).
 #pragma once
 
+#include <type_traits>
+
 #include "device_common.cuh"
 #include "internal.h"
+#include "march_quad.cuh"
 #include "tile_march.cuh"
 
 namespace coulps {
@@ -52,6 +55,9 @@ __host__ __device__ inline PassLayout pass_layout(int TY, int W, int es, bool or
 // keeps the origin out of registers).
 template <typename T>
 struct PassTile {
+  // the CTA may have whole warps past the tile's rows (one block size for
+  // tiles of every system): they skip the stages
+  static constexpr bool kIdleWarps = true;
   const CUtensorMap *tm_c1_, *tm_c0_;
   int map_c1_, map_c0_;
   T *dst_;
@@ -93,39 +99,31 @@ __device__ __forceinline__ void pass_ring_init(unsigned char *smem) {
 template <typename T, bool OR, bool GATHER, typename Job>
 __device__ bool march_pass(const Job &a, const PhiloxKeys &K, unsigned char *smem, int *err,
                            int &gbase, double &sq, double &sp) {
-  constexpr int R = 1;  // rows per thread
   const PassLayout lay = pass_layout(a.TY(), a.W(), (int)sizeof(T), OR);
   uint64_t *bars = reinterpret_cast<uint64_t *>(smem);
   volatile int *abort_flag = reinterpret_cast<volatile int *>(smem + 64);
-  unsigned char *ring = smem + kHeaderBytes;
-  T *newbuf = reinterpret_cast<T *>(ring + kPassStages * lay.slot_bytes);
   const int gb = gbase;
-  auto c1_slot = [&](int j) {
-    return reinterpret_cast<T *>(ring + ((gb + j) % kPassStages) * lay.slot_bytes);
+  // ring slot of plane j, as a byte offset; the colour-0 box lies c0_off in
+  auto slot_at = [&](int j) {
+    return (uint32_t)(kHeaderBytes + ((gb + j) % kPassStages) * lay.slot_bytes);
   };
-  auto c0_slot = [&](int j) {
-    return reinterpret_cast<T *>(ring + ((gb + j) % kPassStages) * lay.slot_bytes +
-                                 round_up_int(lay.c1_bytes, 128));
-  };
-  auto new_plane = [&](int s) {
-    return reinterpret_cast<T *>(reinterpret_cast<unsigned char *>(newbuf) + (s & 1) * lay.new_bytes);
-  };
+  auto at = [&](uint32_t off) { return reinterpret_cast<T *>(smem + off); };
+  const uint32_t c0_off = (uint32_t)round_up_int(lay.c1_bytes, 128);
 
-  const int W = a.W(), TY = a.TY();
+  const int W = a.W(), TY = a.TY(), QW = a.QW(), Lz = a.Lz();
   const int y0 = a.y0(), z0 = a.z0(), nz = a.nz();
   const int tid = threadIdx.x;
-  // this thread: quad qx of row r0 (y = y0 - 1 + r0; rows 0 and TY + 1 are
-  // the halo of stage 0)
-  const int qx = tid % a.QW(), r0 = R * (tid / a.QW());
-  const bool in_tile = r0 < TY + 2;
-  bool live0[R], live1[R];
-  int yk[R];
-#pragma unroll
-  for (int k = 0; k < R; ++k) {
-    yk[k] = y0 - 1 + r0 + k;
-    live0[k] = in_tile && yk[k] >= 0 && yk[k] < a.Ly() && qx < a.Wq();
-    live1[k] = live0[k] && r0 + k >= 1 && r0 + k <= TY;
-  }
+  const int rows = TY + 2;
+  // this thread: quad qx of row r (y = y0 - 1 + r; rows 0 and TY + 1 are the
+  // halo of stage 0); lanes past the last row alias its addresses for their
+  // loads and store nothing
+  const int qx = tid % QW;
+  const bool lane_ok = tid < rows * QW;
+  const int r = lane_ok ? tid / QW : rows - 1;
+  const int y = y0 - 1 + r;
+  const bool live = lane_ok && y >= 0 && y < a.Ly() && qx < a.Wq();
+  const bool own_row = live && r >= 1 && r <= TY;  // a row of this tile: written out
+  const bool warp_in0 = (tid & ~31) < rows * QW;
   const int n_ring = nz + 4;  // colour-1 planes z0 - 2 .. z0 + nz + 1
   T *dst0 = a.dst();
   T *dst1 = dst0 + a.colour_elems();
@@ -140,8 +138,9 @@ __device__ bool march_pass(const Job &a, const PhiloxKeys &K, unsigned char *sme
     const uint32_t bar = smem_addr(&bars[(gb + j) % kPassStages]);
     const bool own = OR && j >= 2;
     mbar_arrive_expect_tx(bar, lay.c1_bytes + (own ? lay.c0_bytes : 0));
-    tma_load_4d(smem_addr(c1_slot(j)), a.tm_c1(), 0, y0 - 2, z0 - 2 + j, a.map_c1(), bar);
-    if (own) tma_load_4d(smem_addr(c0_slot(j)), a.tm_c0(), 0, y0 - 1, z0 - 3 + j, a.map_c0(), bar);
+    const uint32_t slot = smem_addr(at(slot_at(j)));
+    tma_load_4d(slot, a.tm_c1(), 0, y0 - 2, z0 - 2 + j, a.map_c1(), bar);
+    if (own) tma_load_4d(slot + c0_off, a.tm_c0(), 0, y0 - 1, z0 - 3 + j, a.map_c0(), bar);
   };
   auto wait_plane = [&](int j) -> bool {
     return mbar_wait_bounded(smem_addr(&bars[(gb + j) % kPassStages]),
@@ -169,177 +168,141 @@ __device__ bool march_pass(const Job &a, const PhiloxKeys &K, unsigned char *sme
     if (2 * (4 * qx + i) >= a.Lx()) pad0 |= 1u << i;
     if (2 * (4 * qx + i) + 1 >= a.Lx()) pad1 |= 1u << i;
   }
+  // the whole warp is inside the box and has no padding lanes
+  const bool warp_full = __all_sync(0xffffffffu, live && pad0 == 0u && pad1 == 0u);
   const bool lo_ok = qx > 0, hi_ok = 4 * qx + 4 < W;
-  const int row = r0 * W + 4 * qx;  // first row of this thread in a box starting at y0 - 1
-  T *out0 = dst0 + (size_t)yk[0] * W + 4 * qx;
-  T *out1 = dst1 + (size_t)yk[0] * W + 4 * qx;
-  const size_t plane = (size_t)a.Ly() * W;
+  // byte offsets: row r of the colour-0 box and of the buffers; the colour-1
+  // box holds it one row further
+  const uint32_t wb = (uint32_t)W * (uint32_t)sizeof(T);
+  const uint32_t o_r = (uint32_t)r * wb + (uint32_t)(4 * qx) * (uint32_t)sizeof(T);
+  const uint32_t bb = (uint32_t)lay.new_bytes;
+  const uint32_t b_r = (uint32_t)(kHeaderBytes + kPassStages * lay.slot_bytes) + o_r;
+  const size_t plane_elems = (size_t)a.Ly() * W;
+  const size_t row_off = (size_t)(y < 0 ? 0 : y) * W + 4 * qx;
+  // Philox counter word 0 of the quad at plane p: (p Ly + y) Wq + qx
+  const uint32_t qrow = (uint32_t)y * (uint32_t)a.Wq() + (uint32_t)qx;
+  const uint32_t qplane = (uint32_t)a.Ly() * (uint32_t)a.Wq();
+  const uint32_t rng = a.rng_id();
 
-  // registers along z, per row: colour 1 old at p0 - 1, p0, p0 + 1; colour 0
-  // new at p1 - 1, p1, p1 + 1 (p1 = p0 - 1)
-  T am[R][4], ac[R][4], ap[R][4], nm[R][4], nc[R][4], np[R][4];
-#pragma unroll
-  for (int k = 0; k < R; ++k)
-#pragma unroll
-    for (int i = 0; i < 4; ++i) am[k][i] = ac[k][i] = ap[k][i] = nm[k][i] = nc[k][i] = np[k][i] = T(0);
-  bool ok = wait_plane(0);
-  if (ok && in_tile)
-#pragma unroll
-    for (int k = 0; k < R; ++k) ld_quad(c1_slot(0) + row + (k + 1) * W, am[k]);
-  ok = ok && wait_plane(1);
-  if (ok && in_tile)
-#pragma unroll
-    for (int k = 0; k < R; ++k) ld_quad(c1_slot(1) + row + (k + 1) * W, ac[k]);
-  if (!ok) {
-    atomicOr(err, kErrTimeout);
-    *abort_flag = 1;
+  {
+    const bool ok = wait_plane(0) && wait_plane(1);
+    if (!ok) {
+      atomicOr(err, kErrTimeout);
+      *abort_flag = 1;
+    }
   }
   __syncthreads();
   bool aborted = *abort_flag != 0;
   int done = 1;  // ring planes 0 .. done waited for by every thread
 
-  // One step s: stage 0 at p0 = z0 - 1 + s, then stage 1 at p0 - 1.  The
-  // register triples rotate from step to step (A0 = plane - 1, A1 = plane,
-  // A2 = plane + 1; A2 and N2 written here); the loop below calls it with the
-  // names rotated, so no values are moved.  The y neighbours inside the
-  // thread's rows come from its own registers, the outer two from shared
-  // memory.
-  auto step = [&](int s, T(&A0)[R][4], T(&A1)[R][4], T(&A2)[R][4], T(&N0)[R][4],
-                  T(&N1)[R][4], T(&N2)[R][4]) -> bool {
-    const int j = s + 2;
-    const int p0 = z0 - 1 + s;
-    const bool got = wait_plane(j);
-    T v0[R][4];
-#pragma unroll
-    for (int k = 0; k < R; ++k)
-#pragma unroll
-      for (int i = 0; i < 4; ++i) v0[k][i] = T(0);
-    if (got) {
-      const T *C1 = c1_slot(j) + row;
-#pragma unroll
-      for (int k = 0; k < R; ++k) {
-        if (in_tile) {
-          ld_quad(C1 + (k + 1) * W, A2[k]);
-        } else {
-#pragma unroll
-          for (int i = 0; i < 4; ++i) A2[k][i] = T(0);
-        }
-      }
-      if (in_tile && p0 >= 0 && p0 < a.Lz()) {
-        const T *Pz = c1_slot(j - 1) + row;  // colour 1 old, plane p0; row r0 + k at + (k + 1) W
-        T lo[4], hi[4];
-        ld_quad(Pz, lo);                // row r0 - 1
-        ld_quad(Pz + (R + 1) * W, hi);  // row r0 + R
-#pragma unroll
-        for (int k = 0; k < R; ++k) {
-          if (!live0[k]) continue;
-          const T *ym = k == 0 ? lo : A1[k - 1];
-          const T *yp = k == R - 1 ? hi : A1[k + 1];
-          T xs[4], S[4];
-          const int par = (yk[k] + p0) & 1;
-          const bool odd = par != 0;
-          const T e = (odd ? hi_ok : lo_ok) ? Pz[(k + 1) * W + (odd ? 4 : -1)] : T(0);
-          x_neighbours(odd, e, A1[k], xs);
-#pragma unroll
-          for (int i = 0; i < 4; ++i)
-            S[i] = ((A0[k][i] + A2[k][i]) + (ym[i] + yp[i])) + (A1[k][i] + xs[i]);
-          if (!OR) {
-            const uint32_t quad = ((uint32_t)p0 * (uint32_t)a.Ly() + (uint32_t)yk[k]) *
-                                      (uint32_t)a.Wq() + (uint32_t)qx;
-            const uint4 w = philox4x32_10(make_uint4(quad, pass, a.rng_id(), 0u), K);
-            v0[k][0] = fma(S[0], Coef<T>::sixth, Noise<T>::of(w.x));
-            v0[k][1] = fma(S[1], Coef<T>::sixth, Noise<T>::of(w.y));
-            v0[k][2] = fma(S[2], Coef<T>::sixth, Noise<T>::of(w.z));
-            v0[k][3] = fma(S[3], Coef<T>::sixth, Noise<T>::of(w.w));
-          } else {
-            T old[4];
-            ld_quad(c0_slot(j) + row + k * W, old);
-#pragma unroll
-            for (int i = 0; i < 4; ++i) v0[k][i] = fma(S[i], Coef<T>::third, -old[i]);
-          }
-          const uint32_t pm = par ? pad1 : pad0;
-          if (pm) {
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-              if ((pm >> i) & 1u) v0[k][i] = T(0);
-          }
-          if (live1[k] && p0 >= z0 && p0 < z0 + nz)
-            st_quad(out0 + (size_t)p0 * plane + (size_t)k * W, v0[k]);
-        }
-      }
-      if (in_tile)
-#pragma unroll
-        for (int k = 0; k < R; ++k) st_quad(new_plane(s) + row + k * W, v0[k]);
-    } else {
+  // windows of the quad's three planes: old colour 1 (P), new colour 0 (N)
+  Quad<T> P0 = qzero<T>(), P1 = qzero<T>(), P2 = qzero<T>();
+  Quad<T> N0 = qzero<T>(), N1 = qzero<T>(), N2 = qzero<T>();
+  if (!aborted) {
+    P0 = qload<T>(at(slot_at(0) + o_r + wb));
+    P1 = qload<T>(at(slot_at(1) + o_r + wb));
+  }
+
+  // What advances from step to step: this thread's row in the ring slots of
+  // planes s + 1 and s + 2, the mbarrier of plane s + 2 and its parity, the
+  // buffer, the row parity, the output pointer of stage 0's plane.
+  const uint32_t ring_o = (uint32_t)kHeaderBytes + o_r;
+  const uint32_t ring_end = ring_o + (uint32_t)(kPassStages * lay.slot_bytes);
+  uint32_t n1 = slot_at(1) + o_r, n2 = slot_at(2) + o_r;
+  const uint32_t bar0 = smem_addr(bars);
+  uint32_t bar_n = bar0 + 8u * (uint32_t)((gb + 2) % kPassStages);
+  uint32_t par_n = (uint32_t)(((gb + 2) / kPassStages) & 1);
+  uint32_t w_r = b_r;                  // the buffer row the step writes (the other is read)
+  const uint32_t b_sum = 2u * b_r + bb;
+  bool odd = ((y + z0 - 1) & 1) != 0;  // the same row parity for both stages
+  T *out = dst0 + (ptrdiff_t)(z0 - 1) * (ptrdiff_t)plane_elems + row_off;  // plane f
+  const ptrdiff_t out1 = (ptrdiff_t)a.colour_elems() - (ptrdiff_t)plane_elems;
+
+  // Step s, stage 0 at plane f = z0 - 1 + s and stage 1 at f - 1, with the
+  // windows' names rotated by the caller.  At entry: P0, P1 = old colour 1 at
+  // f - 1, f (P2 loaded here: f + 1); N0, N1 = new colour 0 at f - 2, f - 1
+  // (N2 made here: f).  Ring planes s, s + 1 have arrived; s + 2 is waited
+  // for here.  The deviates and stage 0 read no other warp's work of this
+  // step and come before its one barrier, so that a warp through the previous
+  // step goes on with them; stage 1 reads the previous step's buffer after
+  // it.  STEADY: s >= 3.
+  auto step = [&](auto steady, int s, Quad<T> &P0, Quad<T> &P1, Quad<T> &P2, Quad<T> &N0,
+                  Quad<T> &N1, Quad<T> &N2) -> bool {
+    constexpr bool STEADY = decltype(steady)::value;
+    const int f = z0 - 1 + s;
+    const bool e_ok = odd ? hi_ok : lo_ok;
+    const uint32_t eo = odd ? 4u * (uint32_t)sizeof(T) : 0u - (uint32_t)sizeof(T);
+    // nothing to zero in either stage
+    const bool fast = warp_full && (STEADY || f >= 0) && f < Lz;
+    bool got = mbar_wait_bounded(bar_n, par_n);
+    // the heatbath deviates take the whole warp through the same path
+    if (!OR) got = __all_sync(0xffffffffu, got);
+    if (!got) {
       atomicOr(err, kErrTimeout);
       *abort_flag = 1;
     }
-#pragma unroll
-    for (int k = 0; k < R; ++k)
-#pragma unroll
-      for (int i = 0; i < 4; ++i) N2[k][i] = v0[k][i];
-    // ---- stage 1: colour 1 at plane p1 = p0 - 1 on this tile's rows.  It
-    // reads the new colour-0 rows of plane p1 (written in the previous step,
-    // before the barrier that ends it) and this thread's own registers, none
-    // of what stage 0 of this step wrote to shared memory, so no barrier
-    // between the stages.
-    const int p1 = p0 - 1;
-    if (s >= 2 && (live1[0] || live1[R - 1])) {
-      const T *N = new_plane(s - 1) + row;  // colour 0 new, plane p1
-      T lo[4], hi[4];
-      if (live1[0]) ld_quad(N - W, lo);      // row r0 - 1 (r0 >= 1 here)
-      if (live1[R - 1]) ld_quad(N + R * W, hi);  // row r0 + R (<= TY + 1 here)
-#pragma unroll
-      for (int k = 0; k < R; ++k) {
-        if (!live1[k]) continue;
-        const T *ym = k == 0 ? lo : N1[k - 1];
-        const T *yp = k == R - 1 ? hi : N1[k + 1];
-        T xs[4], S[4], v[4];
-        const int par = (1 + yk[k] + p1) & 1;
-        const bool odd = par != 0;
-        const T e = (odd ? hi_ok : lo_ok) ? N[k * W + (odd ? 4 : -1)] : T(0);
-        x_neighbours(odd, e, N1[k], xs);
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-          S[i] = ((N0[k][i] + N2[k][i]) + (ym[i] + yp[i])) + (N1[k][i] + xs[i]);
-        if (!OR) {
-          const uint32_t quad = ((uint32_t)p1 * (uint32_t)a.Ly() + (uint32_t)yk[k]) *
-                                    (uint32_t)a.Wq() + (uint32_t)qx;
-          const uint4 w = philox4x32_10(make_uint4(quad, pass, a.rng_id(), 1u), K);
-          v[0] = fma(S[0], Coef<T>::sixth, Noise<T>::of(w.x));
-          v[1] = fma(S[1], Coef<T>::sixth, Noise<T>::of(w.y));
-          v[2] = fma(S[2], Coef<T>::sixth, Noise<T>::of(w.z));
-          v[3] = fma(S[3], Coef<T>::sixth, Noise<T>::of(w.w));
-        } else {
-          // colour 1's own old value at plane p1 = p0 - 1 is A0
-#pragma unroll
-          for (int i = 0; i < 4; ++i) v[i] = fma(S[i], Coef<T>::third, -A0[k][i]);
-        }
-        const uint32_t pm = par ? pad1 : pad0;
-        if (pm) {
-#pragma unroll
-          for (int i = 0; i < 4; ++i)
-            if ((pm >> i) & 1u) v[i] = T(0);
-        }
-        st_quad(out1 + (size_t)p1 * plane + (size_t)k * W, v);
+    Quad<T> n0 = qzero<T>(), n1_dev = qzero<T>();
+    if (got && (!Job::kIdleWarps || warp_in0)) {
+      if (!OR) {
+        const uint4 w0 =
+            philox4x32_10(make_uint4((uint32_t)f * qplane + qrow, pass, rng, 0u), K);
+        const uint4 w1 =
+            philox4x32_10(make_uint4((uint32_t)(f - 1) * qplane + qrow, pass, rng, 1u), K);
+        StageNoise<T>::of(w0, w1, n0, n1_dev);
       }
+      // ---- stage 0: colour 0 at plane f (ring only)
+      P2 = qload<T>(at(n2 + wb));
+      const Quad<T> ym = qload<T>(at(n1)), yp = qload<T>(at(n1 + 2u * wb));
+      const T e = e_ok ? *at(n1 + wb + eo) : T(0);
+      if (OR) n0 = qload<T>(at(n2 + c0_off));
+      N2 = update<T, OR>(P0, P2, ym, yp, P1, odd, e, n0);
+      if (!fast) mask(N2, live && f >= 0 && f < Lz, odd ? pad1 : pad0);
     }
-    // new plane s visible to the next step's stage 1; new plane s - 1 and
-    // ring plane s free for reuse
     __syncthreads();
     if (*abort_flag) return false;
-    done = j;
+    done = s + 2;
+    // ring plane s was last read in the previous step: refill its slot
     if (tid == 0 && issued < n_ring) issue(issued++);
+    if (lane_ok) qstore(at(w_r), N2);
+    // the tile's planes: s = 1 .. nz
+    if (own_row && (STEADY || s >= 1) && s <= nz) qstore(out, N2);
+    // ---- stage 1: colour 1 at plane f - 1 (old value: P0)
+    if ((STEADY || s >= 2) && own_row) {
+      const uint32_t br = b_sum - w_r;
+      const Quad<T> ym = qload<T>(at(br - wb)), yp = qload<T>(at(br + wb));
+      const T e = e_ok ? *at(br + eo) : T(0);
+      Quad<T> v = update<T, OR>(N0, N2, ym, yp, N1, odd, e, OR ? P0 : n1_dev);
+      if (!fast) mask(v, true, odd ? pad1 : pad0);
+      qstore(out + out1, v);
+    }
+    n1 = n2;
+    n2 += (uint32_t)lay.slot_bytes;
+    if (n2 == ring_end) n2 = ring_o;
+    bar_n += 8u;
+    if (bar_n == bar0 + 8u * kPassStages) {
+      bar_n = bar0;
+      par_n ^= 1u;
+    }
+    w_r = b_sum - w_r;
+    odd = !odd;
+    out += plane_elems;
     return true;
   };
 
   const int n_steps = nz + 2;
-  for (int s = 0; s < n_steps && !aborted; s += 3) {
-    if (!step(s, am, ac, ap, nm, nc, np)) { aborted = true; break; }
+  using First = std::integral_constant<bool, false>;
+  using Steady = std::integral_constant<bool, true>;
+  if (!aborted)
+    aborted = !(step(First(), 0, P0, P1, P2, N0, N1, N2) &&
+                step(First(), 1, P1, P2, P0, N1, N2, N0) &&
+                step(First(), 2, P2, P0, P1, N2, N0, N1));
+#pragma unroll 1
+  for (int s = 3; s < n_steps && !aborted; s += 3) {
+    if (!step(Steady(), s, P0, P1, P2, N0, N1, N2)) { aborted = true; break; }
     if (s + 1 >= n_steps) break;
-    if (!step(s + 1, ac, ap, am, nc, np, nm)) { aborted = true; break; }
+    if (!step(Steady(), s + 1, P1, P2, P0, N1, N2, N0)) { aborted = true; break; }
     if (s + 2 >= n_steps) break;
-    if (!step(s + 2, ap, am, ac, np, nm, nc)) { aborted = true; break; }
+    if (!step(Steady(), s + 2, P2, P0, P1, N2, N0, N1)) { aborted = true; break; }
   }
   if (aborted && tid == 0) {
     // leave no copy in flight into this CTA's shared memory
