@@ -292,6 +292,121 @@ Tile fill_grid(const Geometry &g, Tile t, int target, int min_dz) {
   return t;
 }
 
+// Time of one launch over all chains (us) of a march kernel with this tile,
+// as far as the tile decides it.  CTAs run in waves of as many as an SM holds
+// (registers, shared memory, threads); a wave takes its steps (planes and
+// halo planes) times the largest of a step's latency, the issue time of the
+// SM's warps and its TMA rows, and a start; the launch is no shorter than its
+// reads (with the halo) and writes take (joined as cubes: neither hides the
+// other fully near the line).  Constants per kernel and precision, fitted to
+// 24 FP32 and 9 FP64 lattices (16^3 x 512 to 512^3, 2000 tiles) within 13%
+// rms near each one's best tile.
+enum TileKind { kTileHalf, kTilePassK, kTilePairK };
+struct TileCost {
+  int regs;      // per thread, for the CTAs an SM holds
+  double warp;   // us of an SM per warp and step
+  double step;   // us: least time of a step
+  double row;    // us of an SM per TMA row and step
+  double wave, cta;  // us: start of a wave, of each CTA of an SM
+  double bytes;  // bytes per us
+};
+constexpr TileCost kTileCost[3][2] = {
+    {{96, 0.060, 0.77, 0.0, 1.0, 0.010, 7.3e6}, {80, 0.40, 2.9, 0.033, 1.0, 0.012, 1.9e6}},
+    {{64, 0.0268, 0.57, 0.0029, 3.1, 0.025, 10.6e6}, {96, 0.41, 2.2, 0.031, 1.0, 0.015, 2.7e6}},
+    {{120, 0.0437, 0.59, 0.0017, 1.0, 0.098, 10.1e6}, {160, 0.67, 1.0, 0.040, 1.0, 0.012, 1.1e6}}};
+
+double tile_time(const Geometry &g, TileKind kind, const Tile &t, int sms) {
+  const bool f64 = g.precision == COULPS_F64;
+  const TileCost &k = kTileCost[kind][f64 ? 1 : 0];
+  const double row_bytes = (double)g.W * g.es;
+  const int qw = g.W / 4;
+  int threads, steps, planes, box_rows;
+  size_t smem;
+  if (kind == kTilePairK) {
+    threads = pair_threads(g, t); steps = t.dz + 6; planes = 8; box_rows = 2 * t.ty + 14;
+    smem = pair_smem_bytes(g, t, true);
+  } else if (kind == kTilePassK) {
+    threads = pass_threads(g, t); steps = t.dz + 2; planes = 4; box_rows = 2 * t.ty + 6;
+    smem = pass_smem_bytes(g, t, true);
+  } else {
+    // heatbath (FP32: two quads per thread); the other colour only
+    threads = ((f64 ? qw : (qw + 1) / 2) * t.ty + 31) / 32 * 32; steps = t.dz + 2; planes = 2;
+    box_rows = t.ty + 2;
+    smem = halfsweep_smem_bytes(g, t, false);
+  }
+  const int per_sm = std::max(1, std::min(std::min(65536 / (k.regs * threads), 2048 / threads),
+                                          std::min((int)(228 * 1024 / (smem + 1024)), 32)));
+  const int64_t ny = (g.Ly + t.ty - 1) / t.ty, nz = (g.Lz + t.dz - 1) / t.dz;
+  const int64_t ctas = ny * nz * g.n_chains, full = ctas / ((int64_t)sms * per_sm);
+  const int64_t rest = (ctas - full * sms * per_sm + sms - 1) / sms;
+  auto wave = [&](int64_t n) {
+    return steps * std::max(k.step, (double)n * std::max(threads / 32 * k.warp, box_rows * k.row)) +
+           k.wave + k.cta * (double)n;
+  };
+  const double work = (double)full * wave(per_sm) + (rest > 0 ? wave(rest) : 0.0);
+  const double volume = row_bytes * g.Ly * g.Lz * g.n_chains;
+  const double traffic =
+      row_bytes * box_rows * (double)(ny * g.n_chains) * (double)(g.Lz + nz * planes) +
+      volume * (kind == kTileHalf ? 1.0 : 2.0);
+  const double mem = traffic / k.bytes;
+  return std::cbrt(work * work * work + mem * mem * mem) + 4.0;
+}
+
+// A lattice's tile for one kernel: the default shape t, unless the estimate
+// finds one clearly shorter (below `clear` of the default's): rows that divide
+// Ly evenly or the most that fit, slabs that divide Lz evenly (half-sweeps:
+// 4 .. 16 planes by whole groups of ring waits; longer slabs measured slower
+// than estimated).  What the default shape costs is mostly a nearly empty last
+// wave or CTAs that leave SMs idle: pass pair of 64^3 x 128 chains 125 us with
+// 58 x 32 (256 CTAs of one per SM: two waves), 85 with 22 x 32; 128^3 x 16 109
+// (160 CTAs, two waves) -> 73; 160 x 96 x 130 x 8 62 -> 41; fused pass of
+// 96^3 x 16 34.8 -> 24.5.  Below 2^19 sites a launch is its latency whatever
+// the tile, and most such sweeps run resident: the default shapes stay.
+Tile best_tile(const Geometry &g, TileKind kind, Tile t, int sms, double clear) {
+  if (t.ty < 1 || t.dz < 1 || sms < 1) return t;
+  if (2 * (int64_t)g.colour_elems * g.n_chains < ((int64_t)1 << 19)) return t;
+  const int qw = g.W / 4;
+  const int threads = kind == kTilePairK
+                          ? (g.precision == COULPS_F32 ? kPairMaxThreads32 : kPairMaxThreads64)
+                          : (kind == kTilePassK ? 512 : 256);
+  const int halo = kind == kTilePairK ? 6 : (kind == kTilePassK ? 2 : 0);
+  const int ty_max = std::min(std::min(threads / qw - halo, g.Ly), 248);
+  double best = clear * tile_time(g, kind, t, sms);
+  Tile out = t;
+  int last_ty = 0;
+  for (int ny = 1; ny <= g.Ly; ++ny) {
+    int ty = (g.Ly + ny - 1) / ny;
+    if (ty > ty_max) {
+      if ((g.Ly + ny) / (ny + 1) > ty_max) continue;
+      ty = ty_max;  // the most rows that fit, ahead of the first even division
+    }
+    if (ty < 2 || ty == last_ty) continue;
+    last_ty = ty;
+    int last_dz = 0;
+    for (int nz = 1; nz <= g.Lz; ++nz) {
+      int dz = (g.Lz + nz - 1) / nz;
+      if (kind == kTileHalf) {
+        if (nz > 4) break;
+        dz = 4 * nz;
+      }
+      if (dz < 4) break;
+      if (dz == last_dz || dz > g.Lz) continue;
+      last_dz = dz;
+      const Tile c{ty, dz};
+      const size_t smem = kind == kTilePairK   ? pair_smem_bytes(g, c, true)
+                          : kind == kTilePassK ? pass_smem_bytes(g, c, true)
+                                               : halfsweep_smem_bytes(g, c, true);
+      if (smem > 227 * 1024) continue;
+      const double e = tile_time(g, kind, c, sms);
+      if (e < best) {
+        best = e;
+        out = c;
+      }
+    }
+  }
+  return out;
+}
+
 // The resident plan of a lattice: the cluster size with the shortest compound
 // sweep of 1 heatbath : 3 over-relaxation passes; {cluster = 0} if the chain
 // fits no cluster.
@@ -1249,7 +1364,8 @@ int coulps_lattice_create(int Lx, int Ly, int Lz, int n_chains, int precision, u
   if (!L) return COULPS_ENOMEM;
   L->g = g;
   const int sms = device_sms();
-  L->tile = fill_grid(g, default_tile(g), 2 * sms, 4);
+  L->tile = best_tile(g, kTileHalf, fill_grid(g, default_tile(g), 2 * sms, 4), sms,
+                      g.precision == COULPS_F32 ? 0.86 : 0.93);
   L->seed = seed;
   L->stream = (cudaStream_t)stream;
   L->alloc = g_allocator;
@@ -1306,9 +1422,13 @@ static int set_fused(coulps_lattice *L, int enable) {
     // row padding and never-written quads stay 0 in both copies
     CK(cudaMemsetAsync(L->field2, 0, fbytes, L->stream));
   }
-  if (L->ptile.ty == 0) L->ptile = fill_grid(L->g, default_pass_tile(L->g), 2 * device_sms(), 4);
+  const int sms = device_sms();
+  if (L->ptile.ty == 0)
+    L->ptile = best_tile(L->g, kTilePassK, fill_grid(L->g, default_pass_tile(L->g), 2 * sms, 4),
+                         sms, 0.93);
   if (enable >= 3 && L->qtile.ty == 0)
-    L->qtile = fill_grid(L->g, default_pair_tile(L->g), device_sms(), 8);
+    L->qtile = best_tile(L->g, kTilePairK, fill_grid(L->g, default_pair_tile(L->g), sms, 8), sms,
+                         0.93);
   L->fused = enable;
   int st = rebuild_maps(L);
   if (st) return st;
