@@ -252,13 +252,16 @@ Tile default_pass_tile(const Geometry &g) {
 
 // Pass-pair tile: the CTA computes ty + 6 rows (3 halo rows each side) of
 // W / 4 quads, one thread per quad, within 512 threads (FP32) or 256 (FP64);
-// {0, 0} when fewer than 4 rows fit (the halo would dominate).  z slabs of
+// {0, 0} when fewer than 4 rows fit (the halo would dominate), and for FP64:
+// the FP64 unit is the bound there, and a pair's halo rows and planes cost it
+// more than the second trip through memory costs two fused passes (best tiles of each: 128^3 x 8 chains 685 us against 2 x 260, 96^3 x 8
+// 297 against 2 x 115, 64^3 x 4 65 against 2 x 29).  z slabs of
 // 64 planes from Lz = 128 (measured at 128^3 x 64 chains, two streams: 0.802
 // ms per 1 HB : 3 OR compound sweep against 0.828 with 32 planes).
 Tile default_pair_tile(const Geometry &g) {
+  if (g.precision == COULPS_F64) return Tile{0, 0};
   const int qw = g.W / 4;
-  const int max_threads = g.precision == COULPS_F32 ? kPairMaxThreads32 : kPairMaxThreads64;
-  int ty = max_threads / qw - 6;
+  int ty = kPairMaxThreads32 / qw - 6;
   if (ty > g.Ly) ty = g.Ly;
   if (ty > 248) ty = 248;  // TMA box rows ty + 8 <= 256
   const int dz = g.Lz >= 128 ? 64 : (g.Lz >= 64 ? 32 : g.Lz);
@@ -360,11 +363,13 @@ double tile_time(const Geometry &g, TileKind kind, const Tile &t, int sms) {
 // wave or CTAs that leave SMs idle: pass pair of 64^3 x 128 chains 125 us with
 // 58 x 32 (256 CTAs of one per SM: two waves), 85 with 22 x 32; 128^3 x 16 109
 // (160 CTAs, two waves) -> 73; 160 x 96 x 130 x 8 62 -> 41; fused pass of
-// 96^3 x 16 34.8 -> 24.5.  Below 2^19 sites a launch is its latency whatever
-// the tile, and most such sweeps run resident: the default shapes stay.
+// 96^3 x 16 34.8 -> 24.5.  Below 2^19 FP32 sites a launch is its latency
+// whatever the tile, and most such sweeps run resident: the default shapes stay.
 Tile best_tile(const Geometry &g, TileKind kind, Tile t, int sms, double clear) {
   if (t.ty < 1 || t.dz < 1 || sms < 1) return t;
-  if (2 * (int64_t)g.colour_elems * g.n_chains < ((int64_t)1 << 19)) return t;
+  if (g.precision == COULPS_F32 &&
+      2 * (int64_t)g.colour_elems * g.n_chains < ((int64_t)1 << 19))
+    return t;
   const int qw = g.W / 4;
   const int threads = kind == kTilePairK
                           ? (g.precision == COULPS_F32 ? kPairMaxThreads32 : kPairMaxThreads64)
@@ -428,15 +433,16 @@ ResidentPlan resident_plan(const Geometry &g) {
 // Time of a compound sweep by the march kernels (us): launches of 5 us at
 // least each, then the work of their passes.  Fitted to measured sweeps
 // (FP32 1:3: 64^3 x 1 37.4, x 12 62, x 64 163, 72^3 x 30 137; 1:0: 19, 23,
-// 58, 48; FP64 1:3: 64^3 x 1 153, 40^3 x 30 185, 80^3 x 4 329; 1:0: 48, 72,
-// 115), for FP64 on the low side.
+// 58, 48; FP64 1:3: 64^3 x 2 86, 40^3 x 30 172, 40^3 x 60 308, 48 x 30 x 20 x 200
+// 573; 1:0: 41, 74, 130, 205), for FP64 between even and uneven shapes.
 double march_time(const Geometry &g, int n_hb, int n_or) {
   const double sites = 2.0 * (double)g.colour_elems * g.n_chains;
   const int trips = (n_or + 1) / 2;
   if (g.precision == COULPS_F32)
     return std::max(5.0 * (2 * n_hb + 2) + 9.0 * trips,
                     15.0 + 5.0 * trips + sites * (2.8e-6 * n_hb + 1.9e-6 * n_or));
-  return std::max(38.0 * n_hb + 19.0 * n_or, sites * (4.0e-5 * n_hb + 2.5e-5 * n_or));
+  return std::max(38.0 * n_hb + 19.0 * n_or,
+                  14.0 * n_hb + 8.0 * n_or + sites * (3.4e-5 * n_hb + 1.8e-5 * n_or));
 }
 
 int rebuild_pass_maps(coulps_lattice *L) {
@@ -517,10 +523,10 @@ PassPlan pass_plan(const coulps_lattice *L, int n_hb, int n_or) {
 // the shorter way (profiling times the march kernels one by one, the other
 // schedules are theirs).  The same for every number of sweeps, so that a run
 // gives bitwise the same samples however it is divided into calls.  Measured
-// (us per compound sweep, march against resident): FP64 16^3 x 1 94 -> 7.7
-// (1:0 39 -> 2.7), 32^3 x 1 112 -> 28, 40^3 x 30 185 -> 177; FP32 16^3 x 1
-// 31 -> 4.7, 64^3 x 1 37 -> 18, x 30 94 -> 58, x 64 163 -> 112, 80^3 x 12 79 ->
-// 67, and past the line 80^3 x 30 147 -> 166, FP64 64^3 x 4 172 -> 177.
+// (us per compound sweep, march against resident): FP64 16^3 x 1 88 -> 7.0
+// (1:0 35 -> 3.2), 32^3 x 1 111 -> 27, 32^3 x 100 287 -> 270; FP32 16^3 x 1
+// 31 -> 4.7, 64^3 x 1 34 -> 18, x 30 68 -> 58, x 64 118 -> 112, and past the
+// line 80^3 x 30 109 -> 166, FP64 40^3 x 60 308 -> 350, 64^3 x 4 115 -> 177.
 bool resident_on(const coulps_lattice *L, int n_hb, int n_or) {
   if (L->rplan.cluster == 0 || L->pinned || L->profiling ||
       L->schedule != COULPS_SCHEDULE_ALIGNED || n_hb + n_or == 0)
