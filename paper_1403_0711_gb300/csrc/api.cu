@@ -527,22 +527,42 @@ PassPlan pass_plan(const coulps_lattice *L, int n_hb, int n_or) {
 // (1:0 35 -> 3.2), 32^3 x 1 111 -> 27, 32^3 x 100 287 -> 270; FP32 16^3 x 1
 // 31 -> 4.7, 64^3 x 1 34 -> 18, x 30 68 -> 58, x 64 118 -> 112, and past the
 // line 80^3 x 30 109 -> 166, FP64 40^3 x 60 308 -> 350, 64^3 x 4 115 -> 177.
-bool resident_on(const coulps_lattice *L, int n_hb, int n_or) {
+//
+// n_sweeps = 0: sampled runs (one launch for many sweeps).  n_sweeps > 0: that
+// many sweeps in a launch, whose samples, if any, something else takes: their
+// launch, load and store count too (a launch of one sweep, us beyond the sweep:
+// 16^3 x 1 11, 64^3 x 1 13, x 30 24, 80^3 x 1 16), and the march is taken nearer
+// its measured time than the formula's (one off-lattice sample per sweep, march
+// against resident: 64^3 x 30 70 against 84, 157 x 36 x 41 x 12 1:1 33 against 41,
+// 48^3 x 4 35 against 29, FP64 48^3 x 4 87 against 97, 24^3 x 30 83 against 62).
+bool resident_on(const coulps_lattice *L, int n_hb, int n_or, int n_sweeps = 0) {
   if (L->rplan.cluster == 0 || L->pinned || L->profiling ||
       L->schedule != COULPS_SCHEDULE_ALIGNED || n_hb + n_or == 0)
     return false;
-  return resident_time(L->g, L->rplan, n_hb, n_or) < 0.9 * march_time(L->g, n_hb, n_or);
+  const Geometry &g = L->g;
+  const ResidentPlan &p = L->rplan;
+  double t = resident_time(g, p, n_hb, n_or), clear = 0.9;
+  if (n_sweeps > 0) {
+    const int waves = (g.n_chains + p.active - 1) / p.active;
+    t += (8.0 + waves * (2.5 + 0.02e-3 * (double)p.smem)) / n_sweeps;
+    if (n_sweeps < 8) clear = g.precision == COULPS_F32 ? 0.75 : 0.85;
+  }
+  return t < clear * march_time(g, n_hb, n_or);
 }
 
 // The tile by which a measured compound sweep (aligned schedule) gathers Q
-// and P: one column of planes (resident), or that of its last kernel, the
-// pass pair's, the fused pass's, or the half-sweep's.
-Tile fused_gather_tile(const coulps_lattice *L, int n_hb, int n_or) {
+// and P: that of its last kernel, the pass pair's, the fused pass's, or the
+// half-sweep's; one column of planes for the resident kernel.
+Tile march_gather_tile(const coulps_lattice *L, int n_hb, int n_or) {
   const int n = n_hb + n_or;
-  if (resident_on(L, n_hb, n_or)) return Tile{L->g.Ly, L->g.Lz};
   const PassPlan P = pass_plan(L, n_hb, n_or);
   if (P.head + 2 * P.pairs + P.singles < n || P.pairs + P.singles == 0) return L->tile;
   return P.singles > 0 ? L->ptile : L->qtile;
+}
+
+Tile fused_gather_tile(const coulps_lattice *L, int n_hb, int n_or, int n_sweeps = 0) {
+  if (resident_on(L, n_hb, n_or, n_sweeps)) return Tile{L->g.Ly, L->g.Lz};
+  return march_gather_tile(L, n_hb, n_or);
 }
 
 Tile default_tile(const Geometry &g) {
@@ -636,7 +656,7 @@ int enqueue_part(coulps_lattice *L, cudaStream_t st, int n_hb, int n_or, coulps_
   const int n_pass = n_hb + n_or;
   if (fuse) {
     // the charges must be grouped by the tile of the kernel that gathers
-    const Tile gt = fused_gather_tile(L, n_hb, n_or);
+    const Tile gt = march_gather_tile(L, n_hb, n_or);
     if (fuse->gather_dirty || fuse->gather_tile.ty != gt.ty || fuse->gather_tile.dz != gt.dz)
       return COULPS_EINVAL;
   }
@@ -797,7 +817,7 @@ int enqueue_resident(coulps_lattice *L, int n_sweeps, int n_hb, int n_or, coulps
 // kernels can share the GPU; each chain's passes, draws and sample are
 // unchanged.  The pass counter is advanced once, after the join.
 int enqueue_compound(coulps_lattice *L, int n_hb, int n_or, coulps_charges *fuse = nullptr) {
-  if (resident_on(L, n_hb, n_or)) return enqueue_resident(L, 1, n_hb, n_or, fuse);
+  if (resident_on(L, n_hb, n_or, 1)) return enqueue_resident(L, 1, n_hb, n_or, fuse);
   const int k = L->split < L->g.n_chains ? L->split : L->g.n_chains;
   if (k >= 2) {
     CK(cudaEventRecord(L->ev_fork, L->stream));
@@ -1591,7 +1611,7 @@ int coulps_field_set(coulps_lattice_t L, int chain, const double *host) {
 
 int coulps_sweep(coulps_lattice_t L, int n_compound, int n_hb, int n_or) {
   if (!L || n_compound < 0 || n_hb < 0 || n_or < 0) return COULPS_EINVAL;
-  if (resident_on(L, n_hb, n_or)) {
+  if (n_compound > 0 && resident_on(L, n_hb, n_or, n_compound)) {
     const int st = enqueue_resident(L, n_compound, n_hb, n_or, nullptr);
     if (!st) L->pass += (uint64_t)n_compound * (uint64_t)(n_hb + n_or);
     return st;
@@ -2452,7 +2472,7 @@ int coulps_gcv_run(coulps_gcv_t G, int n_meas, int n_hb, int n_or, double c) {
   if (n_meas == 0) return COULPS_OK;
   const bool fused = n_hb + n_or > 0;
   if (fused) {
-    int st = stage_gather(L, C, fused_gather_tile(L, n_hb, n_or));
+    int st = stage_gather(L, C, fused_gather_tile(L, n_hb, n_or, 1));
     if (st) return st;
   }
   auto one = [&]() -> int {
