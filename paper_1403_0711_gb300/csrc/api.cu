@@ -318,7 +318,8 @@ constexpr TileCost kTileCost[3][2] = {
     {{64, 0.0268, 0.57, 0.0029, 3.1, 0.025, 10.6e6}, {96, 0.41, 2.2, 0.031, 1.0, 0.015, 2.7e6}},
     {{120, 0.0437, 0.59, 0.0017, 1.0, 0.098, 10.1e6}, {160, 0.67, 1.0, 0.040, 1.0, 0.012, 1.1e6}}};
 
-double tile_time(const Geometry &g, TileKind kind, const Tile &t, int sms) {
+double tile_time(const Geometry &g, TileKind kind, const Tile &t, int sms,
+                 int64_t *full_waves = nullptr) {
   const bool f64 = g.precision == COULPS_F64;
   const TileCost &k = kTileCost[kind][f64 ? 1 : 0];
   const double row_bytes = (double)g.W * g.es;
@@ -342,6 +343,7 @@ double tile_time(const Geometry &g, TileKind kind, const Tile &t, int sms) {
   const int64_t ny = (g.Ly + t.ty - 1) / t.ty, nz = (g.Lz + t.dz - 1) / t.dz;
   const int64_t ctas = ny * nz * g.n_chains, full = ctas / ((int64_t)sms * per_sm);
   const int64_t rest = (ctas - full * sms * per_sm + sms - 1) / sms;
+  if (full_waves) *full_waves = full;
   auto wave = [&](int64_t n) {
     return steps * std::max(k.step, (double)n * std::max(threads / 32 * k.warp, box_rows * k.row)) +
            k.wave + k.cta * (double)n;
@@ -363,8 +365,11 @@ double tile_time(const Geometry &g, TileKind kind, const Tile &t, int sms) {
 // wave or CTAs that leave SMs idle: pass pair of 64^3 x 128 chains 125 us with
 // 58 x 32 (256 CTAs of one per SM: two waves), 85 with 22 x 32; 128^3 x 16 109
 // (160 CTAs, two waves) -> 73; 160 x 96 x 130 x 8 62 -> 41; fused pass of
-// 96^3 x 16 34.8 -> 24.5.  Below 2^19 FP32 sites a launch is its latency
-// whatever the tile, and most such sweeps run resident: the default shapes stay.
+// 96^3 x 16 34.8 -> 24.5.  From five full waves on they run into one
+// another and the default shapes stay (fused pass of 128^3 x 64 chains: 19 x 64,
+// three waves, would be 2% faster alone but 672 us a sweep on two streams, where
+// 13 x 32 makes 651).  Below 2^19 FP32 sites a launch is its latency whatever the
+// tile, and most such sweeps run resident: the default shapes stay as well.
 Tile best_tile(const Geometry &g, TileKind kind, Tile t, int sms, double clear) {
   if (t.ty < 1 || t.dz < 1 || sms < 1) return t;
   if (g.precision == COULPS_F32 &&
@@ -376,7 +381,9 @@ Tile best_tile(const Geometry &g, TileKind kind, Tile t, int sms, double clear) 
                           : (kind == kTilePassK ? 512 : 256);
   const int halo = kind == kTilePairK ? 6 : (kind == kTilePassK ? 2 : 0);
   const int ty_max = std::min(std::min(threads / qw - halo, g.Ly), 248);
-  double best = clear * tile_time(g, kind, t, sms);
+  int64_t waves = 0;
+  double best = clear * tile_time(g, kind, t, sms, &waves);
+  if (waves >= 5) return t;
   Tile out = t;
   int last_ty = 0;
   for (int ny = 1; ny <= g.Ly; ++ny) {
