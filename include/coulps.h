@@ -384,7 +384,7 @@ int coulps_set_schedule(coulps_lattice_t lat, int schedule);
  * fused passes so that the number of kernels is even (n = 1 pass: two
  * half-sweeps; n mod 4 = 0: n / 2 pairs; 1: (n - 3) / 2 pairs + 3 singles;
  * 2: n / 2 - 1 pairs + 2 singles; 3: (n - 1) / 2 pairs + 1 single).  Rows
- * too wide for a pair CTA (fewer than 4 rows fit) run enable = 3 as 1 and
+ * too wide for a pair CTA (fewer than 8 rows fit; FP64) run enable = 3 as 1 and
  * 4 as 2.  enable = 0 none (and frees the second copy).  Results are bitwise those of
  * the half-sweep path (same arithmetic per site, same Philox counters).  The
  * sample of a measured compound sweep is gathered by its last kernel.  Not

@@ -252,7 +252,10 @@ Tile default_pass_tile(const Geometry &g) {
 
 // Pass-pair tile: the CTA computes ty + 6 rows (3 halo rows each side) of
 // W / 4 quads, one thread per quad, within 512 threads (FP32) or 256 (FP64);
-// {0, 0} when fewer than 4 rows fit (the halo would dominate), and for FP64:
+// {0, 0} when fewer than 8 rows fit (the six halo rows then cost more than the
+// second trip; compound sweep 1:3 with pairs against fused passes: 4 rows, 384^3
+// 395 against 360 us, 7 rows, 300^3 x 2 373 against 344, 8 rows, 288^3 154 against
+// 163, 10 rows, 256^3 x 4 362 against 393), and for FP64:
 // the FP64 unit is the bound there, and a pair's halo rows and planes cost it
 // more than the second trip through memory costs two fused passes (best tiles of each: 128^3 x 8 chains 685 us against 2 x 260, 96^3 x 8
 // 297 against 2 x 115, 64^3 x 4 65 against 2 x 29).  z slabs of
@@ -266,7 +269,7 @@ Tile default_pair_tile(const Geometry &g) {
   if (ty > 248) ty = 248;  // TMA box rows ty + 8 <= 256
   const int dz = g.Lz >= 128 ? 64 : (g.Lz >= 64 ? 32 : g.Lz);
   while (ty >= 1 && pair_smem_bytes(g, Tile{ty, dz}, true) > 227 * 1024) --ty;
-  if (ty < 4 && ty < g.Ly) return Tile{0, 0};
+  if (ty < 8 && ty < g.Ly) return Tile{0, 0};
   if (ty < 1) return Tile{0, 0};
   return Tile{ty, dz};
 }
