@@ -304,24 +304,8 @@ Tile fill_grid(const Geometry &g, Tile t, int target, int min_dz) {
 // halo planes) times the largest of a step's latency, the issue time of the
 // SM's warps and its TMA rows, and a start; the launch is no shorter than its
 // reads (with the halo) and writes take (joined as cubes: neither hides the
-// other fully near the line).  Constants per kernel and precision, fitted to
-// 24 FP32 and 9 FP64 lattices (16^3 x 512 to 512^3, 2000 tiles) within 13%
-// rms near each one's best tile.
-enum TileKind { kTileHalf, kTilePassK, kTilePairK };
-struct TileCost {
-  int regs;      // per thread, for the CTAs an SM holds
-  double warp;   // us of an SM per warp and step
-  double step;   // us: least time of a step
-  double row;    // us of an SM per TMA row and step
-  double wave, cta;  // us: start of a wave, of each CTA of an SM
-  double bytes;  // bytes per us
-};
-constexpr TileCost kTileCost[3][2] = {
-    {{96, 0.060, 0.77, 0.0, 1.0, 0.010, 7.3e6}, {80, 0.40, 2.9, 0.033, 1.0, 0.012, 1.9e6}},
-    {{64, 0.0268, 0.57, 0.0029, 3.1, 0.025, 10.6e6}, {96, 0.41, 2.2, 0.031, 1.0, 0.015, 2.7e6}},
-    {{120, 0.0437, 0.59, 0.0017, 1.0, 0.098, 10.1e6}, {160, 0.67, 1.0, 0.040, 1.0, 0.012, 1.1e6}}};
-
-double tile_time(const Geometry &g, TileKind kind, const Tile &t, int sms,
+// other fully near the line).
+double tile_time(const Geometry &g, MarchKind kind, const Tile &t, int sms,
                  int64_t *full_waves = nullptr) {
   const bool f64 = g.precision == COULPS_F64;
   const TileCost &k = kTileCost[kind][f64 ? 1 : 0];
@@ -329,10 +313,10 @@ double tile_time(const Geometry &g, TileKind kind, const Tile &t, int sms,
   const int qw = g.W / 4;
   int threads, steps, planes, box_rows;
   size_t smem;
-  if (kind == kTilePairK) {
+  if (kind == kMarchPair) {
     threads = pair_threads(g, t); steps = t.dz + 6; planes = 8; box_rows = 2 * t.ty + 14;
     smem = pair_smem_bytes(g, t, true);
-  } else if (kind == kTilePassK) {
+  } else if (kind == kMarchPass) {
     threads = pass_threads(g, t); steps = t.dz + 2; planes = 4; box_rows = 2 * t.ty + 6;
     smem = pass_smem_bytes(g, t, true);
   } else {
@@ -355,7 +339,7 @@ double tile_time(const Geometry &g, TileKind kind, const Tile &t, int sms,
   const double volume = row_bytes * g.Ly * g.Lz * g.n_chains;
   const double traffic =
       row_bytes * box_rows * (double)(ny * g.n_chains) * (double)(g.Lz + nz * planes) +
-      volume * (kind == kTileHalf ? 1.0 : 2.0);
+      volume * (kind == kMarchHalf ? 1.0 : 2.0);
   const double mem = traffic / k.bytes;
   return std::cbrt(work * work * work + mem * mem * mem) + 4.0;
 }
@@ -373,16 +357,16 @@ double tile_time(const Geometry &g, TileKind kind, const Tile &t, int sms,
 // three waves, would be 2% faster alone but 672 us a sweep on two streams, where
 // 13 x 32 makes 651).  Below 2^19 FP32 sites a launch is its latency whatever the
 // tile, and most such sweeps run resident: the default shapes stay as well.
-Tile best_tile(const Geometry &g, TileKind kind, Tile t, int sms, double clear) {
+Tile best_tile(const Geometry &g, MarchKind kind, Tile t, int sms, double clear) {
   if (t.ty < 1 || t.dz < 1 || sms < 1) return t;
   if (g.precision == COULPS_F32 &&
       2 * (int64_t)g.colour_elems * g.n_chains < ((int64_t)1 << 19))
     return t;
   const int qw = g.W / 4;
-  const int threads = kind == kTilePairK
+  const int threads = kind == kMarchPair
                           ? (g.precision == COULPS_F32 ? kPairMaxThreads32 : kPairMaxThreads64)
-                          : (kind == kTilePassK ? 512 : 256);
-  const int halo = kind == kTilePairK ? 6 : (kind == kTilePassK ? 2 : 0);
+                          : (kind == kMarchPass ? 512 : 256);
+  const int halo = kind == kMarchPair ? 6 : (kind == kMarchPass ? 2 : 0);
   const int ty_max = std::min(std::min(threads / qw - halo, g.Ly), 248);
   int64_t waves = 0;
   double best = clear * tile_time(g, kind, t, sms, &waves);
@@ -400,7 +384,7 @@ Tile best_tile(const Geometry &g, TileKind kind, Tile t, int sms, double clear) 
     int last_dz = 0;
     for (int nz = 1; nz <= g.Lz; ++nz) {
       int dz = (g.Lz + nz - 1) / nz;
-      if (kind == kTileHalf) {
+      if (kind == kMarchHalf) {
         if (nz > 4) break;
         dz = 4 * nz;
       }
@@ -408,8 +392,8 @@ Tile best_tile(const Geometry &g, TileKind kind, Tile t, int sms, double clear) 
       if (dz == last_dz || dz > g.Lz) continue;
       last_dz = dz;
       const Tile c{ty, dz};
-      const size_t smem = kind == kTilePairK   ? pair_smem_bytes(g, c, true)
-                          : kind == kTilePassK ? pass_smem_bytes(g, c, true)
+      const size_t smem = kind == kMarchPair   ? pair_smem_bytes(g, c, true)
+                          : kind == kMarchPass ? pass_smem_bytes(g, c, true)
                                                : halfsweep_smem_bytes(g, c, true);
       if (smem > 227 * 1024) continue;
       const double e = tile_time(g, kind, c, sms);
@@ -1400,7 +1384,7 @@ int coulps_lattice_create(int Lx, int Ly, int Lz, int n_chains, int precision, u
   if (!L) return COULPS_ENOMEM;
   L->g = g;
   const int sms = device_sms();
-  L->tile = best_tile(g, kTileHalf, fill_grid(g, default_tile(g), 2 * sms, 4), sms,
+  L->tile = best_tile(g, kMarchHalf, fill_grid(g, default_tile(g), 2 * sms, 4), sms,
                       g.precision == COULPS_F32 ? 0.86 : 0.93);
   L->seed = seed;
   L->stream = (cudaStream_t)stream;
@@ -1460,10 +1444,10 @@ static int set_fused(coulps_lattice *L, int enable) {
   }
   const int sms = device_sms();
   if (L->ptile.ty == 0)
-    L->ptile = best_tile(L->g, kTilePassK, fill_grid(L->g, default_pass_tile(L->g), 2 * sms, 4),
+    L->ptile = best_tile(L->g, kMarchPass, fill_grid(L->g, default_pass_tile(L->g), 2 * sms, 4),
                          sms, 0.93);
   if (enable >= 3 && L->qtile.ty == 0)
-    L->qtile = best_tile(L->g, kTilePairK, fill_grid(L->g, default_pair_tile(L->g), sms, 8), sms,
+    L->qtile = best_tile(L->g, kMarchPair, fill_grid(L->g, default_pair_tile(L->g), sms, 8), sms,
                          0.93);
   L->fused = enable;
   int st = rebuild_maps(L);

@@ -97,10 +97,55 @@ constexpr int batch_quads_per_thread() {
   return (sizeof(T) == 4 && !OR && !GATHER) ? 2 : 1;
 }
 
+// The tile of the half-sweep: what only the gather after the march needs again
+// is read from the tile's and the system's records there, not kept in registers
+// through the march.
+template <typename T>
+struct BatchHalf {
+  const BatchArgs &a;
+  int it_;
+  uint32_t rng_id_, pass_;  // the system is the chain
+  const CUtensorMap *tm_halo_, *tm_own_;
+  int Lx_, Ly_, Lz_, W_, Wq_, QW_, TY_;
+  int y0_, z0_, nz_;
+  __device__ __forceinline__ BatchHalf(const BatchArgs &args, int it, uint32_t pass)
+      : a(args), it_(it), pass_(pass) {
+    const BatchItem item = a.items[it];
+    const BatchSystem &S = a.sys[item.sys];
+    rng_id_ = (uint32_t)item.sys;
+    tm_halo_ = &a.maps[2 * item.sys];
+    tm_own_ = &a.maps[2 * item.sys + 1];
+    Lx_ = S.Lx; Ly_ = S.Ly; Lz_ = S.Lz; W_ = S.W; Wq_ = S.Wq; QW_ = S.QW; TY_ = S.TY;
+    y0_ = item.y0; z0_ = item.z0; nz_ = item.nz;
+  }
+  COULPS_FIELD(const CUtensorMap *, tm_halo) COULPS_FIELD(const CUtensorMap *, tm_own)
+  COULPS_FIELD(int, Lx) COULPS_FIELD(int, Ly) COULPS_FIELD(int, Lz) COULPS_FIELD(int, W)
+  COULPS_FIELD(int, Wq) COULPS_FIELD(int, QW) COULPS_FIELD(int, TY)
+  COULPS_FIELD(int, y0) COULPS_FIELD(int, z0) COULPS_FIELD(int, nz)
+  COULPS_FIELD(uint32_t, rng_id) COULPS_FIELD(uint32_t, pass)
+  __device__ __forceinline__ int colour() const { return a.colour; }
+  __device__ __forceinline__ int map_other() const { return a.colour ^ 1; }
+  __device__ __forceinline__ int map_own() const { return a.colour; }
+  __device__ __forceinline__ T *field(int c) const {
+    const BatchSystem &S = a.sys[rng_id_];
+    return reinterpret_cast<T *>(a.field) + S.field_off + (long long)c * S.colour_elems;
+  }
+  __device__ __forceinline__ T *out() const { return field(a.colour); }
+  __device__ __forceinline__ const T *other() const { return field(a.colour ^ 1); }
+  __device__ __forceinline__ const uint32_t *g_off() const {
+    const BatchSystem &S = a.sys[rng_id_];
+    return a.g_off + S.goff_base + (size_t)(a.items[it_].y0 / S.TY) * S.Lz;
+  }
+  __device__ __forceinline__ const uint32_t *g_ent() const { return a.g_ent; }
+  __device__ __forceinline__ const double *g_q() const { return a.g_q; }
+};
+
 template <typename T, bool OR, bool GATHER, int V>
-// (two quads per thread: at most 80 registers, six CTAs of 128 threads per SM;
-// unbounded it takes 106 and a compound sweep of 256 systems 600 instead of 588 us)
-__global__ void __launch_bounds__(kBatchThreads, V == 2 ? 3 : 1)
+// (FP32, two quads per thread: at most 80 registers, six CTAs of 128 threads per
+// SM; unbounded it takes 106 and a compound sweep of 256 systems 600 instead of
+// 588 us.  One quad: at most 64, or the heatbath's gather form takes 96 and such a
+// sweep of heatbath passes only 242 instead of 234 us)
+__global__ void __launch_bounds__(kBatchThreads, sizeof(T) == 8 ? 1 : (V == 2 ? 3 : 4))
     batch_halfsweep_kernel(const BatchArgs a) {
   extern __shared__ unsigned char smem_raw[];
   unsigned char *smem = align_smem128(smem_raw);
@@ -109,30 +154,9 @@ __global__ void __launch_bounds__(kBatchThreads, V == 2 ? 3 : 1)
   int gbase = 0;
   ring_init(smem);
   for (int it; (it = next_tile(a.ctr, a.order, a.n_items)) >= 0;) {
-    const BatchItem item = a.items[it];
-    const BatchSystem S = a.sys[item.sys];
-    TileJob<T> j;
-    j.tm_halo_ = &a.maps[2 * item.sys];
-    j.tm_own_ = &a.maps[2 * item.sys + 1];
-    j.colour_ = a.colour;
-    j.map_other_ = a.colour ^ 1;
-    j.map_own_ = a.colour;
-    j.out_ = reinterpret_cast<T *>(a.field) + S.field_off + (long long)a.colour * S.colour_elems;
-    j.Lx_ = S.Lx; j.Ly_ = S.Ly; j.Lz_ = S.Lz; j.W_ = S.W; j.Wq_ = S.Wq; j.QW_ = S.QW; j.TY_ = S.TY;
-    j.y0_ = item.y0;
-    j.z0_ = item.z0;
-    j.nz_ = item.nz;
-    j.rng_id_ = (uint32_t)item.sys;
-    j.pass_ = pass;
-    if (GATHER) {
-      j.g_off_ = a.g_off + S.goff_base + (size_t)(item.y0 / S.TY) * S.Lz;
-      j.g_ent_ = a.g_ent;
-      j.other_ = reinterpret_cast<const T *>(a.field) + S.field_off +
-                (long long)(a.colour ^ 1) * S.colour_elems;
-      j.g_q_ = a.g_q;
-    }
+    const BatchHalf<T> j(a, it, pass);
     double sq = 0.0, sp = 0.0;
-    const bool ok = march_tile<T, OR, GATHER, V>(j, K, smem, a.err, gbase, sq, sp);
+    const bool ok = march_tile<T, OR, GATHER, V, kStages, 2>(j, K, smem, a.err, gbase, sq, sp);
     if (GATHER) block_partials(sq, sp, smem, a.g_partials + 2 * (size_t)it);
     if (!ok) break;
   }
@@ -329,12 +353,10 @@ int batch_row_stride(int Lx, int es) {
   return ((4 * ((Lx + 7) / 8) + a - 1) / a) * a;
 }
 
-size_t batch_smem_bytes(const coulps_batch *B, bool orx) {
+size_t batch_smem_bytes(const coulps_batch *B) {
   size_t m = 0;
-  for (const auto &S : B->sys) {
-    const SmemLayout lay = smem_layout(S.TY, S.W, B->es, orx);
-    m = std::max(m, (size_t)lay.total);
-  }
+  for (const auto &S : B->sys)
+    m = std::max(m, (size_t)smem_layout(S.TY, S.W, B->es, true).total);
   return m + 128;
 }
 
@@ -440,6 +462,159 @@ size_t batch_pair_smem_bytes(const coulps_batch *B) {
   for (const auto &S : B->sys)
     m = std::max(m, (size_t)pair_layout(S.QTY, S.W, B->es, true).total);
   return m + 128;
+}
+
+// A tiling of all systems by one rule: at most `threads` per tile (rows that
+// divide Ly evenly) and at most dz planes (slabs that divide Lz evenly;
+// half-sweeps: exactly dz, whole groups of ring waits).
+struct TileRule {
+  int threads, dz;
+};
+Tile rule_tile(const BatchSystem &S, MarchKind kind, const TileRule &r, int widest) {
+  auto even = [](int n, int most) {
+    const int k = (n + most - 1) / most;
+    return (n + k - 1) / k;
+  };
+  const int halo = kind == kMarchPair ? 6 : (kind == kMarchPass ? 2 : 0);
+  int rows = r.threads / S.QW - halo;
+  if (rows < (kind == kMarchPair ? 2 : 1)) rows = widest / S.QW - halo;  // wide rows
+  if (kind == kMarchHalf) rows = std::max(rows, std::min(4, widest / S.QW));
+  rows = std::max(1, std::min(std::min(rows, S.Ly), 248));
+  return Tile{even(S.Ly, rows), kind == kMarchHalf ? std::min(r.dz, S.Lz) : even(S.Lz, r.dz)};
+}
+
+// Time (us) of one launch of a persistent kernel over all systems' tiles: a
+// tile takes its steps times the largest of a step's latency, the issue time of
+// its and its neighbours' warps and their TMA rows, and a start (tile fetch,
+// ring fill); the CTAs share the tiles evenly, and the longest tile is the least.
+double batch_time(const coulps_batch *B, MarchKind kind, const std::vector<Tile> &tiles, int sms) {
+  const bool f64 = B->precision == COULPS_F64;
+  const TileCost &c = kTileCost[kind][f64 ? 1 : 0];
+  const int regs = f64 ? (kind == kMarchPair ? 208 : 120) : (kind == kMarchPair ? 128 : 80);
+  const double start = kind == kMarchPair ? 2.5 : (kind == kMarchPass ? 2.0 : 1.5);
+  int threads = 32;
+  size_t smem = 0;
+  double n = 0.0, steps = 0.0, warp_steps = 0.0, row_steps = 0.0;
+  auto load = [&](int s, int &warps, int &rows) {
+    const BatchSystem &S = B->sys[s];
+    const int ty = tiles[s].ty;
+    const int t = kind == kMarchPair   ? S.QW * (ty + 6)
+                  : kind == kMarchPass ? S.QW * (ty + 2)
+                                       : (f64 ? S.QW : (S.QW + 1) / 2) * ty;
+    warps = (t + 31) / 32;
+    rows = kind == kMarchPair ? 2 * ty + 14 : (kind == kMarchPass ? 2 * ty + 6 : ty + 2);
+  };
+  for (int s = 0; s < B->n_sys; ++s) {
+    const BatchSystem &S = B->sys[s];
+    int warps, rows;
+    load(s, warps, rows);
+    threads = std::max(threads, 32 * warps);
+    smem = std::max(smem, (size_t)(kind == kMarchPair   ? pair_layout(tiles[s].ty, S.W, B->es, true).total
+                                   : kind == kMarchPass ? pass_layout(tiles[s].ty, S.W, B->es, true).total
+                                                        : smem_layout(tiles[s].ty, S.W, B->es, true).total));
+    const int nz = (S.Lz + tiles[s].dz - 1) / tiles[s].dz;
+    const double m = (double)nz * ((S.Ly + tiles[s].ty - 1) / tiles[s].ty);
+    const double st = (double)(S.Lz + nz * (kind == kMarchPair ? 6 : 2)) / nz;
+    n += m;
+    steps += m * st;
+    warp_steps += m * st * warps;
+    row_steps += m * st * rows;
+  }
+  const int per_sm = std::max(
+      1, std::min(std::min(65536 / (regs * threads), 2048 / threads),
+                  std::min((int)(228 * 1024 / (smem + 1152)), 32)));
+  const double slots = (double)sms * per_sm;
+  const double others = std::max(0.0, std::min((double)per_sm, n / sms) - 1.0);
+  const double warps_av = warp_steps / steps, rows_av = row_steps / steps;
+  double sum = 0.0, longest = 0.0, mean = 0.0;
+  for (int s = 0; s < B->n_sys; ++s) {
+    const BatchSystem &S = B->sys[s];
+    int warps, rows;
+    load(s, warps, rows);
+    const double step = std::max(c.step, std::max((warps + others * warps_av) * c.warp,
+                                                  (rows + others * rows_av) * c.row));
+    const int nz = (S.Lz + tiles[s].dz - 1) / tiles[s].dz;
+    const double m = (double)nz * ((S.Ly + tiles[s].ty - 1) / tiles[s].ty);
+    const int halo = kind == kMarchPair ? 6 : 2;
+    sum += m * start + (double)(S.Lz + nz * halo) * (m / nz) * step;
+    longest = std::max(longest, (tiles[s].dz + halo) * step + start);
+  }
+  mean = sum / n;
+  return n > slots ? std::max(longest, sum / slots + 0.5 * mean) : longest;
+}
+
+// The systems' default tiles: the rule whose launch is estimated shortest, where
+// that is clearly below the estimate for the largest tiles (given).  Those leave
+// SMs idle in a batch of few systems and CTAs waiting for the last, largest tiles
+// in one of more.  Compound sweep 1:3, largest tiles against chosen ones, us: 256
+// systems of 32 .. 96 561 against 523, 64 of 32 .. 80 160 against 123, 20 of 37 .. 90
+// 177 against 68, 8 of 50 .. 90 163 against 60; FP64 64 systems 2967 (with the
+// deviates by erfcinv) against 1044.  Batches below 2^19 sites (a launch is its latency) keep the
+// largest tiles.
+void batch_choose_tiles(coulps_batch *B) {
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+    cudaGetLastError();
+    return;
+  }
+  long long sites = 0;
+  for (const auto &S : B->sys) sites += (long long)S.Lx * S.Ly * S.Lz;
+  if (sites < (1ll << 19)) return;
+  const int pair_max = batch_pair_threads(B->es);
+  static const int kThreads[3][3] = {{64, 128, 256}, {160, 192, 256}, {192, 256, 512}};
+  static const int kPlanes[3][6] = {{4, 8, 12, 16, 0, 0}, {12, 16, 24, 32, 48, 64}, {16, 24, 32, 48, 64, 127}};
+  for (int kind = kMarchHalf; kind <= kMarchPair; ++kind) {
+    std::vector<Tile> tiles(B->sys.size()), best;
+    bool given = true;
+    for (size_t s = 0; s < tiles.size(); ++s) {
+      const BatchSystem &S = B->sys[s];
+      tiles[s] = kind == kMarchPair ? Tile{S.QTY, S.QDZ}
+                                    : (kind == kMarchPass ? Tile{S.PTY, S.PDZ} : Tile{S.TY, S.DZ});
+      given = given && tiles[s].ty > 0;
+    }
+    if (!given) continue;  // a system without a pair tile: no pairs
+    const int widest = kind == kMarchPair ? pair_max : 256;
+    double clear = 0.95;
+    if (kind == kMarchHalf) {
+      // smaller than the largest tiles in any case (heatbath only, 500 systems of
+      // 40, 56: 201 -> 190 us, 100 of 64^3 86.2 -> 83.7)
+      for (size_t s = 0; s < tiles.size(); ++s)
+        best.push_back(rule_tile(B->sys[s], kMarchHalf, TileRule{128, 16}, widest));
+      tiles = best;
+      clear = 0.97;
+    }
+    double t_best = clear * batch_time(B, (MarchKind)kind, tiles, sms);
+    for (int threads : kThreads[kind])
+      for (int dz : kPlanes[kind]) {
+        if (dz == 0 || threads > widest) continue;
+        bool ok = true;
+        for (size_t s = 0; s < tiles.size() && ok; ++s) {
+          const BatchSystem &S = B->sys[s];
+          tiles[s] = rule_tile(S, (MarchKind)kind, TileRule{threads, dz}, widest);
+          ok = kind == kMarchPair   ? batch_pair_fits(S, tiles[s].ty, B->es)
+               : kind == kMarchPass ? pass_layout(tiles[s].ty, S.W, B->es, true).total + 128 <= 227 * 1024
+                                    : true;
+        }
+        if (!ok) continue;
+        const double t = batch_time(B, (MarchKind)kind, tiles, sms);
+        if (t < t_best) {
+          t_best = t;
+          best = tiles;
+        }
+      }
+    for (size_t s = 0; s < best.size(); ++s) {
+      BatchSystem &S = B->sys[s];
+      if (kind == kMarchPair) { S.QTY = best[s].ty; S.QDZ = best[s].dz; }
+      else if (kind == kMarchPass) { S.PTY = best[s].ty; S.PDZ = best[s].dz; }
+      else { S.TY = best[s].ty; S.DZ = best[s].dz; }
+    }
+  }
+  // FP64, bound by the FP64 unit: a pair's halo rows cost more than the second
+  // trip through memory (compound sweep 1:3 with pairs against fused passes: 64
+  // systems of 32 .. 80 1129 against 1044 us, 200 of 14 .. 40 529 against 457, 1000
+  // of 14 .. 33 1492 against 1270; only 8 of 50 .. 90 330 against 359).
+  if (B->precision == COULPS_F64) B->pairs_pay = false;
 }
 
 // Tile lists, tensor maps and gather lists for the current tile shapes.
@@ -574,39 +749,47 @@ int batch_layout(coulps_batch *B) {
     }
   }
   // persistent grids: as many CTAs as are co-resident at the largest smem need
-  B->smem = batch_smem_bytes(B, true);
+  B->smem = batch_smem_bytes(B);
   B->psmem = batch_pass_smem_bytes(B);
   int dev = 0, sms = 0;
   CK(cudaGetDevice(&dev));
   CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  const int per_sm = std::max(1, std::min(8, (int)((200 * 1024) / B->smem)));
-  B->grid = std::max(1, std::min((int)B->items.size(), sms * per_sm));
-  // two quads per thread: ceil(QW / 2) threads a row, the widest tile's count
-  B->threads2 = 32;
-  for (const auto &S : B->sys)
+  // half-sweeps: one quad per thread, or (FP32 heatbath without a gather) two:
+  // QW or ceil(QW / 2) threads a row, the widest tile's count
+  B->threads = B->threads2 = 32;
+  for (const auto &S : B->sys) {
+    B->threads = std::max(B->threads, S.QW * S.TY);
     B->threads2 = std::max(B->threads2, (S.QW + 1) / 2 * S.TY);
-  B->threads2 = (B->threads2 + 31) / 32 * 32;
-  {
-    int per_sm2 = 0;
-    auto hk = B->precision == COULPS_F32 ? batch_halfsweep_kernel<float, false, false, 2>
-                                         : batch_halfsweep_kernel<double, false, false, 2>;
-    if (cudaFuncSetAttribute(hk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)B->smem) !=
-            cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm2, hk, B->threads2, B->smem) !=
-            cudaSuccess ||
-        per_sm2 < 1) {
-      cudaGetLastError();
-      per_sm2 = per_sm;
-    }
-    B->grid2 = std::max(1, std::min((int)B->items.size(), sms * per_sm2));
   }
+  B->threads = (B->threads + 31) / 32 * 32;
+  B->threads2 = (B->threads2 + 31) / 32 * 32;
+  auto resident = [&](const void *k, int threads) {
+    int n = 0;
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)B->smem) !=
+            cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, threads, B->smem) != cudaSuccess ||
+        n < 1) {
+      cudaGetLastError();
+      n = 1;
+    }
+    return std::max(1, std::min((int)B->items.size(), sms * n));
+  };
+  const bool f32k = B->precision == COULPS_F32;
+  B->grid = resident(f32k ? (const void *)batch_halfsweep_kernel<float, false, true, 1>
+                          : (const void *)batch_halfsweep_kernel<double, false, true, 1>,
+                     B->threads);
+  B->grid2 = f32k ? resident((const void *)batch_halfsweep_kernel<float, false, false, 2>, B->threads2)
+                  : B->grid;
   // pass CTAs per SM: as many as registers, threads and shared memory allow
+  B->pthreads = 32;
+  for (const auto &S : B->sys) B->pthreads = std::max(B->pthreads, S.QW * (S.PTY + 2));
+  B->pthreads = (B->pthreads + 31) / 32 * 32;
   int pper_sm = 0;
   auto pk = B->precision == COULPS_F32 ? batch_pass_kernel<float, true, false>
                                        : batch_pass_kernel<double, true, false>;
   if (cudaFuncSetAttribute(pk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)B->psmem) !=
           cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pper_sm, pk, kBatchPassThreads, B->psmem) !=
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pper_sm, pk, B->pthreads, B->psmem) !=
           cudaSuccess ||
       pper_sm < 1) {
     cudaGetLastError();
@@ -663,7 +846,7 @@ cudaError_t launch_batch_t(coulps_batch *B, const BatchArgs &a) {
   if (V == 2)
     kfn<<<B->grid2, B->threads2, B->smem, B->stream>>>(a);
   else
-    kfn<<<B->grid, kBatchThreads, B->smem, B->stream>>>(a);
+    kfn<<<B->grid, B->threads, B->smem, B->stream>>>(a);
   return cudaGetLastError();
 }
 
@@ -684,7 +867,7 @@ cudaError_t launch_bpass_t(coulps_batch *B, const BatchPassArgs &a) {
     if (e != cudaSuccess) return e;
     configured = B->psmem;
   }
-  kfn<<<B->pgrid, kBatchPassThreads, B->psmem, B->stream>>>(a);
+  kfn<<<B->pgrid, B->pthreads, B->psmem, B->stream>>>(a);
   return cudaGetLastError();
 }
 
@@ -752,7 +935,7 @@ int batch_enqueue_compound(coulps_batch *B, int n_hb, int n_or, bool measure) {
       default: d = (n - 1) / 2; s = 1; break;
     }
   } else if (B->fused && B->field2) {
-    d = B->fused >= 2 ? n_or / 2 : 0;
+    d = B->fused >= 2 && B->pairs_pay ? n_or / 2 : 0;
     s = n_or - 2 * d;
     if ((d + s) % 2 == 1) {
       if (n_hb > 0) {
@@ -971,6 +1154,7 @@ int coulps_batch_create(int n_systems, const int32_t *dims, int precision, uint6
   }
   batch_reset_stats_kernel<<<(n_systems * kStatStride + 255) / 256, 256, 0, B->stream>>>(
       B->d_stats, n_systems);
+  batch_choose_tiles(B);
   int st = coulps_batch_set_fused(B, batch_pairs_ok(B) ? 2 : 1);
   if (!st) st = batch_layout(B);
   if (st) {
@@ -1040,6 +1224,7 @@ int coulps_batch_set_pair_tiles(coulps_batch_t B, const int32_t *ty_dz) {
     if (dz > 0) S.QDZ = dz;
     if (!batch_pair_fits(S, S.QTY, B->es)) return COULPS_EINVAL;
   }
+  B->pairs_pay = true;
   B->sys = next;
   B->layout_dirty = true;
   return batch_layout(B);
@@ -1102,7 +1287,7 @@ int coulps_batch_set_tiles(coulps_batch_t B, const int32_t *ty_dz) {
   }
   B->sys = next;
   B->layout_dirty = true;
-  if (batch_smem_bytes(B, true) > 227 * 1024) return COULPS_EINVAL;
+  if (batch_smem_bytes(B) > 227 * 1024) return COULPS_EINVAL;
   return batch_layout(B);
 }
 

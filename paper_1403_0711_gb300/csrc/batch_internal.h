@@ -50,6 +50,7 @@ struct coulps_batch {
   // the pass tiles, their maps [copy][system][2] and gather lists; with
   // fused = 2 also the pair tiles
   int fused = 0;
+  bool pairs_pay = true;  // mode 2 runs pairs (else fused passes only)
   void *field2 = nullptr;
   std::vector<coulps::BatchItem> pitems;
   coulps::BatchItem *d_pitems = nullptr;
@@ -72,7 +73,9 @@ struct coulps_batch {
   uint64_t pass = 0;
   int grid = 0;        // persistent CTAs
   size_t smem = 0;     // dynamic shared memory per CTA (largest system)
+  int threads = 0;               // of a half-sweep CTA
   int grid2 = 0, threads2 = 0;  // the same with two quads per thread
+  int pthreads = 0;              // of a fused-pass CTA
   bool layout_dirty = true;
   // charges and estimator
   bool has_charges = false;

@@ -85,6 +85,23 @@ struct SweepArgs {
   double *g_partials;  // [chain][y tiles * z slabs][2]
 };
 
+// March kernels' costs, for choosing tiles: fitted to 24 FP32 and 9 FP64
+// lattices (16^3 x 512 to 512^3, 2000 tiles) within 13% rms near each one's best
+// tile; the half-sweep's is the heatbath's.
+enum MarchKind { kMarchHalf, kMarchPass, kMarchPair };
+struct TileCost {
+  int regs;          // per thread, for the CTAs an SM holds
+  double warp;       // us of an SM per warp and step
+  double step;       // us: least time of a step
+  double row;        // us of an SM per TMA row and step
+  double wave, cta;  // us: start of a wave, of each CTA of an SM
+  double bytes;      // bytes per us
+};
+constexpr TileCost kTileCost[3][2] = {  // [kernel][FP64]
+    {{96, 0.060, 0.77, 0.0, 1.0, 0.010, 7.3e6}, {80, 0.40, 2.9, 0.033, 1.0, 0.012, 1.9e6}},
+    {{64, 0.0268, 0.57, 0.0029, 3.1, 0.025, 10.6e6}, {96, 0.41, 2.2, 0.031, 1.0, 0.015, 2.7e6}},
+    {{120, 0.0437, 0.59, 0.0017, 1.0, 0.098, 10.1e6}, {160, 0.67, 1.0, 0.040, 1.0, 0.012, 1.1e6}}};
+
 // Fused pass (pass_fused.cu): both half-sweeps of one pass, colour 0 then
 // colour 1, read from src and written to dst (two copies of the field, same
 // layout).  TMA maps are built on src with boxes of TY + 4 rows (colour 1)
