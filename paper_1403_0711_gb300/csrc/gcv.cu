@@ -22,6 +22,7 @@
 // 2^24 2^-k in magnitude and exact in FP32; h~ . rho is formed in FP64.  Thus
 // E[T g] = 0 holds for the h~ actually used.  The per-sample v . phi adds FP32
 // products in FP32 over 16 sites and those partial sums in FP64.
+#include <algorithm>
 #include <cmath>
 
 #include "device_common.cuh"
@@ -128,8 +129,19 @@ __global__ void gcv_c0_kernel(const double *__restrict__ partials, int nblk,
   res[0] = hr;
 }
 
-// v = A h~ (exact in FP32, see above), written in the field's per-chain
-// layout (colour-split, padded rows; padding and the x >= Lx tail stay 0)
+// Where element e of a chain's storage lies in v.  FP32 fields: within each
+// whole run of 512 elements (32 chunks of 16), the four quads of the chunk that
+// lane l sums (gcv_eval_kernel: chunk 8 (l % 4) + l / 4) lie 32 quads apart, in
+// the lanes' order, so that a warp's loads are contiguous.
+__host__ __device__ __forceinline__ size_t v_place(size_t e, size_t chain_elems, bool f32) {
+  if (!f32 || (e | 511) >= chain_elems) return e;
+  const size_t chunk = (e >> 4) & 31, lane = 4 * (chunk & 7) + (chunk >> 3);
+  return (e & ~(size_t)511) | ((e & 12) << 5) | (lane << 2) | (e & 3);
+}
+
+// v = A h~ (exact in FP32, see above), in the field's per-chain layout
+// (colour-split, padded rows; padding and the x >= Lx tail stay 0), permuted
+// by v_place
 __global__ void gcv_v_kernel(const float *__restrict__ h32, Geometry g, float *__restrict__ v) {
   const int64_t n = (int64_t)g.Lx * g.Ly * g.Lz;
   const int Lx = g.Lx, Ly = g.Ly, Lz = g.Lz;
@@ -143,104 +155,257 @@ __global__ void gcv_v_kernel(const float *__restrict__ h32, Geometry g, float *_
     const double val = 6.0 * (double)h32[i] - at(x - 1, y, z) - at(x + 1, y, z) - at(x, y - 1, z) -
                        at(x, y + 1, z) - at(x, y, z - 1) - at(x, y, z + 1);
     const int c = (x + y + z) & 1;
-    v[(size_t)c * g.colour_elems + ((size_t)z * Ly + y) * g.W + (x >> 1)] = (float)val;
+    const size_t e = (size_t)c * g.colour_elems + ((size_t)z * Ly + y) * g.W + (x >> 1);
+    v[v_place(e, g.chain_elems, g.precision == COULPS_F32)] = (float)val;
   }
 }
 
-// per (chain, block): s = v . phi over the chain's storage, Q = sum q_i phi(r_i)
+// One launch for both sums, a chain's blocks one after another in the grid: the
+// local term's charge neighbourhoods are then read while the chain is still in
+// L2 from its v . phi.
+//
+// v . phi: a lane adds the products of 16 consecutive elements in FP32, those
+// sums in FP64.  A warp loads its 512 elements in four contiguous pieces, four
+// lanes a chunk of 16 at a time, and four lanes then exchange quads so that each
+// has one chunk (a lane loading its own 64 bytes made 16 cache line accesses per
+// load, and those, not DRAM, were the time; through shared memory by bulk
+// copies 113 us, its barriers and v's latency in the way).
+//
+// Local term: a warp takes up to kEvalCharges charges of a chain, two at a time;
+// it loads the cube's sites and their neighbours once each (gcv_points: sorted
+// by row and colour, a cache line access for each such pair; seven loads per
+// point of the cube made three times as many, and these are what it spent its
+// time on), then lane t computes k(d) (A phi)(r_i + d) for points t, t + 32, ...
+// of the cube, in the field's precision, and leaves its share in shared memory;
+// then 32 / per lanes add each charge's shares in FP64 (a butterfly sum per
+// charge was six FP64-unit instructions a charge, one lane per charge 54 a warp,
+// and that unit has two lanes per clock).
+//
+// Measured, evaluation of 128^3 x 64 chains, 4096 charges (cold L2, the finish
+// kernel included): R = 1 313 -> 243 us, R = 0 144 -> 116.  v . phi is near its
+// DRAM time (77); the local term is bound by its accesses to L1.
+constexpr int kEvalTile = 4096;  // elements a block takes at a time
+constexpr int kEvalWarps = kGcvThreads / 32;
+template <typename T> constexpr int kEvalCharges = sizeof(T) == 4 ? 16 : 8;
+
+struct EvalArgs {
+  const void *field;
+  const float *v;
+  const uint32_t *idx;
+  const double *q;
+  int64_t n_q;
+  const float *kt;  // kernel values, then the points (gcv_points)
+  int R, per;       // per: charges of a warp
+  int n_pts;
+  int nblk, nblk_p;
+  double *partials, *ppart;
+};
+
+__device__ __forceinline__ float4 pick(bool c, const float4 &x, const float4 &y) {
+  return make_float4(c ? x.x : y.x, c ? x.y : y.y, c ? x.z : y.z, c ? x.w : y.w);
+}
+__device__ __forceinline__ float4 swap_lanes(const float4 &x, int mask) {
+  return make_float4(__shfl_xor_sync(0xffffffffu, x.x, mask), __shfl_xor_sync(0xffffffffu, x.y, mask),
+                     __shfl_xor_sync(0xffffffffu, x.z, mask), __shfl_xor_sync(0xffffffffu, x.w, mask));
+}
+// Four lanes' 4 x 4 quads transposed: lane l % 4 = j holds x[i] = quad j of chunk
+// i before, quads x[0 .. 3] of chunk j after.
+__device__ __forceinline__ void transpose_quads(float4 (&x)[4], int lane) {
+#pragma unroll
+  for (int b = 1; b <= 2; b *= 2) {
+    const bool up = lane & b;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      if (i & b) continue;
+      const float4 got = swap_lanes(pick(up, x[i], x[i + b]), b);
+      x[i] = pick(up, got, x[i]);
+      x[i + b] = pick(up, x[i + b], got);
+    }
+  }
+}
+
+__device__ __forceinline__ float dot16(const float4 (&w)[4], const float4 (&x)[4]) {
+  float a = 0.f;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    a = fmaf(w[j].x, x[j].x, a);
+    a = fmaf(w[j].y, x[j].y, a);
+    a = fmaf(w[j].z, x[j].z, a);
+    a = fmaf(w[j].w, x[j].w, a);
+  }
+  return a;
+}
+
 template <typename T>
-__global__ void __launch_bounds__(kGcvThreads)
-    gcv_sample_kernel(const T *__restrict__ field, size_t chain_elems,
-                      const float *__restrict__ v, const uint32_t *__restrict__ idx,
-                      const double *__restrict__ q, int64_t n_q, double *__restrict__ partials) {
-  const int chain = blockIdx.y;
-  const T *f = field + (size_t)chain * chain_elems;
+__device__ __forceinline__ void eval_dot(const Geometry &g, const EvalArgs &A, int chain) {
+  const T *f = reinterpret_cast<const T *>(A.field) + (size_t)chain * g.chain_elems;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int64_t stride = (int64_t)A.nblk * kGcvThreads;
   double s = 0.0, Q = 0.0;
-  const int64_t stride = (int64_t)gridDim.x * kGcvThreads;
-  if (sizeof(T) == 4) {
-    // 16 sites per step: four float4 of the field and of v, FP32 partial sum
-    const float4 *f4 = reinterpret_cast<const float4 *>(f);
-    const float4 *v4 = reinterpret_cast<const float4 *>(v);
-    const int64_t n16 = (int64_t)chain_elems / 16;
-    for (int64_t k = (int64_t)blockIdx.x * kGcvThreads + threadIdx.x; k < n16; k += stride) {
-      float a = 0.f;
+  if constexpr (sizeof(T) == 4) {
+    const int64_t n512 = (int64_t)g.chain_elems / 512, n16 = (int64_t)g.chain_elems / 16;
+    for (int64_t k = (int64_t)blockIdx.x * (kGcvThreads / 32) + (tid >> 5); k < n512;
+         k += (int64_t)A.nblk * (kGcvThreads / 32)) {
+      const float4 *x4 = reinterpret_cast<const float4 *>(f) + 128 * k + lane;
+      const float4 *w4 = reinterpret_cast<const float4 *>(A.v) + 128 * k + lane;
+      float4 x[4], w[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) x[j] = x4[32 * j];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) w[j] = __ldg(w4 + 32 * j);
+      transpose_quads(x, lane);
+      s += (double)dot16(w, x);
+    }
+    for (int64_t k = n512 * 32 + (int64_t)blockIdx.x * kGcvThreads + tid; k < n16; k += stride) {
+      float4 w[4], x[4];
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        const float4 x = f4[4 * k + j], w = v4[4 * k + j];
-        a = fmaf(w.x, x.x, a);
-        a = fmaf(w.y, x.y, a);
-        a = fmaf(w.z, x.z, a);
-        a = fmaf(w.w, x.w, a);
+        x[j] = reinterpret_cast<const float4 *>(f)[4 * k + j];
+        w[j] = reinterpret_cast<const float4 *>(A.v)[4 * k + j];
       }
-      s += (double)a;
+      s += (double)dot16(w, x);
     }
-    for (int64_t e = n16 * 16 + (int64_t)blockIdx.x * kGcvThreads + threadIdx.x;
-         e < (int64_t)chain_elems; e += stride)
-      s += (double)(v[e] * (float)f[e]);
+    for (int64_t e = n16 * 16 + (int64_t)blockIdx.x * kGcvThreads + tid;
+         e < (int64_t)g.chain_elems; e += stride)
+      s += (double)(A.v[e] * (float)f[e]);
   } else {
-    for (int64_t e = (int64_t)blockIdx.x * kGcvThreads + threadIdx.x; e < (int64_t)chain_elems;
+    for (int64_t e = (int64_t)blockIdx.x * kGcvThreads + tid; e < (int64_t)g.chain_elems;
          e += stride)
-      s += (double)v[e] * (double)f[e];
+      s += (double)A.v[e] * (double)f[e];
   }
-  for (int64_t i = (int64_t)blockIdx.x * kGcvThreads + threadIdx.x; i < n_q; i += stride)
-    Q += q[i] * (double)f[idx[i]];
-  block_sum2(s, Q, partials + 2 * ((size_t)chain * gridDim.x + blockIdx.x));
+  for (int64_t i = (int64_t)blockIdx.x * kGcvThreads + tid; i < A.n_q; i += stride)
+    Q += A.q[i] * (double)f[A.idx[i]];
+  block_sum2(s, Q, A.partials + 2 * ((size_t)chain * A.nblk + blockIdx.x));
 }
 
-// phi at (x, y, z) of one chain in the field layout (0 outside the box), in
-// the field's precision
+// shared memory: per warp the neighbourhoods of two charges ((m + 2)^3 each) and
+// the lanes' shares [charge][33], then the cube's points (offsets in such a
+// neighbourhood), the kernel's values and the neighbourhood's points
 template <typename T>
-__device__ __forceinline__ T phi_at(const T *f, const Geometry &g, int x, int y, int z) {
-  if (x < 0 || y < 0 || z < 0 || x >= g.Lx || y >= g.Ly || z >= g.Lz) return T(0);
-  const int c = (x + y + z) & 1;
-  return f[(size_t)c * g.colour_elems + ((size_t)z * g.Ly + y) * g.W + (x >> 1)];
+__host__ __device__ __forceinline__ size_t eval_local_bytes(int R, int n_pts) {
+  const int m = 2 * R + 1;
+  return kEvalWarps * (2 * (m + 2) * (m + 2) * (m + 2) + kEvalCharges<T> * 33) * sizeof(T) +
+         4 * (size_t)(2 * m * m * m + n_pts);
 }
 
-// warp per (charge, chain): q_i^2 phi(r_i) w_i; per block of 8 charges one
-// partial per chain.  A phi and each lane's share of w are in the field's
-// precision (FP32 fields: GB300's FP64 rate made the FP64 form several times
-// slower; any kernel k keeps the Stein term's mean 0 and FP32 rounding of w
-// adds a zero-mean error of about 1e-6 relative); lanes are added in FP64.
 template <typename T>
-__global__ void __launch_bounds__(256)
-    gcv_p_kernel(const T *__restrict__ field, const Geometry g, const uint32_t *__restrict__ idx,
-                 const double *__restrict__ q, int64_t n_q, const float *__restrict__ kt, int R,
-                 double *__restrict__ partials) {
-  const int chain = blockIdx.y;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int64_t i = (int64_t)blockIdx.x * 8 + wid;
-  const T *f = field + (size_t)chain * g.chain_elems;
-  double contrib = 0.0;
-  if (i < n_q) {
-    // site of charge i from its storage offset
-    const uint32_t e = idx[i];
-    const int c = (int)(e / g.colour_elems);
-    const uint32_t r = e - (uint32_t)c * (uint32_t)g.colour_elems;
-    const int h = (int)(r % g.W), y = (int)((r / g.W) % g.Ly), z = (int)(r / ((uint32_t)g.W * g.Ly));
-    const int x = 2 * h + ((c + y + z) & 1);
-    const int m = 2 * R + 1, m3 = m * m * m;
-    T wl = T(0);
-    for (int t = lane; t < m3; t += 32) {
-      const int dx = t % m - R, dy = (t / m) % m - R, dz = t / (m * m) - R;
-      const int xx = x + dx, yy = y + dy, zz = z + dz;
-      if (xx < 0 || yy < 0 || zz < 0 || xx >= g.Lx || yy >= g.Ly || zz >= g.Lz) continue;
-      const T Ap = T(6) * phi_at(f, g, xx, yy, zz) - phi_at(f, g, xx - 1, yy, zz) -
-                   phi_at(f, g, xx + 1, yy, zz) - phi_at(f, g, xx, yy - 1, zz) -
-                   phi_at(f, g, xx, yy + 1, zz) - phi_at(f, g, xx, yy, zz - 1) -
-                   phi_at(f, g, xx, yy, zz + 1);
-      wl += (T)kt[t] * Ap;
+__device__ __forceinline__ void eval_local(const Geometry &g, const EvalArgs &A, int chain, int pb,
+                                           unsigned char *smem) {
+  const T *f = reinterpret_cast<const T *>(A.field) + (size_t)chain * g.chain_elems;
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const int m = 2 * A.R + 1, m3 = m * m * m, d = m + 2, d3 = d * d * d;
+  T *near = reinterpret_cast<T *>(smem) + wid * (2 * d3 + kEvalCharges<T> * 33);
+  T *share = near + 2 * d3;
+  int *pt = reinterpret_cast<int *>(reinterpret_cast<T *>(smem) +
+                                    kEvalWarps * (2 * d3 + kEvalCharges<T> * 33));
+  float *kv = reinterpret_cast<float *>(pt + m3);
+  int *all = reinterpret_cast<int *>(kv + m3);
+  for (int t = tid; t < m3; t += kGcvThreads) {
+    pt[t] = (t % m + 1) + ((t / m) % m + 1) * d + (t / (m * m) + 1) * d * d;
+    kv[t] = A.kt[t];
+  }
+  for (int t = tid; t < A.n_pts; t += kGcvThreads)
+    all[t] = reinterpret_cast<const int *>(A.kt + m3)[t];
+  __syncthreads();
+  const int64_t i0 = ((int64_t)pb * kEvalWarps + wid) * A.per;
+  const int n = (int)max((int64_t)0, min((int64_t)A.per, A.n_q - i0));
+  // lane j: site of charge i0 + j from its storage offset
+  int sx = 0, sy = 0, sz = 0;
+  double qq = 0.0;
+  if (lane < n) {
+    const uint32_t e = A.idx[i0 + lane], ce = (uint32_t)g.colour_elems;
+    const int c = e >= ce ? 1 : 0;
+    const uint32_t r = e - (c ? ce : 0u), row = r / (uint32_t)g.W;
+    sz = (int)(row / (uint32_t)g.Ly);
+    sy = (int)(row - (uint32_t)sz * (uint32_t)g.Ly);
+    sx = 2 * (int)(r - row * (uint32_t)g.W) + ((c + sy + sz) & 1);
+    const double qi = A.q[i0 + lane];
+    qq = qi * qi * (double)f[e];
+  }
+  // a point of the neighbourhood (packed x, y, z offsets from its corner): phi
+  // there, 0 outside the box
+  auto phi = [&](int x, int y, int z, int o) -> T {
+    const int xx = x + (o & 255), yy = y + ((o >> 8) & 255), zz = z + (o >> 16);
+    const bool in = (unsigned)xx < (unsigned)g.Lx && (unsigned)yy < (unsigned)g.Ly &&
+                    (unsigned)zz < (unsigned)g.Lz;
+    const size_t at = ((xx + yy + zz) & 1 ? g.colour_elems : (size_t)0) +
+                      ((size_t)zz * g.Ly + yy) * g.W + (xx >> 1);
+    return in ? f[at] : T(0);
+  };
+  auto place = [&](int o) { return (o & 255) + ((o >> 8) & 255) * d + (o >> 16) * d * d; };
+  for (int j = 0; j < n; j += 2) {
+    const int k = min(j + 1, n - 1);  // (an odd last charge alone)
+    const int R1 = A.R + 1;
+    const int x0 = __shfl_sync(0xffffffffu, sx, j) - R1, x1 = __shfl_sync(0xffffffffu, sx, k) - R1;
+    const int y0 = __shfl_sync(0xffffffffu, sy, j) - R1, y1 = __shfl_sync(0xffffffffu, sy, k) - R1;
+    const int z0 = __shfl_sync(0xffffffffu, sz, j) - R1, z1 = __shfl_sync(0xffffffffu, sz, k) - R1;
+#pragma unroll 3
+    for (int t = lane; t < A.n_pts; t += 32) {
+      const int o = all[t], at = place(o);
+      const T p0 = phi(x0, y0, z0, o), p1 = k > j ? phi(x1, y1, z1, o) : T(0);
+      near[at] = p0;
+      near[d3 + at] = p1;
     }
-    const double w = warp_sum((double)wl);
-    contrib = q[i] * q[i] * (double)f[e] * w;
+    __syncwarp();
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      if (h && k == j) break;
+      const int x = (h ? x1 : x0) + 1, y = (h ? y1 : y0) + 1, z = (h ? z1 : z0) + 1;
+      T wl = T(0);
+      for (int t = lane; t < m3; t += 32) {
+        const int o = pt[t], dx = t % m, dy = (t / m) % m, dz = t / (m * m);
+        const T *c = near + (h ? d3 : 0) + o;
+        const T Ap = T(6) * c[0] - c[-1] - c[1] - c[-d] - c[d] - c[-d * d] - c[d * d];
+        if ((unsigned)(x + dx) < (unsigned)g.Lx && (unsigned)(y + dy) < (unsigned)g.Ly &&
+            (unsigned)(z + dz) < (unsigned)g.Lz)
+          wl += (T)kv[t] * Ap;
+      }
+      share[(h ? k : j) * 33 + lane] = wl;
+    }
+    __syncwarp();
   }
-  __shared__ double red[8];
+  // 32 / per lanes to a charge (per: a power of two)
+  const int each = 32 / A.per, j = lane / each;
+  double w = 0.0;
+  if (j < n)
+    for (int l = lane % each, k = min(32, m3); l < k; l += each) w += (double)share[j * 33 + l];
+  for (int o = each >> 1; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
+  double contrib = __shfl_sync(0xffffffffu, qq, j) * w;
+  if (lane % each != 0) contrib = 0.0;
+  __shared__ double red[kEvalWarps];
+  contrib = warp_sum(contrib);
   if (lane == 0) red[wid] = contrib;
   __syncthreads();
-  if (threadIdx.x == 0) {
+  if (tid == 0) {
     double sum = 0.0;
-    for (int k = 0; k < 8; ++k) sum += red[k];
-    partials[(size_t)chain * gridDim.x + blockIdx.x] = sum;
+    for (int k = 0; k < kEvalWarps; ++k) sum += red[k];
+    A.ppart[(size_t)chain * A.nblk_p + pb] = sum;
   }
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kGcvThreads, 4)
+    gcv_eval_kernel(const Geometry g, const EvalArgs A) {
+  extern __shared__ __align__(128) unsigned char smem[];
+  const int pb = (int)blockIdx.x - A.nblk;
+  if (pb < 0)
+    eval_dot<T>(g, A, blockIdx.y);
+  else
+    eval_local<T>(g, A, blockIdx.y, pb, smem);
+}
+
+template <typename T>
+cudaError_t launch_eval(const Geometry &g, const EvalArgs &A, cudaStream_t s) {
+  const size_t smem = A.nblk_p > 0 ? eval_local_bytes<T>(A.R, A.n_pts) : (size_t)0;
+  static size_t configured = 0;  // per instantiation
+  if (smem > configured) {
+    cudaError_t e = cudaFuncSetAttribute(gcv_eval_kernel<T>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    configured = smem;
+  }
+  gcv_eval_kernel<T><<<dim3(A.nblk + A.nblk_p, g.n_chains), kGcvThreads, smem, s>>>(g, A);
+  return cudaGetLastError();
 }
 
 // warp per chain: fixed-order sums, then
@@ -266,11 +431,27 @@ __global__ void gcv_finish_kernel(const double *__restrict__ partials, int nblk,
 
 }  // namespace
 
+// Sites of the cube of radius R and their neighbours, by row, then by parity of
+// x: packed offsets from the corner of the (2R + 3)^3 box.
+std::vector<int> gcv_points(int R) {
+  const int d = 2 * R + 3;
+  std::vector<int> out;
+  for (int z = 0; z < d; ++z)
+    for (int y = 0; y < d; ++y)
+      for (int parity = 0; parity < 2; ++parity)
+        for (int x = parity; x < d; x += 2) {
+          const int faces = (x == 0 || x == d - 1) + (y == 0 || y == d - 1) + (z == 0 || z == d - 1);
+          if (faces <= 1) out.push_back(x | y << 8 | z << 16);
+        }
+  return out;
+}
+
+// v . phi blocks of a chain: eight tiles each, at most 64; more where the
+// chains alone would not fill the GPU (4 blocks on each of 152 SMs)
 int gcv_blocks(const Geometry &g) {
-  // enough blocks per chain to stream the chain's storage at full bandwidth
-  const int64_t per = (int64_t)g.chain_elems / (kGcvThreads * 16);
-  int b = per < 1 ? 1 : (per > 64 ? 64 : (int)per);
-  return b;
+  const int64_t tiles = std::max<int64_t>(1, (int64_t)g.chain_elems / kEvalTile);
+  const int64_t b = std::min<int64_t>(64, (tiles + 7) / 8);
+  return (int)std::max<int64_t>(b, std::min<int64_t>(tiles, 608 / g.n_chains));
 }
 
 cudaError_t gcv_solve(const Geometry &g, int64_t n_q, const int32_t *sites, const double *q,
@@ -307,40 +488,40 @@ cudaError_t gcv_solve(const Geometry &g, int64_t n_q, const int32_t *sites, cons
   return cudaGetLastError();
 }
 
-// The local term (DRAM-latency-bound charge neighbourhoods) runs on `side`
-// beside the v . phi sums (bandwidth-bound), forked and joined by events
-// (two branches of a captured graph).
 cudaError_t gcv_eval(const Geometry &g, const void *field, const float *v_layout,
                      const uint32_t *idx, const double *q, int64_t n_q, double *partials,
                      int nblk, const double *c0, const float *kt, int R, double cP,
-                     double *ppart, double *tg, cudaStream_t s, cudaStream_t side,
-                     cudaEvent_t fork, cudaEvent_t join) {
-  const int nblk_p = R > 0 && n_q > 0 ? (int)((n_q + 7) / 8) : 0;
-  cudaError_t e;
-  if (nblk_p > 0) {
-    if ((e = cudaEventRecord(fork, s)) != cudaSuccess ||
-        (e = cudaStreamWaitEvent(side, fork, 0)) != cudaSuccess)
-      return e;
-    dim3 pgrid(nblk_p, g.n_chains);
-    if (g.precision == COULPS_F32)
-      gcv_p_kernel<float><<<pgrid, 256, 0, side>>>(reinterpret_cast<const float *>(field), g, idx,
-                                                  q, n_q, kt, R, ppart);
-    else
-      gcv_p_kernel<double><<<pgrid, 256, 0, side>>>(reinterpret_cast<const double *>(field), g,
-                                                   idx, q, n_q, kt, R, ppart);
-    if ((e = cudaGetLastError()) != cudaSuccess || (e = cudaEventRecord(join, side)) != cudaSuccess)
-      return e;
+                     double *ppart, double *tg, cudaStream_t s) {
+  EvalArgs A;
+  A.field = field;
+  A.v = v_layout;
+  A.idx = idx;
+  A.q = q;
+  A.n_q = n_q;
+  A.kt = kt;
+  A.R = R;
+  A.nblk = nblk;
+  A.partials = partials;
+  A.ppart = ppart;
+  A.nblk_p = 0;
+  A.per = 1;
+  const int m = 2 * R + 1;
+  A.n_pts = m * m * (m + 6);
+  if (R > 0 && n_q > 0) {
+    // as many charges a warp as leave 32 warps for each of 152 SMs (evaluation of
+    // 128^3 x 4 chains, 4096 charges, 16 / 32 / 64 warps: 39.6 / 37.5 / 47.7 us; 40^3 x
+    // 64, 500 charges 39.6 / 43.7 / 47.7)
+    const int most = g.precision == COULPS_F32 ? kEvalCharges<float> : kEvalCharges<double>;
+    while (2 * A.per <= most && n_q * g.n_chains / (2 * A.per) >= 32 * 152) A.per *= 2;
+    const int per_block = A.per * (kGcvThreads / 32);
+    A.nblk_p = (int)((n_q + per_block - 1) / per_block);
   }
-  dim3 grid(nblk, g.n_chains);
-  if (g.precision == COULPS_F32)
-    gcv_sample_kernel<float><<<grid, kGcvThreads, 0, s>>>(
-        reinterpret_cast<const float *>(field), g.chain_elems, v_layout, idx, q, n_q, partials);
-  else
-    gcv_sample_kernel<double><<<grid, kGcvThreads, 0, s>>>(
-        reinterpret_cast<const double *>(field), g.chain_elems, v_layout, idx, q, n_q, partials);
-  if (nblk_p > 0 && (e = cudaStreamWaitEvent(s, join, 0)) != cudaSuccess) return e;
-  gcv_finish_kernel<<<(g.n_chains + 7) / 8, 256, 0, s>>>(partials, nblk, ppart, nblk_p,
-                                                        g.n_chains, c0, nblk_p > 0 ? cP : 0.0, tg);
+  const cudaError_t e = g.precision == COULPS_F32 ? launch_eval<float>(g, A, s)
+                                                  : launch_eval<double>(g, A, s);
+  if (e != cudaSuccess) return e;
+  gcv_finish_kernel<<<(g.n_chains + 7) / 8, 256, 0, s>>>(partials, nblk, ppart, A.nblk_p,
+                                                        g.n_chains, c0, A.nblk_p > 0 ? cP : 0.0,
+                                                        tg);
   return cudaGetLastError();
 }
 

@@ -222,7 +222,7 @@ struct Allocator;
 // Global control variate (gcv.cu).  gcv_solve: red/black SOR on A u = -rho for
 // the n_q charges (host sites and values; u and rho are left in u_nat and
 // rho_nat, natural order, Lx*Ly*Lz doubles), h32 = u rounded to a fixed-point grid (exact FP32), v_layout = A h32 (exact in FP32) in one
-// chain's field layout (chain_elems floats), res[0] = h32 . rho,
+// chain's field layout (chain_elems floats, permuted as gcv_eval reads it), res[0] = h32 . rho,
 // res[1] = |A u + rho| / |rho|, res[2] = max |u| (res: 3 doubles); scratch
 // >= 4 * nblk_red doubles; synchronises.  gcv_eval: per chain
 // T g = res[0] - Q (v . phi) into tg; partials >= 2 * nblk * n_chains
@@ -236,13 +236,13 @@ cudaError_t gcv_solve(const Geometry &g, int64_t n_q, const int32_t *sites, cons
                       double *scratch, int nblk_red, int n_iter, double *res,
                       const Allocator &alloc, cudaStream_t s);
 // With R > 0 also the local term of P (kt: (2R+1)^3 floats, index
-// (dz + R)(2R+1)^2 + (dy + R)(2R+1) + dx + R; cP = kt[centre] sum q^2; ppart
+// (dz + R)(2R+1)^2 + (dy + R)(2R+1) + dx + R, then gcv_points(R); cP = kt[centre] sum q^2; ppart
 // >= ceil(n_q / 8) * n_chains doubles).
+std::vector<int> gcv_points(int R);
 cudaError_t gcv_eval(const Geometry &g, const void *field, const float *v_layout,
                      const uint32_t *idx, const double *q, int64_t n_q, double *partials,
                      int nblk, const double *c0, const float *kt, int R, double cP,
-                     double *ppart, double *tg, cudaStream_t s, cudaStream_t side,
-                     cudaEvent_t fork, cudaEvent_t join);
+                     double *ppart, double *tg, cudaStream_t s);
 
 // Entry packing of the fused gather.
 constexpr uint32_t kGatherColourBit = 0x80000000u;

@@ -109,3 +109,50 @@ def test_single_sweep_launches(cl, L, chains, prec):
         c.close()
         lat.close()
     _same(*out)
+
+
+@pytest.mark.parametrize("L,chains,prec,n,R", [
+    ((23, 18, 15), 3, "F32", 30, 1),     # whole runs of 512 elements and a rest
+    ((16, 16, 16), 40, "F32", 700, 2),   # several charges a warp, an odd count
+    ((5, 4, 3), 2, "F32", 4, 4),         # a cube larger than the box
+    ((40, 33, 20), 90, "F32", 801, 1),
+    ((23, 18, 15), 40, "F64", 301, 1),
+    ((9, 8, 7), 1, "F64", 5, 0),
+])
+def test_control_variate_sums(cl, L, chains, prec, n, R):
+    """T g of the first and last chain against a direct evaluation in FP64 from
+    the field and h.  Bound: FP32 fields round each product and each cube point's
+    seven terms, |error| <= 32 * 2^-24 * (sum of magnitudes); FP64 fields 1e-12."""
+    import torch
+    from oracle import stein as ost
+    from paper_1403_0711_gb300 import inputs
+    sites, q = inputs.uniform_q(L, n, seed=6)
+    lat = cl.Lattice(L, n_chains=chains, precision=getattr(cl, prec), seed=2,
+                     stream=torch.cuda.Stream())
+    lat.sweep(4, 1, 2)
+    c = cl.Charges(lat, sites, q)
+    g = cl.GlobalCV(c, n_iter=60, R=R)
+    tg = torch.zeros(chains, dtype=torch.float64, device="cuda")
+    g.eval(tg.data_ptr())
+    lat.sync()
+    h = g.h().astype(np.float64)
+    v = ost.apply_A(h)
+    k = ost.cube_green(R).astype(np.float32).astype(np.float64) if R > 0 else None
+    rho = np.zeros(L[::-1])
+    for (x, y, z), qi in zip(np.asarray(sites), q):
+        rho[z, y, x] += qi
+    eps = 32 * 2.0 ** -24 if prec == "F32" else 1e-12
+    for ch in {0, chains - 1}:
+        phi = np.asarray(lat.field(ch), dtype=np.float64)
+        Q = float(np.sum(rho * phi))
+        ref = g.info()["h_dot_rho"] - Q * float(np.sum(v * phi))
+        scale = abs(g.info()["h_dot_rho"]) + abs(Q) * float(np.sum(np.abs(v * phi)))
+        if R > 0:
+            ref += ost.local_p_stein_term(phi, sites, q, k)
+            amax = float(np.abs(phi).max())
+            scale += 12 * amax * float(np.abs(k).sum()) * float(
+                sum(qi * qi * abs(phi[z, y, x]) for (x, y, z), qi in zip(np.asarray(sites), q)))
+        assert abs(float(tg[ch]) - ref) <= eps * scale, (ch, float(tg[ch]), ref, scale)
+    g.close()
+    c.close()
+    lat.close()
