@@ -53,7 +53,7 @@ PROFILE_TRAFFIC = {
     "halfsweep_kernel<float, heatbath>": ROOT / "profiles" / "heatbath_halfsweep_128c_64ch.txt",
 }
 KERNEL_SOURCES = ["sweep.cu", "pass_fused.cu", "pass_pair.cu", "tile_march.cuh", "pass_march.cuh",
-                  "pair_march.cuh",
+                  "pair_march.cuh", "march_quad.cuh",
                   "device_common.cuh", "internal.h"]
 FUSED_MODES = {"off": 0, "on": 1, "all": 2, "pairs": 3, "allpairs": 4}
 

@@ -229,14 +229,12 @@ int rebuild_maps(coulps_lattice *L) {
 }
 
 // Fused-pass tile: rows + 2 halo rows of quads per CTA within 256 threads,
-// an odd row count (measured a little faster at 128^3: 13 rows 0.202 ms, 14
-// rows 0.211 ms per pass of 64 chains); z slabs of 32 planes (several CTAs
-// per column fill the GPU's slots evenly).  Rows of more than 42 quads leave
-// fewer than 5 rows in 256 threads, and the 4 halo rows of colour 1 are then
-// re-read for every row or two: such rows take up to 512 threads (measured,
-// one chain: 512^3 0.321 ms per pass with 1 row, 0.221 with 3, 0.183 with 5;
-// 384^3 0.104 with 7 rows; at 256^3 the 256-thread 5 rows are faster than 9
-// or 13 rows: 0.039, 0.041, 0.049 ms).
+// an odd row count; z slabs of 32 planes (several CTAs per column fill the
+// GPU's slots evenly).  Rows of more than 42 quads leave fewer than 5 rows in
+// 256 threads, and the 4 halo rows of colour 1 are then re-read for every row
+// or two: such rows take up to 512 threads (measured, one chain: 512^3 181 us
+// per pass with 4 rows, 173 with 5; 384^3 78 with 7).  best_tile starts from
+// this shape.
 Tile default_pass_tile(const Geometry &g) {
   const int qw = g.W / 4;
   int ty = 256 / qw - 2;
@@ -259,8 +257,8 @@ Tile default_pass_tile(const Geometry &g) {
 // the FP64 unit is the bound there, and a pair's halo rows and planes cost it
 // more than the second trip through memory costs two fused passes (best tiles of each: 128^3 x 8 chains 685 us against 2 x 260, 96^3 x 8
 // 297 against 2 x 115, 64^3 x 4 65 against 2 x 29).  z slabs of
-// 64 planes from Lz = 128 (measured at 128^3 x 64 chains, two streams: 0.802
-// ms per 1 HB : 3 OR compound sweep against 0.828 with 32 planes).
+// 64 planes from Lz = 128 (measured at 128^3 x 64 chains, two streams: 672 us
+// per 1 HB : 3 OR compound sweep against 677 with 32 planes).
 Tile default_pair_tile(const Geometry &g) {
   if (g.precision == COULPS_F64) return Tile{0, 0};
   const int qw = g.W / 4;

@@ -17,8 +17,8 @@ namespace tile {
 
 // Ring depth of the fused pass (slots of one colour-1 box and one colour-0
 // box); at most 8 (mbarriers at 0 .. 63 of the header, abort flag at 64).
-// Measured at 128^3 x 64 chains: 0.203 ms per over-relaxation pass with 4
-// slots, 0.194 with 6, 0.196 with 8.
+// Measured per over-relaxation pass, 128^3 x 64 chains / 512^3: 204 / 204 us with
+// 4 slots, 183 / 175 with 6, 179 / 227 with 8 (a CTA less per SM).
 constexpr int kPassStages = 6;
 static_assert(kPassStages <= 8, "mbarriers must end before the abort flag");
 
