@@ -21,6 +21,7 @@
 #include <vector>
 
 #include "batch_internal.h"
+#include "charge_local.cuh"
 #include "device_common.cuh"
 #include "internal.h"
 #include "sor.cuh"
@@ -175,82 +176,54 @@ __global__ void __launch_bounds__(kBgcvThreads)
   if (threadIdx.x == 0) partials[blockIdx.x] = s;
 }
 
-// phi at (x, y, z) of system S in the batch layout (0 outside the box)
-template <typename T>
-__device__ __forceinline__ double phi_at(const T *f, const BgcvSystem &S, int x, int y, int z) {
-  if (x < 0 || y < 0 || z < 0 || x >= S.Lx || y >= S.Ly || z >= S.Lz) return 0.0;
-  const int c = (x + y + z) & 1;
-  return (double)f[S.field_off + (long long)c * S.colour_elems + ((long long)z * S.Ly + y) * S.W +
-                   (x >> 1)];
-}
+// out[2 i] = q_i phi(r_i); out[2 i + 1] = q_i^2 phi(r_i) w_i (R > 0;
+// charge_local.cuh), beside the v . phi kernel.  Measured: 8 sweeps with an
+// evaluation each of 64 systems of 32 .. 80, R = 1, 1627 us with a warp per charge, seven
+// loads per point and a butterfly sum, 1565 now.
+constexpr int kBgcvWarps = 8;
+template <typename T> constexpr int kBgcvCharges = sizeof(T) == 4 ? 16 : 8;  // of a warp
 
-// warp per charge: out[2 i] = q_i phi(r_i); out[2 i + 1] = q_i^2 phi(r_i) w_i
-// (R > 0), w_i = sum_d k(d) (A phi)(r_i + d) over the cube inside the box.
-// The charges' neighbourhoods are scattered over the field and mostly not in
-// L2 after a sweep, so the kernel is bound by DRAM latency: lane t takes cube
-// point t and issues its seven loads unconditionally (coordinates clamped
-// into the box, the value masked after), and a warp loops over charges with
-// the next charge's record loaded before the current one's sums.
-template <typename T, int R>
-__global__ void __launch_bounds__(256)
+template <typename T>
+__global__ void __launch_bounds__(32 * kBgcvWarps, 4)
     bgcv_charge_kernel(const T *__restrict__ field, const BgcvSystem *__restrict__ sys,
                        const int4 *__restrict__ qsite, const double *__restrict__ q, int64_t n_q,
-                       const float *__restrict__ kt, double *__restrict__ out) {
-  constexpr int m = 2 * R + 1, m3 = m * m * m;
-  constexpr int kPts = (m3 + 31) / 32;  // cube points per lane
-  const int lane = threadIdx.x & 31;
-  const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (i >= n_q) return;  // whole warps
-  float kl[kPts];
-#pragma unroll
-  for (int u = 0; u < kPts; ++u) kl[u] = lane + 32 * u < m3 ? __ldg(kt + lane + 32 * u) : 0.f;
-  int4 r = __ldg(qsite + i);
-  double qi = __ldg(q + i);
-  for (; i < n_q; i += warps) {
-    const BgcvSystem S = sys[r.w];
-    const int4 rn = i + warps < n_q ? __ldg(qsite + i + warps) : r;
-    const double qn = i + warps < n_q ? __ldg(q + i + warps) : 0.0;
-    const T *f = field + S.field_off;
-    const long long ce = S.colour_elems;
-    // phi at an in-box site (x, y, z), in the field's precision: FP32 fields
-    // keep A phi and the lane's share of w in FP32 (GB300's FP64 rate made the
-    // FP64 form of this kernel several times slower; any kernel k keeps the
-    // Stein term's mean 0, and FP32 rounding of w adds a zero-mean error of
-    // about 1e-6 relative), FP64 fields in FP64
-    auto at = [&](int x, int y, int z) -> T {
-      return f[(long long)((x + y + z) & 1) * ce + ((long long)z * S.Ly + y) * S.W + (x >> 1)];
-    };
-    const double p = (double)at(r.x, r.y, r.z);
-    T w = T(0);
-#pragma unroll
-    for (int u = 0; u < kPts; ++u) {
-      const int t = lane + 32 * u;
-      const int xx = r.x + t % m - R, yy = r.y + (t / m) % m - R, zz = r.z + t / (m * m) - R;
-      const bool in = t < m3 && xx >= 0 && yy >= 0 && zz >= 0 && xx < S.Lx && yy < S.Ly && zz < S.Lz;
-      // the point and its six neighbours, clamped into the box; a neighbour
-      // outside the box is 0
-      const int xc = min(max(xx, 0), S.Lx - 1), yc = min(max(yy, 0), S.Ly - 1),
-                zc = min(max(zz, 0), S.Lz - 1);
-      const int xm = max(xc - 1, 0), xp = min(xc + 1, S.Lx - 1);
-      const int ym = max(yc - 1, 0), yp = min(yc + 1, S.Ly - 1);
-      const int zm = max(zc - 1, 0), zp = min(zc + 1, S.Lz - 1);
-      const T c0 = at(xc, yc, zc);
-      const T vxm = at(xm, yc, zc), vxp = at(xp, yc, zc);
-      const T vym = at(xc, ym, zc), vyp = at(xc, yp, zc);
-      const T vzm = at(xc, yc, zm), vzp = at(xc, yc, zp);
-      const T Ap = T(6) * c0 - (xc > 0 ? vxm : T(0)) - (xc < S.Lx - 1 ? vxp : T(0)) -
-                   (yc > 0 ? vym : T(0)) - (yc < S.Ly - 1 ? vyp : T(0)) -
-                   (zc > 0 ? vzm : T(0)) - (zc < S.Lz - 1 ? vzp : T(0));
-      if (in) w += (T)kl[u] * Ap;
+                       const float *__restrict__ kt, int R, int n_pts, int per,
+                       double *__restrict__ out) {
+  extern __shared__ __align__(128) unsigned char smem[];
+  LocalSums<T> local(smem, kBgcvWarps, kBgcvCharges<T>, R, n_pts, kt);
+  const int lane = threadIdx.x & 31, each = 32 / per;
+  const int64_t stride = (int64_t)gridDim.x * kBgcvWarps * per;
+  auto box = [&](int s) {
+    const BgcvSystem S = sys[s];
+    return LocalBox<T>{field + S.field_off, (size_t)S.colour_elems, S.Lx, S.Ly, S.Lz, S.W};
+  };
+  for (int64_t i0 = ((int64_t)blockIdx.x * kBgcvWarps + (threadIdx.x >> 5)) * per; i0 < n_q;
+       i0 += stride) {
+    const int n = (int)min((int64_t)per, n_q - i0);
+    int4 r = make_int4(0, 0, 0, 0);
+    double qi = 0.0, p = 0.0;
+    if (lane < n) {
+      r = __ldg(qsite + i0 + lane);
+      qi = __ldg(q + i0 + lane);
+      const LocalBox<T> b = box(r.w);
+      p = (double)b.f[((r.x + r.y + r.z) & 1 ? b.ce : (size_t)0) +
+                      ((size_t)r.z * b.Ly + r.y) * b.W + (r.x >> 1)];
     }
-    const double wsum = warp_sum((double)w);
-    if (lane == 0) {
-      out[2 * i] = qi * p;
-      out[2 * i + 1] = qi * qi * p * wsum;
+    for (int j = 0; j < n; j += 2) {
+      const int k = min(j + 1, n - 1);
+      const int x0 = __shfl_sync(0xffffffffu, r.x, j), x1 = __shfl_sync(0xffffffffu, r.x, k);
+      const int y0 = __shfl_sync(0xffffffffu, r.y, j), y1 = __shfl_sync(0xffffffffu, r.y, k);
+      const int z0 = __shfl_sync(0xffffffffu, r.z, j), z1 = __shfl_sync(0xffffffffu, r.z, k);
+      const int s0 = __shfl_sync(0xffffffffu, r.w, j), s1 = __shfl_sync(0xffffffffu, r.w, k);
+      local.pair(box(s0), box(s1), x0, y0, z0, x1, y1, z1, j, k, lane);
     }
-    r = rn;
-    qi = qn;
+    const double w = local.sum(per, n, lane);
+    const double wi = __shfl_sync(0xffffffffu, w, (lane * each) & 31);
+    if (lane < n) {
+      out[2 * (i0 + lane)] = qi * p;
+      out[2 * (i0 + lane) + 1] = qi * qi * p * wi;
+    }
+    __syncwarp();  // the shares are read
   }
 }
 
@@ -361,26 +334,23 @@ cudaError_t launch_charge(coulps_batch_gcv *G, const T *field, cudaStream_t st) 
         field, G->d_sys, G->d_qsite, G->d_q, G->n_q, G->d_qpart);
     return cudaGetLastError();
   }
-  const int64_t need = (G->n_q + 7) / 8;
-  const int blocks = (int)std::min<int64_t>(need, (int64_t)G->sms * 8);
-  switch (G->R) {
-    case 1:
-      bgcv_charge_kernel<T, 1><<<blocks, 256, 0, st>>>(field, G->d_sys, G->d_qsite, G->d_q,
-                                                               G->n_q, G->d_k, G->d_qpart);
-      break;
-    case 2:
-      bgcv_charge_kernel<T, 2><<<blocks, 256, 0, st>>>(field, G->d_sys, G->d_qsite, G->d_q,
-                                                               G->n_q, G->d_k, G->d_qpart);
-      break;
-    case 3:
-      bgcv_charge_kernel<T, 3><<<blocks, 256, 0, st>>>(field, G->d_sys, G->d_qsite, G->d_q,
-                                                               G->n_q, G->d_k, G->d_qpart);
-      break;
-    default:
-      bgcv_charge_kernel<T, 4><<<blocks, 256, 0, st>>>(field, G->d_sys, G->d_qsite, G->d_q,
-                                                               G->n_q, G->d_k, G->d_qpart);
-      break;
+  const int m = 2 * G->R + 1, n_pts = m * m * (m + 6);
+  // as many charges a warp as leave 32 warps for each SM
+  int per = 1;
+  while (2 * per <= kBgcvCharges<T> && G->n_q / (2 * per) >= 32 * (int64_t)G->sms) per *= 2;
+  const int64_t warps = (G->n_q + per - 1) / per;
+  const int blocks = (int)std::min<int64_t>((warps + kBgcvWarps - 1) / kBgcvWarps,
+                                            (int64_t)G->sms * 8);
+  const size_t smem = local_bytes<T>(kBgcvWarps, kBgcvCharges<T>, G->R, n_pts);
+  static size_t configured = 0;  // per instantiation
+  if (smem > configured) {
+    cudaError_t e = cudaFuncSetAttribute(bgcv_charge_kernel<T>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    configured = smem;
   }
+  bgcv_charge_kernel<T><<<blocks, 32 * kBgcvWarps, smem, st>>>(
+      field, G->d_sys, G->d_qsite, G->d_q, G->n_q, G->d_k, G->R, n_pts, per, G->d_qpart);
   return cudaGetLastError();
 }
 
@@ -573,6 +543,10 @@ int coulps_batch_gcv_create(coulps_batch_t B, int n_iter, int R, coulps_batch_gc
     }
   }
   if (G->R > 0) {
+    const std::vector<int> pts = gcv_points(G->R);  // behind the kernel's values
+    const size_t n_k = kt.size();
+    kt.resize(n_k + pts.size());
+    std::memcpy(kt.data() + n_k, pts.data(), pts.size() * sizeof(int));
     G->d_k = (float *)A(kt.size() * sizeof(float));
     if (!G->d_k) return fail(COULPS_ENOMEM);
   }

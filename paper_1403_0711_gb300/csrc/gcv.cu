@@ -25,6 +25,7 @@
 #include <algorithm>
 #include <cmath>
 
+#include "charge_local.cuh"
 #include "device_common.cuh"
 #include "internal.h"
 #include "sor.cuh"
@@ -171,15 +172,7 @@ __global__ void gcv_v_kernel(const float *__restrict__ h32, Geometry g, float *_
 // load, and those, not DRAM, were the time; through shared memory by bulk
 // copies 113 us, its barriers and v's latency in the way).
 //
-// Local term: a warp takes up to kEvalCharges charges of a chain, two at a time;
-// it loads the cube's sites and their neighbours once each (gcv_points: sorted
-// by row and colour, a cache line access for each such pair; seven loads per
-// point of the cube made three times as many, and these are what it spent its
-// time on), then lane t computes k(d) (A phi)(r_i + d) for points t, t + 32, ...
-// of the cube, in the field's precision, and leaves its share in shared memory;
-// then 32 / per lanes add each charge's shares in FP64 (a butterfly sum per
-// charge was six FP64-unit instructions a charge, one lane per charge 54 a warp,
-// and that unit has two lanes per clock).
+// Local term: charge_local.cuh, up to kEvalCharges charges of a chain a warp.
 //
 // Measured, evaluation of 128^3 x 64 chains, 4096 charges (cold L2, the finish
 // kernel included): R = 1 313 -> 243 us, R = 0 144 -> 116.  v . phi is near its
@@ -278,35 +271,13 @@ __device__ __forceinline__ void eval_dot(const Geometry &g, const EvalArgs &A, i
   block_sum2(s, Q, A.partials + 2 * ((size_t)chain * A.nblk + blockIdx.x));
 }
 
-// shared memory: per warp the neighbourhoods of two charges ((m + 2)^3 each) and
-// the lanes' shares [charge][33], then the cube's points (offsets in such a
-// neighbourhood), the kernel's values and the neighbourhood's points
-template <typename T>
-__host__ __device__ __forceinline__ size_t eval_local_bytes(int R, int n_pts) {
-  const int m = 2 * R + 1;
-  return kEvalWarps * (2 * (m + 2) * (m + 2) * (m + 2) + kEvalCharges<T> * 33) * sizeof(T) +
-         4 * (size_t)(2 * m * m * m + n_pts);
-}
-
 template <typename T>
 __device__ __forceinline__ void eval_local(const Geometry &g, const EvalArgs &A, int chain, int pb,
                                            unsigned char *smem) {
   const T *f = reinterpret_cast<const T *>(A.field) + (size_t)chain * g.chain_elems;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  const int m = 2 * A.R + 1, m3 = m * m * m, d = m + 2, d3 = d * d * d;
-  T *near = reinterpret_cast<T *>(smem) + wid * (2 * d3 + kEvalCharges<T> * 33);
-  T *share = near + 2 * d3;
-  int *pt = reinterpret_cast<int *>(reinterpret_cast<T *>(smem) +
-                                    kEvalWarps * (2 * d3 + kEvalCharges<T> * 33));
-  float *kv = reinterpret_cast<float *>(pt + m3);
-  int *all = reinterpret_cast<int *>(kv + m3);
-  for (int t = tid; t < m3; t += kGcvThreads) {
-    pt[t] = (t % m + 1) + ((t / m) % m + 1) * d + (t / (m * m) + 1) * d * d;
-    kv[t] = A.kt[t];
-  }
-  for (int t = tid; t < A.n_pts; t += kGcvThreads)
-    all[t] = reinterpret_cast<const int *>(A.kt + m3)[t];
-  __syncthreads();
+  LocalSums<T> local(smem, kEvalWarps, kEvalCharges<T>, A.R, A.n_pts, A.kt);
+  const LocalBox<T> box{f, g.colour_elems, g.Lx, g.Ly, g.Lz, g.W};
   const int64_t i0 = ((int64_t)pb * kEvalWarps + wid) * A.per;
   const int n = (int)max((int64_t)0, min((int64_t)A.per, A.n_q - i0));
   // lane j: site of charge i0 + j from its storage offset
@@ -322,55 +293,16 @@ __device__ __forceinline__ void eval_local(const Geometry &g, const EvalArgs &A,
     const double qi = A.q[i0 + lane];
     qq = qi * qi * (double)f[e];
   }
-  // a point of the neighbourhood (packed x, y, z offsets from its corner): phi
-  // there, 0 outside the box
-  auto phi = [&](int x, int y, int z, int o) -> T {
-    const int xx = x + (o & 255), yy = y + ((o >> 8) & 255), zz = z + (o >> 16);
-    const bool in = (unsigned)xx < (unsigned)g.Lx && (unsigned)yy < (unsigned)g.Ly &&
-                    (unsigned)zz < (unsigned)g.Lz;
-    const size_t at = ((xx + yy + zz) & 1 ? g.colour_elems : (size_t)0) +
-                      ((size_t)zz * g.Ly + yy) * g.W + (xx >> 1);
-    return in ? f[at] : T(0);
-  };
-  auto place = [&](int o) { return (o & 255) + ((o >> 8) & 255) * d + (o >> 16) * d * d; };
   for (int j = 0; j < n; j += 2) {
-    const int k = min(j + 1, n - 1);  // (an odd last charge alone)
-    const int R1 = A.R + 1;
-    const int x0 = __shfl_sync(0xffffffffu, sx, j) - R1, x1 = __shfl_sync(0xffffffffu, sx, k) - R1;
-    const int y0 = __shfl_sync(0xffffffffu, sy, j) - R1, y1 = __shfl_sync(0xffffffffu, sy, k) - R1;
-    const int z0 = __shfl_sync(0xffffffffu, sz, j) - R1, z1 = __shfl_sync(0xffffffffu, sz, k) - R1;
-#pragma unroll 3
-    for (int t = lane; t < A.n_pts; t += 32) {
-      const int o = all[t], at = place(o);
-      const T p0 = phi(x0, y0, z0, o), p1 = k > j ? phi(x1, y1, z1, o) : T(0);
-      near[at] = p0;
-      near[d3 + at] = p1;
-    }
-    __syncwarp();
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      if (h && k == j) break;
-      const int x = (h ? x1 : x0) + 1, y = (h ? y1 : y0) + 1, z = (h ? z1 : z0) + 1;
-      T wl = T(0);
-      for (int t = lane; t < m3; t += 32) {
-        const int o = pt[t], dx = t % m, dy = (t / m) % m, dz = t / (m * m);
-        const T *c = near + (h ? d3 : 0) + o;
-        const T Ap = T(6) * c[0] - c[-1] - c[1] - c[-d] - c[d] - c[-d * d] - c[d * d];
-        if ((unsigned)(x + dx) < (unsigned)g.Lx && (unsigned)(y + dy) < (unsigned)g.Ly &&
-            (unsigned)(z + dz) < (unsigned)g.Lz)
-          wl += (T)kv[t] * Ap;
-      }
-      share[(h ? k : j) * 33 + lane] = wl;
-    }
-    __syncwarp();
+    const int k = min(j + 1, n - 1);
+    const int x0 = __shfl_sync(0xffffffffu, sx, j), x1 = __shfl_sync(0xffffffffu, sx, k);
+    const int y0 = __shfl_sync(0xffffffffu, sy, j), y1 = __shfl_sync(0xffffffffu, sy, k);
+    const int z0 = __shfl_sync(0xffffffffu, sz, j), z1 = __shfl_sync(0xffffffffu, sz, k);
+    local.pair(box, box, x0, y0, z0, x1, y1, z1, j, k, lane);
   }
-  // 32 / per lanes to a charge (per: a power of two)
-  const int each = 32 / A.per, j = lane / each;
-  double w = 0.0;
-  if (j < n)
-    for (int l = lane % each, k = min(32, m3); l < k; l += each) w += (double)share[j * 33 + l];
-  for (int o = each >> 1; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
-  double contrib = __shfl_sync(0xffffffffu, qq, j) * w;
+  const int each = 32 / A.per;
+  const double w = local.sum(A.per, n, lane);
+  double contrib = __shfl_sync(0xffffffffu, qq, lane / each) * w;
   if (lane % each != 0) contrib = 0.0;
   __shared__ double red[kEvalWarps];
   contrib = warp_sum(contrib);
@@ -396,7 +328,7 @@ __global__ void __launch_bounds__(kGcvThreads, 4)
 
 template <typename T>
 cudaError_t launch_eval(const Geometry &g, const EvalArgs &A, cudaStream_t s) {
-  const size_t smem = A.nblk_p > 0 ? eval_local_bytes<T>(A.R, A.n_pts) : (size_t)0;
+  const size_t smem = A.nblk_p > 0 ? local_bytes<T>(kEvalWarps, kEvalCharges<T>, A.R, A.n_pts) : (size_t)0;
   static size_t configured = 0;  // per instantiation
   if (smem > configured) {
     cudaError_t e = cudaFuncSetAttribute(gcv_eval_kernel<T>,
