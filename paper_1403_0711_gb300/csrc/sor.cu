@@ -40,11 +40,14 @@ __global__ void __launch_bounds__(kSorThreads)
   const int t = it.first + (int)threadIdx.x;
   const int y = t / b.Wh, h = t - y * b.Wh;
   const int par = (colour + y + it.z) & 1;
-  if (t >= b.Ly * b.Wh || 2 * h + par >= b.Lx) return;
   const long long at = b.off + (long long)colour * b.colour + (it.z + 1) * plane +
                        (long long)(y + 1) * b.Ws + h;
   const double *o = u + at + (colour ? -b.colour : b.colour);
+  // every thread waits, also those without a site: a grid without a waiting
+  // thread (colour 1 of boxes of one site) would end before the grid ahead of
+  // it, and the grid behind it would then run beside that one
   asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (t >= b.Ly * b.Wh || 2 * h + par >= b.Lx) return;
   const double zm = o[-plane], zp = o[plane], ym = o[-b.Ws], yp = o[b.Ws], c = o[0],
                e = o[par ? 1 : -1], w = u[at], q = r[at];
   const double S = ((zm + zp) + (ym + yp)) + (c + e);

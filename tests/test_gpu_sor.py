@@ -53,3 +53,24 @@ def test_iterates(L, n_iter):
     assert np.array_equal(g.h(), gb.h(1))
     for o in (g, gb, ch, b, lat):
         o.close()
+
+
+@pytest.mark.parametrize("systems", [1, 3, 300])
+def test_boxes_of_one_site(systems):
+    """Colour 1 of such boxes has no site: its launches take part in the chain of
+    dependent launches all the same.  h = -q / 6 for any number of iterations."""
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1403_0711_gb300 import _build, coulps as cl
+    _build.build()
+    cl.use_torch_allocator()
+    q = np.random.default_rng(systems).uniform(-1, 1, systems)
+    b = cl.Batch([(1, 1, 1)] * systems, precision=cl.F32, seed=1, stream=torch.cuda.Stream())
+    b.set_charges([(np.zeros((1, 3), np.int32), q[k:k + 1]) for k in range(systems)])
+    for n_iter in (1, 2, 400):
+        g = cl.BatchGlobalCV(b, n_iter=n_iter, R=0)
+        for k in {0, systems // 2, systems - 1}:
+            assert abs(float(g.h(k).reshape(-1)[0]) + q[k] / 6.0) <= 8e-7 * abs(q[k] / 6.0)
+        g.close()
+    b.close()
