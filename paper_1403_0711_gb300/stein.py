@@ -126,13 +126,19 @@ class Conv3dTC(torch.autograd.Function):
         return da, dW, db
 
 
+def _aligned(t):
+    """t, contiguous from a 16-byte boundary (a view may start off one)."""
+    t = t.contiguous()
+    return t if t.data_ptr() % 16 == 0 else t.clone()
+
+
 class _Act(torch.autograd.Function):
     """(tanh(h) in BF16, 1 - tanh(h)^2 rounded to BF16 values, gradient passed
     straight through the rounding), bitwise the operations on CUDA FP32."""
 
     @staticmethod
     def forward(ctx, h):
-        h = h.contiguous()
+        h = _aligned(h)
         a, s = torch.empty_like(h, dtype=torch.bfloat16), torch.empty_like(h)
         coulps._check(coulps.load().coulps_cv_act_forward(_vp(h), _vp(a), _vp(s), h.numel(),
                                                           _stream()), "coulps_cv_act_forward")
@@ -146,8 +152,8 @@ class _Act(torch.autograd.Function):
         h, = ctx.saved_tensors
         if da is None and ds is None:
             return None
-        da = None if da is None else da.contiguous()
-        ds = None if ds is None else ds.contiguous()
+        da = None if da is None else _aligned(da)
+        ds = None if ds is None else _aligned(ds)
         dh = torch.empty_like(h)
         coulps._check(coulps.load().coulps_cv_act_backward(
             _vp(h), None if da is None else _vp(da), None if ds is None else _vp(ds), _vp(dh),
@@ -161,8 +167,10 @@ class _Neighbours(torch.autograd.Function):
 
     @staticmethod
     def forward(ctx, s, lo, hi):
-        s = s.contiguous()
-        n, Z, Y, X, _ = s.shape
+        n, Z, Y, X, C = s.shape
+        if C != 16 or s.dtype != torch.float32 or not s.is_cuda:  # the kernel reads as much
+            raise ValueError(f"16 channels of CUDA float32, not {tuple(s.shape)} {s.dtype}")
+        s = _aligned(s)
         ctx.box = [(ctypes.c_int32 * 3)(*v) for v in ((X, Y, Z), lo, hi)]
         ctx.shape = s.shape
         m = (hi[0] - lo[0]) * (hi[1] - lo[1]) * (hi[2] - lo[2])
@@ -174,7 +182,7 @@ class _Neighbours(torch.autograd.Function):
     @staticmethod
     @torch.autograd.function.once_differentiable
     def backward(ctx, d):
-        d = d.permute(1, 0, 3, 2).contiguous()  # [m][n][16][27]: as it comes
+        d = _aligned(d.permute(1, 0, 3, 2))  # [m][n][16][27]: as it comes
         ds = torch.empty(ctx.shape, dtype=d.dtype, device=d.device)
         coulps._check(coulps.load().coulps_cv_region_scatter(_vp(d), _vp(ds), ctx.shape[0], *ctx.box,
                                                              _stream()), "coulps_cv_region_scatter")
@@ -538,8 +546,12 @@ def _axis_index(n, lo, hi):
 _SCATTER_SITES = 56320  # coulps_cv_region_scatter's most, of the box grown by one
 
 
-def _grown_sites(lo, hi):
-    return (hi[0] - lo[0] + 2) * (hi[1] - lo[1] + 2) * (hi[2] - lo[2] + 2)
+def _gatherable(s, lo, hi):
+    """Whether _Neighbours takes the sites [lo, hi) of s: rows of 16 FP32 channels
+    (what its kernels read), at least one sample, a box that the scatter holds."""
+    grown = (hi[0] - lo[0] + 2) * (hi[1] - lo[1] + 2) * (hi[2] - lo[2] + 2)
+    return (s.is_cuda and s.dtype == torch.float32 and s.dim() == 5 and s.shape[0] > 0 and
+            s.shape[4] == 16 and grown <= _SCATTER_SITES)
 
 
 class LocalSteinCV(SteinCV):
@@ -612,7 +624,7 @@ class LocalSteinCV(SteinCV):
         qz, qy, qx = self._q[:, 0], self._q[:, 1], self._q[:, 2]
         lo = [max(v - 1, 0) for v in self.r_lo]
         hi = [min(v + 1, e) for v, e in zip(self.r_hi, self.edims)]
-        if s1.is_cuda and s1.dtype == torch.float32 and _grown_sites(lo, hi) <= _SCATTER_SITES:
+        if _gatherable(s1, lo, hi):
             patches = _Neighbours.apply(s1, lo, hi)  # the same sites in the order of _q
         else:
             s1p = torch.nn.functional.pad(s1, (0, 0, 1, 1, 1, 1, 1, 1))
