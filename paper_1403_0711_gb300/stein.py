@@ -161,32 +161,63 @@ class _Act(torch.autograd.Function):
         return dh
 
 
+def _check_rows(t):
+    if t.shape[-1] != 16 or t.dtype != torch.float32 or not t.is_cuda:  # the kernels read as much
+        raise ValueError(f"16 channels of CUDA float32, not {tuple(t.shape)} {t.dtype}")
+
+
 class _Neighbours(torch.autograd.Function):
     """(n, m, 27, 16) neighbours of the sites [lo, hi) of s (n, Z, Y, X, 16), as
     a view of the [m][n][16][27] layout that the batched product takes."""
 
     @staticmethod
     def forward(ctx, s, lo, hi):
-        n, Z, Y, X, C = s.shape
-        if C != 16 or s.dtype != torch.float32 or not s.is_cuda:  # the kernel reads as much
-            raise ValueError(f"16 channels of CUDA float32, not {tuple(s.shape)} {s.dtype}")
+        _check_rows(s)
         s = _aligned(s)
-        ctx.box = [(ctypes.c_int32 * 3)(*v) for v in ((X, Y, Z), lo, hi)]
-        ctx.shape = s.shape
+        n, Z, Y, X, _ = s.shape
+        ctx.box, ctx.shape = (lo, hi), s.shape
         m = (hi[0] - lo[0]) * (hi[1] - lo[1]) * (hi[2] - lo[2])
         left = torch.empty(m, n, 16, 27, dtype=s.dtype, device=s.device)
-        coulps._check(coulps.load().coulps_cv_region_gather(_vp(s), _vp(left), n, *ctx.box,
-                                                            _stream()), "coulps_cv_region_gather")
+        coulps._check(coulps.load().coulps_cv_region_gather(
+            _vp(s), _vp(left), n, *_boxes((X, Y, Z), lo, hi), _stream()), "coulps_cv_region_gather")
         return left.permute(1, 0, 3, 2)
 
     @staticmethod
-    @torch.autograd.function.once_differentiable
     def backward(ctx, d):
+        return _NeighboursBack.apply(d, ctx.shape, *ctx.box), None, None
+
+
+class _NeighboursBack(torch.autograd.Function):
+    """The transpose of _Neighbours, and _Neighbours its own: derivatives of any
+    order, as through the framework operations."""
+
+    @staticmethod
+    def forward(ctx, d, shape, lo, hi):
+        _check_rows(d)
+        ctx.box = lo, hi
         d = _aligned(d.permute(1, 0, 3, 2))  # [m][n][16][27]: as it comes
-        ds = torch.empty(ctx.shape, dtype=d.dtype, device=d.device)
-        coulps._check(coulps.load().coulps_cv_region_scatter(_vp(d), _vp(ds), ctx.shape[0], *ctx.box,
-                                                             _stream()), "coulps_cv_region_scatter")
-        return ds, None, None
+        ds = torch.empty(shape, dtype=d.dtype, device=d.device)
+        coulps._check(coulps.load().coulps_cv_region_scatter(
+            _vp(d), _vp(ds), shape[0], *_boxes(shape[3:0:-1], lo, hi), _stream()),
+            "coulps_cv_region_scatter")
+        return ds
+
+    @staticmethod
+    def backward(ctx, g):
+        return _Neighbours.apply(g, *ctx.box), None, None, None
+
+
+def _boxes(*v):
+    return [(ctypes.c_int32 * 3)(*t) for t in v]
+
+
+def _plain(*ts):
+    """No transform, tracer or tangent on any tensor: a kernel may take their memory."""
+    return not (torch._C._are_functorch_transforms_active() or
+                torch._C._len_torch_dispatch_stack() > 0 or torch.jit.is_tracing() or
+                torch.compiler.is_compiling() or
+                any(type(t) not in (torch.Tensor, torch.nn.Parameter) or
+                    torch.autograd.forward_ad.unpack_dual(t).tangent is not None for t in ts))
 
 
 def _face_masks():
@@ -624,7 +655,7 @@ class LocalSteinCV(SteinCV):
         qz, qy, qx = self._q[:, 0], self._q[:, 1], self._q[:, 2]
         lo = [max(v - 1, 0) for v in self.r_lo]
         hi = [min(v + 1, e) for v, e in zip(self.r_hi, self.edims)]
-        if _gatherable(s1, lo, hi):
+        if _plain(s1, s2) and _gatherable(s1, lo, hi):
             patches = _Neighbours.apply(s1, lo, hi)  # the same sites in the order of _q
         else:
             s1p = torch.nn.functional.pad(s1, (0, 0, 1, 1, 1, 1, 1, 1))

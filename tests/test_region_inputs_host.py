@@ -29,3 +29,27 @@ def test_neighbours_refuse_what_they_would_misread():
     for t in (torch.zeros(1, 4, 4, 4, 8), torch.zeros(1, 4, 4, 4, 16)):  # 8 channels; not CUDA
         with pytest.raises(ValueError):
             stein._Neighbours.apply(t, [1, 1, 1], [2, 2, 2])
+
+
+def test_transforms_and_tracers_keep_the_framework_operations():
+    from paper_1403_0711_gb300 import stein
+    x = torch.ones(2, 3)
+    seen = []
+
+    def f(t):
+        seen.append(stein._plain(t))
+        return (t * t).sum()
+
+    f(x)
+    f(torch.nn.Parameter(x))
+    assert seen == [True, True]
+    seen.clear()
+    torch.func.grad(f)(x)
+    torch.func.vmap(f)(x)
+    torch.func.jvp(f, (x,), (x,))
+    torch.jit.trace(f, x, check_trace=False)
+    with torch.autograd.forward_ad.dual_level():
+        f(torch.autograd.forward_ad.make_dual(x, x))
+    from torch.fx.experimental.proxy_tensor import make_fx
+    make_fx(f)(x)
+    assert len(seen) == 6 and not any(seen)
