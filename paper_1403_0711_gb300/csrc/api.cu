@@ -11,7 +11,10 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <map>
+#include <mutex>
 #include <new>
+#include <utility>
 #include <vector>
 
 #include "device_common.cuh"
@@ -43,6 +46,25 @@ void dev_free(const Allocator &a, void *p, cudaStream_t s) {
     return;
   }
   cudaFreeAsync(p, s);
+}
+
+cudaError_t raise_smem(const void *kernel, size_t bytes) {
+  static std::mutex lock;
+  static std::map<std::pair<int, const void *>, size_t> limits;
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  try {
+    std::lock_guard<std::mutex> hold(lock);
+    size_t &limit = limits[{dev, kernel}];
+    if (bytes > limit) {
+      e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+      if (e == cudaSuccess) limit = bytes;
+    }
+  } catch (...) {  // host memory
+    e = cudaErrorMemoryAllocation;
+  }
+  return e;
 }
 
 }  // namespace coulps

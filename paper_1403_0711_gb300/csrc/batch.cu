@@ -765,8 +765,7 @@ int batch_layout(coulps_batch *B) {
   B->threads2 = (B->threads2 + 31) / 32 * 32;
   auto resident = [&](const void *k, int threads) {
     int n = 0;
-    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)B->smem) !=
-            cudaSuccess ||
+    if (raise_smem(k, B->smem) != cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, threads, B->smem) != cudaSuccess ||
         n < 1) {
       cudaGetLastError();
@@ -787,8 +786,7 @@ int batch_layout(coulps_batch *B) {
   int pper_sm = 0;
   auto pk = B->precision == COULPS_F32 ? batch_pass_kernel<float, true, false>
                                        : batch_pass_kernel<double, true, false>;
-  if (cudaFuncSetAttribute(pk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)B->psmem) !=
-          cudaSuccess ||
+  if (raise_smem((const void *)pk, B->psmem) != cudaSuccess ||
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pper_sm, pk, B->pthreads, B->psmem) !=
           cudaSuccess ||
       pper_sm < 1) {
@@ -806,8 +804,7 @@ int batch_layout(coulps_batch *B) {
     // CTAs per SM: the fewest over the pair kinds the mode runs
     auto per_sm_of = [&](const void *k) {
       int n = 0;
-      if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)B->qsmem) !=
-              cudaSuccess ||
+      if (raise_smem(k, B->qsmem) != cudaSuccess ||
           cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, B->qthreads, B->qsmem) !=
               cudaSuccess ||
           n < 1) {
@@ -836,13 +833,8 @@ template <typename T, bool OR, bool GATHER>
 cudaError_t launch_batch_t(coulps_batch *B, const BatchArgs &a) {
   constexpr int V = batch_quads_per_thread<T, OR, GATHER>();
   auto kfn = batch_halfsweep_kernel<T, OR, GATHER, V>;
-  static size_t configured = 0;
-  if (B->smem > configured) {
-    cudaError_t e = cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)B->smem);
-    if (e != cudaSuccess) return e;
-    configured = B->smem;
-  }
+  const cudaError_t e = raise_smem((const void *)kfn, B->smem);
+  if (e != cudaSuccess) return e;
   if (V == 2)
     kfn<<<B->grid2, B->threads2, B->smem, B->stream>>>(a);
   else
@@ -860,13 +852,8 @@ cudaError_t launch_batch_p(coulps_batch *B, const BatchArgs &a, bool orx) {
 template <typename T, bool OR, bool GATHER>
 cudaError_t launch_bpass_t(coulps_batch *B, const BatchPassArgs &a) {
   auto kfn = batch_pass_kernel<T, OR, GATHER>;
-  static size_t configured = 0;
-  if (B->psmem > configured) {
-    cudaError_t e = cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)B->psmem);
-    if (e != cudaSuccess) return e;
-    configured = B->psmem;
-  }
+  const cudaError_t e = raise_smem((const void *)kfn, B->psmem);
+  if (e != cudaSuccess) return e;
   kfn<<<B->pgrid, B->pthreads, B->psmem, B->stream>>>(a);
   return cudaGetLastError();
 }
@@ -881,13 +868,8 @@ cudaError_t launch_bpass_p(coulps_batch *B, const BatchPassArgs &a, bool orx) {
 template <typename T, bool A_OR, bool B_OR, bool GATHER>
 cudaError_t launch_bpair_t(coulps_batch *B, const BatchPairArgs &a) {
   auto kfn = batch_pair_kernel<T, A_OR, B_OR, GATHER>;
-  static size_t configured = 0;
-  if (B->qsmem > configured) {
-    cudaError_t e = cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)B->qsmem);
-    if (e != cudaSuccess) return e;
-    configured = B->qsmem;
-  }
+  const cudaError_t e = raise_smem((const void *)kfn, B->qsmem);
+  if (e != cudaSuccess) return e;
   kfn<<<B->qgrid, B->qthreads, B->qsmem, B->stream>>>(a);
   return cudaGetLastError();
 }

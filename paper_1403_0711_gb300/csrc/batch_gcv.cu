@@ -342,13 +342,8 @@ cudaError_t launch_charge(coulps_batch_gcv *G, const T *field, cudaStream_t st) 
   const int blocks = (int)std::min<int64_t>((warps + kBgcvWarps - 1) / kBgcvWarps,
                                             (int64_t)G->sms * 8);
   const size_t smem = local_bytes<T>(kBgcvWarps, kBgcvCharges<T>, G->R, n_pts);
-  static size_t configured = 0;  // per instantiation
-  if (smem > configured) {
-    cudaError_t e = cudaFuncSetAttribute(bgcv_charge_kernel<T>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    configured = smem;
-  }
+  const cudaError_t e = raise_smem((const void *)bgcv_charge_kernel<T>, smem);
+  if (e != cudaSuccess) return e;
   bgcv_charge_kernel<T><<<blocks, 32 * kBgcvWarps, smem, st>>>(
       field, G->d_sys, G->d_qsite, G->d_q, G->n_q, G->d_k, G->R, n_pts, per, G->d_qpart);
   return cudaGetLastError();

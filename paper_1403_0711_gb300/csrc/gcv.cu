@@ -329,13 +329,8 @@ __global__ void __launch_bounds__(kGcvThreads, 4)
 template <typename T>
 cudaError_t launch_eval(const Geometry &g, const EvalArgs &A, cudaStream_t s) {
   const size_t smem = A.nblk_p > 0 ? local_bytes<T>(kEvalWarps, kEvalCharges<T>, A.R, A.n_pts) : (size_t)0;
-  static size_t configured = 0;  // per instantiation
-  if (smem > configured) {
-    cudaError_t e = cudaFuncSetAttribute(gcv_eval_kernel<T>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    configured = smem;
-  }
+  const cudaError_t e = raise_smem((const void *)gcv_eval_kernel<T>, smem);
+  if (e != cudaSuccess) return e;
   gcv_eval_kernel<T><<<dim3(A.nblk + A.nblk_p, g.n_chains), kGcvThreads, smem, s>>>(g, A);
   return cudaGetLastError();
 }

@@ -269,6 +269,11 @@ Allocator current_allocator();
 void *dev_alloc(const Allocator &a, size_t bytes, cudaStream_t s);
 void dev_free(const Allocator &a, void *p, cudaStream_t s);
 
+// Lets launches of `kernel` on the current device take `bytes` of dynamic shared
+// memory.  The kernel's limit is only ever raised: objects with tiles of several
+// sizes share it, and one that takes less must not lower it for the others.
+cudaError_t raise_smem(const void *kernel, size_t bytes);
+
 // Launchers (return cudaError_t of the launch).
 cudaError_t launch_halfsweep(const Geometry &g, const Tile &t, const CUtensorMap &tm_halo,
                              const CUtensorMap &tm_own, const SweepArgs &a, bool overrelax,
