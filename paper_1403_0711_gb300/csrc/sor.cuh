@@ -36,8 +36,9 @@ void sor_charges(const SorBox &b, int64_t n, const int32_t *sites, const double 
 
 // Solves every box: n_iter iterations from u = 0 (colour 0, then colour 1).
 // Leaves u and the density in natural order in u_nat and rho_nat; works in
-// split arrays and lists of its own from `alloc`.  Synchronises s once (the
-// host lists' uploads).  cudaErrorMemoryAllocation if an allocation fails.
+// split arrays and lists of its own from `alloc`, or where these do not fit in
+// u_nat and rho_nat themselves (slower, the same u).  Synchronises s once (the
+// host lists' uploads).
 cudaError_t sor_solve(const std::vector<SorBox> &boxes, const std::vector<SorCharge> &charges,
                       int n_iter, double *u_nat, double *rho_nat, const Allocator &alloc,
                       cudaStream_t s);
