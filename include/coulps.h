@@ -447,7 +447,8 @@ int coulps_checkpoint_load(coulps_lattice_t lat, coulps_charges_t ch, const char
  * with that chain id.  Storage, boundary, update rules and estimator are those
  * of the lattice API above; the measured compound sweep gathers Q, P in its
  * last kernel and is replayed as one CUDA graph.  By default the
- * over-relaxation passes run as pass pairs (coulps_batch_set_fused). */
+ * over-relaxation passes run as pass pairs, in FP64 from 2^19 sites on as fused
+ * passes (coulps_batch_set_fused). */
 typedef struct coulps_batch *coulps_batch_t;
 
 /* dims[3s..3s+2] = (Lx, Ly, Lz) of system s, limits as coulps_lattice_create.
@@ -472,7 +473,9 @@ int coulps_batch_info(coulps_batch_t b, int64_t *info);
  * a compound sweep run as fused passes (both half-sweeps of a pass in one
  * z-march, each site read and written once, 8 bytes per site in FP32
  * instead of 12), one persistent launch per pass over a list of pass tiles.
- * enable = 2 (the default when every system admits a pair tile): they run
+ * enable = 2 (the default when every system admits a pair tile, but for FP64
+ * batches of 2^19 sites and more, created with enable = 1 as the faster way;
+ * coulps_batch_set_pair_tiles on such a batch sets enable = 2): they run
  * as pass pairs (two passes in one z-march, 4 bytes per site and pass), one
  * persistent launch per pair over a list of pair tiles, largest first, and
  * a fused pass for an odd remainder.  The heatbath passes stay half-sweeps,

@@ -640,8 +640,9 @@ class Batch:
 
     def set_fused(self, mode):
         """Over-relaxation passes as half-sweeps only (0), fused passes (1) or
-        pass pairs (2, the default where every system admits a pair tile); 3:
-        all passes, heatbath ones included, as pass pairs and fused passes."""
+        pass pairs (2, the default where every system admits a pair tile, but
+        1 for FP64 batches of 2^19 sites and more); 3: all passes, heatbath ones
+        included, as pass pairs and fused passes."""
         _check(self._lib.coulps_batch_set_fused(self.handle, int(mode)), "coulps_batch_set_fused")
 
     def fused(self):

@@ -610,11 +610,19 @@ void batch_choose_tiles(coulps_batch *B) {
       else { S.TY = best[s].ty; S.DZ = best[s].dz; }
     }
   }
-  // FP64, bound by the FP64 unit: a pair's halo rows cost more than the second
-  // trip through memory (compound sweep 1:3 with pairs against fused passes: 64
-  // systems of 32 .. 80 1129 against 1044 us, 200 of 14 .. 40 529 against 457, 1000
-  // of 14 .. 33 1492 against 1270; only 8 of 50 .. 90 330 against 359).
-  if (B->precision == COULPS_F64) B->pairs_pay = false;
+}
+
+// Whether a batch is created with pass pairs (mode 2) or fused passes (mode 1);
+// set_fused and set_pair_tiles choose otherwise.  FP64 is bound by the FP64
+// unit: a pair's halo rows cost it more than the second trip through memory
+// (compound sweep 1:3 with pairs against fused passes: 64 systems of 32 .. 80
+// 1129 against 1044 us, 200 of 14 .. 40 529 against 457, 1000 of 14 .. 33 1492
+// against 1270; only 8 of 50 .. 90 330 against 359).  Below 2^19 sites, where a
+// launch is its latency, the pairs' fewer launches stay.
+bool batch_pairs_pay(const coulps_batch *B) {
+  long long sites = 0;
+  for (const auto &S : B->sys) sites += (long long)S.Lx * S.Ly * S.Lz;
+  return B->precision == COULPS_F32 || sites < (1ll << 19);
 }
 
 // Tile lists, tensor maps and gather lists for the current tile shapes.
@@ -917,7 +925,7 @@ int batch_enqueue_compound(coulps_batch *B, int n_hb, int n_or, bool measure) {
       default: d = (n - 1) / 2; s = 1; break;
     }
   } else if (B->fused && B->field2) {
-    d = B->fused >= 2 && B->pairs_pay ? n_or / 2 : 0;
+    d = B->fused >= 2 ? n_or / 2 : 0;
     s = n_or - 2 * d;
     if ((d + s) % 2 == 1) {
       if (n_hb > 0) {
@@ -1137,8 +1145,10 @@ int coulps_batch_create(int n_systems, const int32_t *dims, int precision, uint6
   batch_reset_stats_kernel<<<(n_systems * kStatStride + 255) / 256, 256, 0, B->stream>>>(
       B->d_stats, n_systems);
   batch_choose_tiles(B);
-  int st = coulps_batch_set_fused(B, batch_pairs_ok(B) ? 2 : 1);
+  const bool pairs = batch_pairs_ok(B), pay = batch_pairs_pay(B);
+  int st = coulps_batch_set_fused(B, pairs && pay ? 2 : 1);
   if (!st) st = batch_layout(B);
+  B->passes_by_default = pairs && !pay;
   if (st) {
     coulps_batch_destroy(B);
     return st;
@@ -1150,6 +1160,7 @@ int coulps_batch_create(int n_systems, const int32_t *dims, int precision, uint6
 int coulps_batch_set_fused(coulps_batch_t B, int enable) {
   if (!B || enable < 0 || enable > 3) return COULPS_EINVAL;
   if (enable >= 2 && !batch_pairs_ok(B)) return COULPS_EINVAL;
+  B->passes_by_default = false;
   batch_drop_graph(B);
   if (!enable) {
     if (B->field2) {
@@ -1206,8 +1217,12 @@ int coulps_batch_set_pair_tiles(coulps_batch_t B, const int32_t *ty_dz) {
     if (dz > 0) S.QDZ = dz;
     if (!batch_pair_fits(S, S.QTY, B->es)) return COULPS_EINVAL;
   }
-  B->pairs_pay = true;
   B->sys = next;
+  if (B->passes_by_default) {  // the tiles ask for pairs
+    B->passes_by_default = false;
+    batch_drop_graph(B);
+    B->fused = 2;
+  }
   B->layout_dirty = true;
   return batch_layout(B);
 }

@@ -50,7 +50,7 @@ struct coulps_batch {
   // the pass tiles, their maps [copy][system][2] and gather lists; with
   // fused = 2 also the pair tiles
   int fused = 0;
-  bool pairs_pay = true;  // mode 2 runs pairs (else fused passes only)
+  bool passes_by_default = false;  // created in mode 1 because pairs would not pay
   void *field2 = nullptr;
   std::vector<coulps::BatchItem> pitems;
   coulps::BatchItem *d_pitems = nullptr;
