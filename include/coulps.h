@@ -113,6 +113,14 @@ int coulps_lattice_info(coulps_lattice_t lat, int64_t info[13]);
  * Errors: EINVAL (ty*W/4 > 256 threads, ty < 1, dz < 1). */
 int coulps_set_tile(coulps_lattice_t lat, int ty, int dz);
 
+/* How compound sweeps of this mix run now: out[0] = CTAs that hold a chain (0:
+ * the tiled kernels), out[1] = compound sweeps in a launch (about 0.1 s of them
+ * at most; 1 with the tiled kernels).  n_sweeps = 0: the measured sweeps of
+ * coulps_run; n_sweeps > 0: so many sweeps between two samples that another
+ * kernel takes (off-lattice and several sets, control variates), or that many
+ * sweeps of coulps_sweep.  Errors: EINVAL. */
+int coulps_resident(coulps_lattice_t lat, int n_hb, int n_or, int n_sweeps, int32_t out[2]);
+
 /* Copy chain `chain`'s field to / from a host array of Lx*Ly*Lz doubles in
  * natural order.  Synchronises the stream.  field_set does not change the
  * pass counter.  Errors: EINVAL, ECUDA, and any recorded device error. */

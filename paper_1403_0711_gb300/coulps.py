@@ -56,7 +56,7 @@ EXPORTS = (
     "coulps_batch_set_fused", "coulps_batch_set_pass_tiles", "coulps_batch_system_pass_tile",
     "coulps_batch_fused", "coulps_batch_set_pair_tiles", "coulps_batch_system_pair_tile",
     "coulps_cv_pack_weights_dev", "coulps_cv_act_forward", "coulps_cv_act_backward",
-    "coulps_cv_region_gather", "coulps_cv_region_scatter",
+    "coulps_cv_region_gather", "coulps_cv_region_scatter", "coulps_resident",
 )
 SCHEDULE_ALIGNED, SCHEDULE_PHASED, SCHEDULE_SHIFTED = 0, 1, 2
 STAT_STRIDE = 72
@@ -190,6 +190,7 @@ def load(path: str | Path | None = None):
         "coulps_set_pass_tile": (i32, [vp, i32, i32]),
         "coulps_set_pair_tile": (i32, [vp, i32, i32]),
         "coulps_pair_tile": (i32, [vp, P(i32)]),
+        "coulps_resident": (i32, [vp, i32, i32, i32, P(i32)]),
         "coulps_kernel_times_n": (i32, [vp, P(f64), i32]),
         "coulps_cv_pack_weights_dev": (i32, [vp, vp, vp]),
         "coulps_cv_act_forward": (i32, [vp, vp, vp, i64, vp]),
@@ -355,6 +356,14 @@ class Lattice:
     def pair_tile(self):
         a = (ctypes.c_int32 * 2)()
         _check(self._lib.coulps_pair_tile(self.handle, a), "coulps_pair_tile")
+        return int(a[0]), int(a[1])
+
+    def resident(self, n_hb=1, n_or=3, n_sweeps=0):
+        """(CTAs that hold a chain, or 0 with the tiled kernels; compound sweeps in
+        a launch) of this mix now (coulps_resident)."""
+        a = (ctypes.c_int32 * 2)()
+        _check(self._lib.coulps_resident(self.handle, int(n_hb), int(n_or), int(n_sweeps), a),
+               "coulps_resident")
         return int(a[0]), int(a[1])
 
     def checkpoint_save(self, path, charges=None):

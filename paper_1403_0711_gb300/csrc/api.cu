@@ -533,6 +533,15 @@ PassPlan pass_plan(const coulps_lattice *L, int n_hb, int n_or) {
   return P;
 }
 
+// A launch cannot be interrupted: it takes as many compound sweeps as are
+// estimated to last 0.1 s (2048 at most; the launch itself is 10 us), and a mix
+// whose single sweep is estimated longer stays with the march kernels.
+constexpr double kResidentLaunch = 1e5;  // us
+int resident_sweeps(const coulps_lattice *L, int n_hb, int n_or) {
+  const double t = resident_time(L->g, L->rplan, n_hb, n_or);
+  return (int)std::min(2048.0, std::max(1.0, kResidentLaunch / t));
+}
+
 // Whether compound sweeps of this mix run resident now: where that is clearly
 // the shorter way (profiling times the march kernels one by one, the other
 // schedules are theirs).  The same for every number of sweeps, so that a run
@@ -556,6 +565,7 @@ bool resident_on(const coulps_lattice *L, int n_hb, int n_or, int n_sweeps = 0) 
   const Geometry &g = L->g;
   const ResidentPlan &p = L->rplan;
   double t = resident_time(g, p, n_hb, n_or), clear = 0.9;
+  if (t > kResidentLaunch) return false;
   if (n_sweeps > 0) {
     const int waves = (g.n_chains + p.active - 1) / p.active;
     t += (8.0 + waves * (2.5 + 0.02e-3 * (double)p.smem)) / n_sweeps;
@@ -788,10 +798,7 @@ int enqueue_part(coulps_lattice *L, cudaStream_t st, int n_hb, int n_or, coulps_
 }
 
 // n_sweeps compound sweeps of every chain (each sampled when `fuse` is given)
-// by the resident kernel, in launches of at most kResidentSweeps (a launch of
-// the largest resident lattices then lasts some 0.1 s).
-constexpr int kResidentSweeps = 2048;
-
+// by the resident kernel, in launches of resident_sweeps.
 int enqueue_resident(coulps_lattice *L, int n_sweeps, int n_hb, int n_or, coulps_charges *fuse) {
   ResidentArgs a = {};
   const Geometry &g = L->g;
@@ -816,8 +823,9 @@ int enqueue_resident(coulps_lattice *L, int n_sweeps, int n_hb, int n_or, coulps
     a.log = fuse->d_log;
     a.log_cap = fuse->log_cap;
   }
-  for (int done = 0; done < n_sweeps; done += kResidentSweeps) {
-    a.n_sweeps = std::min(kResidentSweeps, n_sweeps - done);
+  const int per = resident_sweeps(L, n_hb, n_or);
+  for (int done = 0; done < n_sweeps; done += per) {
+    a.n_sweeps = std::min(per, n_sweeps - done);
     CK(launch_resident(g, L->rplan, a, fuse ? fuse->n : 0, L->stream));
     CK(launch_advance_pass(L->d_pass, (uint32_t)a.n_sweeps * (uint32_t)(n_hb + n_or), L->stream));
   }
@@ -1473,6 +1481,14 @@ static int set_fused(coulps_lattice *L, int enable) {
   int st = rebuild_maps(L);
   if (st) return st;
   return rebuild_pass_maps(L);
+}
+
+int coulps_resident(coulps_lattice_t L, int n_hb, int n_or, int n_sweeps, int32_t out[2]) {
+  if (!L || n_hb < 0 || n_or < 0 || n_sweeps < 0 || !out) return COULPS_EINVAL;
+  const bool on = resident_on(L, n_hb, n_or, n_sweeps);
+  out[0] = on ? L->rplan.cluster : 0;
+  out[1] = on ? resident_sweeps(L, n_hb, n_or) : 1;
+  return COULPS_OK;
 }
 
 int coulps_set_pair_tile(coulps_lattice_t L, int ty, int dz) {
