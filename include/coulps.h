@@ -107,19 +107,25 @@ int coulps_lattice_info(coulps_lattice_t lat, int64_t info[13]);
  * sweeps (aligned schedule, profiling off) with each chain held in the shared
  * memory of a cluster of CTAs wherever that is the faster way (small chains);
  * any call of coulps_set_tile, coulps_set_pass_tile, coulps_set_pair_tile or
- * coulps_set_fused that succeeds selects the tiled kernels instead.  Fields
- * are bitwise the same, samples up to the order of the FP64 sums over the
- * charges.
+ * coulps_set_fused that succeeds selects the tiled kernels instead, until
+ * coulps_set_resident(lat, 1).  Fields are bitwise the same, samples up to the
+ * order of the FP64 sums over the charges.
  * Errors: EINVAL (ty*W/4 > 256 threads, ty < 1, dz < 1). */
 int coulps_set_tile(coulps_lattice_t lat, int ty, int dz);
 
+/* enable = 1: compound sweeps may run with the chains in shared memory, wherever
+ * that is the faster way (the state of a new lattice; tiles and mode stay as
+ * they are); 0: the tiled kernels only.  Errors: EINVAL. */
+int coulps_set_resident(coulps_lattice_t lat, int enable);
+
 /* How compound sweeps of this mix run now: out[0] = CTAs that hold a chain (0:
  * the tiled kernels), out[1] = compound sweeps in a launch (about 0.1 s of them
- * at most; 1 with the tiled kernels).  n_sweeps = 0: the measured sweeps of
+ * at most; 1 with the tiled kernels), out[2] = 1 if the choice is the library's
+ * (coulps_set_resident).  n_sweeps = 0: the measured sweeps of
  * coulps_run; n_sweeps > 0: so many sweeps between two samples that another
  * kernel takes (off-lattice and several sets, control variates), or that many
  * sweeps of coulps_sweep.  Errors: EINVAL. */
-int coulps_resident(coulps_lattice_t lat, int n_hb, int n_or, int n_sweeps, int32_t out[2]);
+int coulps_resident(coulps_lattice_t lat, int n_hb, int n_or, int n_sweeps, int32_t out[3]);
 
 /* Copy chain `chain`'s field to / from a host array of Lx*Ly*Lz doubles in
  * natural order.  Synchronises the stream.  field_set does not change the

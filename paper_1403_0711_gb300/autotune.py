@@ -3,22 +3,28 @@ half-sweep kernel, the fused-pass kernel and the pass-pair kernel.
 
 The shape changes only the work decomposition, never the results (the tests
 check fields bitwise across shapes), so the tuner may pick freely.  For a box
-shape it times every candidate with the library's own per-kernel CUDA-event
-timing (coulps_set_profiling / coulps_kernel_times) over a few compound
-sweeps and keeps the fastest.  Results are cached in a JSON file keyed by box,
+shape it times every candidate, the library's own default among them, with the
+library's per-kernel CUDA-event timing (coulps_set_profiling /
+coulps_kernel_times) over a few compound sweeps and keeps the fastest; then it
+runs whole measured sweeps with the tuned tiles and as the library does by
+itself (small lattices: without tiles, resident in shared memory), and the
+tuned tiles are used only where they are the faster way.  Results are cached in a JSON file keyed by box,
 chain count, precision, compound-sweep mix and GPU name
 ($COULPS_TUNE_CACHE, default ~/.cache/coulps_tune.json).
 
 tune_lattice(lat)  tunes and applies the three shapes of a Lattice (the
-                   half-sweep shape serves passes that are not fused).
+                   half-sweep shape serves passes that are not fused); sweeps
+                   that ran resident and were faster so go on resident.
 tune_batch(batch)  tunes each distinct system shape of a Batch (with as many
                    chains as the batch has systems of that shape, so the tuned
-                   lattice carries the same load) and applies them.
+                   lattice carries the same load) and applies them, unless the
+                   batch's default tiles are faster.
 """
 from __future__ import annotations
 
 import json
 import os
+import time
 from pathlib import Path
 
 from . import coulps
@@ -109,6 +115,11 @@ def _time_shapes(L, n_chains, precision, shapes, n_hb, n_or, reps, stream, fused
     out = {}
     try:
         lat.sweep(2, n_hb, n_or)
+        i = lat.info()
+        own = lat.pair_tile() if pair else (
+            (i["pass_ty"], i["pass_dz"]) if fused else (i["ty"], i["dz"]))
+        if own[0] > 0 and own not in shapes:
+            shapes = [own, *shapes]
         for ty, dz in shapes:
             try:
                 if pair:
@@ -198,18 +209,118 @@ def tune_pair_shape(L, n_chains=1, precision=coulps.F32, n_hb=1, n_or=3, reps=3,
     return best
 
 
+def _run_time(run, sync):
+    """Seconds per sweep of run(n sweeps): the best of three runs of 5 ms or more."""
+    run(2)
+    sync()
+    n, best = 1, float("inf")
+    while True:
+        t = time.perf_counter()
+        run(n)
+        sync()
+        t = time.perf_counter() - t
+        if t >= 5e-3 or n >= 4096:
+            break
+        n *= 4
+    for _ in range(3):
+        t = time.perf_counter()
+        run(n)
+        sync()
+        best = min(best, (time.perf_counter() - t) / n)
+    return best
+
+
+def _apply(lat, tiles):
+    """Half-sweep, pass and pair tile (None: as it is)."""
+    for set_tile, t in zip((lat.set_tile, lat.set_pass_tile, lat.set_pair_tile), tiles):
+        if t is not None:
+            set_tile(*t)
+
+
+def _lattice_tiles(lat):
+    i, q = lat.info(), lat.pair_tile()
+    return (i["ty"], i["dz"]), (i["pass_ty"], i["pass_dz"]), (q if q[0] > 0 else None)
+
+
+def _lattice_times(lat, tiles, n_hb, n_or, stream):
+    """Times of a measured sweep of a lattice like `lat` as the library runs it and
+    with these tiles; the library's tiles; whether it ran resident."""
+    out = []
+    for own in (True, False):
+        c = coulps.Lattice(lat.L, n_chains=lat.n_chains, precision=lat.precision, seed=1,
+                           stream=stream)
+        try:
+            if c.info()["fused"] != lat.info()["fused"]:
+                c.set_fused(lat.info()["fused"])
+            c.set_streams(lat._streams)
+            c.set_resident(lat.resident_enabled())
+            if own:
+                default, resident = _lattice_tiles(c), c.resident(n_hb, n_or)[0] > 0
+            else:
+                _apply(c, tiles)
+            ch = coulps.Charges(c, [[0, 0, 0]], [1.0])
+            try:
+                out.append(_run_time(lambda n: ch.run(0, n, n_hb, n_or), c.sync))
+            finally:
+                ch.close()
+        finally:
+            c.close()
+    return out[0], out[1], default, resident
+
+
 def tune_lattice(lat: "coulps.Lattice", n_hb=1, n_or=3, reps=3, stream=None):
     """Tunes the half-sweep, fused-pass and pass-pair shapes; returns the
     half-sweep shape (the others are applied too: lat.info(), lat.pair_tile())."""
     s = stream or lat._stream
-    best = tune_shape(lat.L, lat.n_chains, lat.precision, n_hb, n_or, reps, s)
-    lat.set_tile(*best)
-    pbest = tune_pass_shape(lat.L, lat.n_chains, lat.precision, n_hb, n_or, reps, s)
-    lat.set_pass_tile(*pbest)
-    qbest = tune_pair_shape(lat.L, lat.n_chains, lat.precision, n_hb, n_or, reps, s)
-    if qbest is not None and lat.pair_tile()[0] > 0:
-        lat.set_pair_tile(*qbest)
-    return best
+    shape = (lat.L, lat.n_chains, lat.precision, n_hb, n_or, reps, s)
+    enabled = lat.resident_enabled()
+    tiles = (tune_shape(*shape), tune_pass_shape(*shape),
+             tune_pair_shape(*shape) if lat.pair_tile()[0] > 0 else None)
+    key = (f"plan|{lat.L[0]}x{lat.L[1]}x{lat.L[2]}|{lat.n_chains}|{lat.precision}|{n_hb}:{n_or}|"
+           f"{lat.info()['fused']}|{lat._streams}|{int(enabled)}|{tiles}|{_gpu_name()}")
+    plan = _load_cache().get(key)
+    if plan is None:
+        plan = {"tile": list(tiles[0]), "resident": False}
+        try:
+            own, tuned, default, resident = _lattice_times(lat, tiles, n_hb, n_or, s)
+        except coulps.CoulpsError as e:
+            if e.status != coulps.ENOMEM:  # no room for another lattice: the tuned tiles
+                raise
+        else:
+            # the library's way where it is no slower; resident sweeps use no tile
+            plan["ms"] = 1e3 * min(own, tuned)
+            if own <= tuned and resident:
+                plan["resident"] = True
+            elif own <= tuned:
+                plan["tile"], plan["tiles"] = list(default[0]), default
+            cache = _load_cache()
+            cache[key] = plan
+            _save_cache(cache)
+    resident = enabled and lat.resident(n_hb, n_or)[0] > 0
+    _apply(lat, plan.get("tiles", tiles))
+    # as before, unless the tuned tiles beat the resident sweeps
+    lat.set_resident(enabled and (plan["resident"] or not resident))
+    return tuple(plan["tile"])
+
+
+def _batch_times(batch, tiles, n_hb, n_or, stream):
+    """Times of a measured sweep of a batch like this one with its default tiles
+    and with these; the default tiles."""
+    out = []
+    for own in (True, False):
+        b = coulps.Batch(batch.dims, precision=batch.precision, seed=1, stream=stream)
+        try:
+            if b.fused() != batch.fused():
+                b.set_fused(batch.fused())
+            if own:
+                default = b.tiles()
+            else:
+                b.set_tiles(tiles)
+            b.set_charges([([[0, 0, 0]], [1.0])] * b.n)
+            out.append(_run_time(lambda n: b.run(0, n, n_hb, n_or), b.sync))
+        finally:
+            b.close()
+    return out[0], out[1], default
 
 
 def tune_batch(batch: "coulps.Batch", n_hb=1, n_or=3, reps=3, stream=None):
@@ -218,5 +329,12 @@ def tune_batch(batch: "coulps.Batch", n_hb=1, n_or=3, reps=3, stream=None):
         shapes[L] = shapes.get(L, 0) + 1
     best = {L: tune_shape(L, cnt, batch.precision, n_hb, n_or, reps, stream)
             for L, cnt in shapes.items()}
+    try:
+        own, tuned, default = _batch_times(batch, [best[L] for L in batch.dims], n_hb, n_or, stream)
+        if own <= tuned:
+            best = dict(zip(batch.dims, default))
+    except coulps.CoulpsError as e:
+        if e.status != coulps.ENOMEM:  # no room for another batch: the tuned tiles
+            raise
     batch.set_tiles([best[L] for L in batch.dims])
     return best

@@ -57,6 +57,7 @@ EXPORTS = (
     "coulps_batch_fused", "coulps_batch_set_pair_tiles", "coulps_batch_system_pair_tile",
     "coulps_cv_pack_weights_dev", "coulps_cv_act_forward", "coulps_cv_act_backward",
     "coulps_cv_region_gather", "coulps_cv_region_scatter", "coulps_resident",
+    "coulps_set_resident",
 )
 SCHEDULE_ALIGNED, SCHEDULE_PHASED, SCHEDULE_SHIFTED = 0, 1, 2
 STAT_STRIDE = 72
@@ -190,6 +191,7 @@ def load(path: str | Path | None = None):
         "coulps_set_pass_tile": (i32, [vp, i32, i32]),
         "coulps_set_pair_tile": (i32, [vp, i32, i32]),
         "coulps_pair_tile": (i32, [vp, P(i32)]),
+        "coulps_set_resident": (i32, [vp, i32]),
         "coulps_resident": (i32, [vp, i32, i32, i32, P(i32)]),
         "coulps_kernel_times_n": (i32, [vp, P(f64), i32]),
         "coulps_cv_pack_weights_dev": (i32, [vp, vp, vp]),
@@ -260,6 +262,7 @@ class Lattice:
         self.precision = int(precision)
         self.seed = int(seed)
         self._stream = stream
+        self._streams = 1
         h = ctypes.c_void_p()
         _check(self._lib.coulps_lattice_create(*self.L, self.n_chains, self.precision,
                                                self.seed, _stream_handle(stream), ctypes.byref(h)),
@@ -334,6 +337,7 @@ class Lattice:
     def set_streams(self, n):
         """1 or 2 streams per compound sweep (coulps_set_streams)."""
         _check(self._lib.coulps_set_streams(self.handle, int(n)), "coulps_set_streams")
+        self._streams = int(n)
 
     def set_schedule(self, schedule):
         _check(self._lib.coulps_set_schedule(self.handle, int(schedule)), "coulps_set_schedule")
@@ -358,13 +362,26 @@ class Lattice:
         _check(self._lib.coulps_pair_tile(self.handle, a), "coulps_pair_tile")
         return int(a[0]), int(a[1])
 
+    def set_resident(self, enable=True):
+        """Small lattices held in shared memory where that is the faster way (the
+        default, left by choosing a tile or a fused mode), or the tiled kernels
+        only (coulps_set_resident)."""
+        _check(self._lib.coulps_set_resident(self.handle, int(bool(enable))),
+               "coulps_set_resident")
+
     def resident(self, n_hb=1, n_or=3, n_sweeps=0):
         """(CTAs that hold a chain, or 0 with the tiled kernels; compound sweeps in
         a launch) of this mix now (coulps_resident)."""
-        a = (ctypes.c_int32 * 2)()
+        a = (ctypes.c_int32 * 3)()
         _check(self._lib.coulps_resident(self.handle, int(n_hb), int(n_or), int(n_sweeps), a),
                "coulps_resident")
         return int(a[0]), int(a[1])
+
+    def resident_enabled(self):
+        """Whether the library chooses (set_resident)."""
+        a = (ctypes.c_int32 * 3)()
+        _check(self._lib.coulps_resident(self.handle, 1, 0, 0, a), "coulps_resident")
+        return bool(a[2])
 
     def checkpoint_save(self, path, charges=None):
         _check(self._lib.coulps_checkpoint_save(self.handle, charges.handle if charges else None,

@@ -100,7 +100,7 @@ struct coulps_lattice {
   Tile qtile = {0, 0};
   CUtensorMap tm_q1[2], tm_q0[2];
   // small lattices run resident (resident.cu) unless the caller has chosen a
-  // tile or a fused mode, which names the march kernels
+  // tile or a fused mode, which names the march kernels (set_resident: again)
   ResidentPlan rplan;  // cluster = 0: the march kernels
   bool pinned = false;
   size_t bytes = 0;
@@ -1483,11 +1483,19 @@ static int set_fused(coulps_lattice *L, int enable) {
   return rebuild_pass_maps(L);
 }
 
-int coulps_resident(coulps_lattice_t L, int n_hb, int n_or, int n_sweeps, int32_t out[2]) {
+int coulps_set_resident(coulps_lattice_t L, int enable) {
+  if (!L || enable < 0 || enable > 1) return COULPS_EINVAL;
+  if (L->pinned != !enable) drop_graph(L);
+  L->pinned = !enable;
+  return COULPS_OK;
+}
+
+int coulps_resident(coulps_lattice_t L, int n_hb, int n_or, int n_sweeps, int32_t out[3]) {
   if (!L || n_hb < 0 || n_or < 0 || n_sweeps < 0 || !out) return COULPS_EINVAL;
   const bool on = resident_on(L, n_hb, n_or, n_sweeps);
   out[0] = on ? L->rplan.cluster : 0;
   out[1] = on ? resident_sweeps(L, n_hb, n_or) : 1;
+  out[2] = !L->pinned;
   return COULPS_OK;
 }
 
