@@ -11,7 +11,7 @@
 // than the work of a small box) overlaps the end of the one before.
 // Measured, us per half-sweep, before (natural order, every second thread
 // idle, 64-bit divisions for the coordinates, an FP64 division) -> now: 16^3
-// 4.2 -> 1.7, 48 x 40 x 44 8.3 -> 2.8, 64^3 12.6 -> 4.5, 128^3 69.9 -> 15.0 (18.4
+// 4.2 -> 1.5, 48 x 40 x 44 8.3 -> 2.6, 64^3 12.6 -> 4.3, 128^3 69.9 -> 14.9 (18.4
 // without the programmatic launches); 256 boxes of 32^3 .. 96^3, 626
 // iterations, 3.42 -> 0.70 s.  Two sites per thread: 96^3 9.6 instead of 7.3,
 // the same at 128^3; 256 threads: 48 x 40 x 44 4.7 instead of 2.8.
@@ -43,11 +43,15 @@ __global__ void __launch_bounds__(kSorThreads)
   const long long at = b.off + (long long)colour * b.colour + (it.z + 1) * plane +
                        (long long)(y + 1) * b.Ws + h;
   const double *o = u + at + (colour ? -b.colour : b.colour);
-  // every thread waits, also those without a site: a grid without a waiting
-  // thread (colour 1 of boxes of one site) would end before the grid ahead of
-  // it, and the grid behind it would then run beside that one
+  if (t >= b.Ly * b.Wh || 2 * h + par >= b.Lx) {
+    // One thread of each CTA waits even without a site: a grid in which none did
+    // (colour 1 of boxes of one site) would end before the grid ahead of it, and
+    // the grid behind it would then run beside that one.  (Every idle thread
+    // waiting costs 48 x 40 x 44 5.0 instead of 2.6 us a half-sweep.)
+    if (threadIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
+    return;
+  }
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  if (t >= b.Ly * b.Wh || 2 * h + par >= b.Lx) return;
   const double zm = o[-plane], zp = o[plane], ym = o[-b.Ws], yp = o[b.Ws], c = o[0],
                e = o[par ? 1 : -1], w = u[at], q = r[at];
   const double S = ((zm + zp) + (ym + yp)) + (c + e);
@@ -99,8 +103,9 @@ __global__ void __launch_bounds__(kSorThreads)
 }
 
 // Where the split arrays do not fit in device memory: the solve in u_nat and
-// rho_nat alone, box by box, with no allocation.  Bitwise the same u; 128^3
-// takes 4.6 times as long.
+// rho_nat alone, box by box, with no allocation.  Bitwise the same u; 400
+// iterations of 64^3 / 128^3 with the set-up around them 6.8 / 30.2 ms instead of
+// 4.0 / 12.7.
 cudaError_t solve_in_place(const std::vector<SorBox> &boxes, const std::vector<SorCharge> &charges,
                            int n_iter, size_t nat, double *u_nat, double *rho_nat,
                            cudaStream_t s) {
