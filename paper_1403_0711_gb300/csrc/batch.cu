@@ -141,10 +141,12 @@ struct BatchHalf {
 };
 
 template <typename T, bool OR, bool GATHER, int V>
-// (FP32, two quads per thread: at most 80 registers, six CTAs of 128 threads per
-// SM; unbounded it takes 106 and a compound sweep of 256 systems 600 instead of
-// 588 us.  One quad: at most 64, or the heatbath's gather form takes 96 and such a
-// sweep of heatbath passes only 242 instead of 234 us)
+// (Compound sweeps of the 256 systems named at batch_choose_tiles, seed 7 / 3.  FP32,
+// two quads per thread: at most 80 registers, six CTAs of 128 threads per SM; it
+// takes 106 unbounded, which made 600 instead of 588 us (seed 3) with the largest
+// tiles and makes 590 / 530 instead of 595 / 532 with the chosen ones.  One quad: at
+// most 64, or the heatbath's gather form takes 96 and a sweep of heatbath passes
+// only 278 / 247 instead of 265 / 234)
 __global__ void __launch_bounds__(kBatchThreads, sizeof(T) == 8 ? 1 : (V == 2 ? 3 : 4))
     batch_halfsweep_kernel(const BatchArgs a) {
   extern __shared__ unsigned char smem_raw[];
@@ -546,11 +548,13 @@ double batch_time(const coulps_batch *B, MarchKind kind, const std::vector<Tile>
 // The systems' default tiles: the rule whose launch is estimated shortest, where
 // that is clearly below the estimate for the largest tiles (given).  Those leave
 // SMs idle in a batch of few systems and CTAs waiting for the last, largest tiles
-// in one of more.  Compound sweep 1:3, largest tiles against chosen ones, us: 256
-// systems of 32 .. 96 561 against 523, 64 of 32 .. 80 160 against 123, 20 of 37 .. 90
-// 177 against 68, 8 of 50 .. 90 163 against 60; FP64 64 systems 2967 (with the
-// deviates by erfcinv) against 1044.  Batches below 2^19 sites (a launch is its latency) keep the
-// largest tiles.
+// in one of more.  Measured compound sweep 1:3, largest tiles against chosen ones,
+// us: 256 cubes of 32 .. 96, 95.7M sites (inputs.batch_systems(256, 7)) 621 against
+// 596, 84.0M sites (seed 3) 561 against 532; 64 of 32 .. 80 160 against 123, 20 of
+// 37 .. 90 177 against 68, 8 of 50 .. 90 163 against 60; FP64 64 systems 2967 (with
+// the deviates by erfcinv) against 1044; heatbath only 264 against 265 and 234
+// against 234 of the 256.  Batches below 2^19 sites (a launch is its latency) keep
+// the largest tiles.
 void batch_choose_tiles(coulps_batch *B) {
   int dev = 0, sms = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
@@ -616,9 +620,10 @@ void batch_choose_tiles(coulps_batch *B) {
 // set_fused and set_pair_tiles choose otherwise.  FP64 is bound by the FP64
 // unit: a pair's halo rows cost it more than the second trip through memory
 // (compound sweep 1:3 with pairs against fused passes: 64 systems of 32 .. 80
-// 1129 against 1044 us, 200 of 14 .. 40 529 against 457, 1000 of 14 .. 33 1492
-// against 1270; only 8 of 50 .. 90 330 against 359).  Below 2^19 sites, where a
-// launch is its latency, the pairs' fewer launches stay.
+// 1105 against 1044 us, 20 of 37 .. 90 590 against 558, 200 of 14 .. 40 528 against
+// 457, 1000 of 14 .. 33 1492 against 1270; only 8 of 50 .. 90 318 against 366).
+// Below 2^19 sites the difference is small (30 systems of 14 .. 31 378 against 361,
+// 5 of 22 .. 40 511 against 509) and the default is pairs as in FP32.
 bool batch_pairs_pay(const coulps_batch *B) {
   long long sites = 0;
   for (const auto &S : B->sys) sites += (long long)S.Lx * S.Ly * S.Lz;

@@ -11,9 +11,10 @@
 //
 // Work per sample, all systems at once: the v . phi sums over fixed-size
 // chunks of the batch's field array (one CTA per chunk, chunks never cross a
-// system), one warp per charge for q phi and q^2 phi w, and one warp per
-// system adding its chunks and charges in a fixed order.  The SOR solve is the
-// lattice solver's (sor.cu), so a system's h is the one coulps_gcv_create makes for the same box and charges.
+// system), warps of up to 16 charges (8 in FP64) for q phi and q^2 phi w
+// (charge_local.cuh), and one CTA per system adding its chunks and charges in a
+// fixed order.  The SOR solve is the lattice solver's (sor.cu), so a system's h
+// is the one coulps_gcv_create makes for the same box and charges.
 #include <algorithm>
 #include <cmath>
 #include <cstring>

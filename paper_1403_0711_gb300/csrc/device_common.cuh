@@ -118,7 +118,7 @@ __device__ __forceinline__ V erfcinv_q_tail(V z) {  // z = sqrt(v) - 3.6, v >= 9
 // (fit_erfcinv.py beside this file; fit error 5.5e-9 and 2.9e-8 relative;
 // emulated FP32 evaluation 2.5e-7 relative at most).  The split at v = 9
 // (u < 2^-10 or so, 1e-3 of the words) rather than 7 makes the tail rare
-// enough that a warp's vote over 64 words takes it 6% of the time instead of
+// enough that 64 words of a warp hold one 6% of the time instead of
 // 22%, for one more term in the common polynomial.  Measured against FP64
 // erfc^-1 over the whole range: a few FP32 ulps.
 __device__ __forceinline__ float hb_noise_f32(uint32_t w) {

@@ -48,8 +48,8 @@ __device__ __forceinline__ void qstore<double>(double *p, const Quad<double> &q)
 }
 
 // The heatbath deviates of two quads (two stages' Philox words): FP32 as
-// four packed pairs under one warp vote (every lane of the warp must call
-// it); FP64 word by word.
+// four packed pairs with one branch per thread for the rare tail words; FP64
+// word by word.
 template <typename T> struct StageNoise;
 template <> struct StageNoise<float> {
   __device__ __forceinline__ static void of(uint4 wa, uint4 wb, Quad<float> &na,

@@ -263,7 +263,7 @@ __device__ bool march_pair(const Job &a, const PhiloxKeys &K, unsigned char *sme
     // padding lanes, and so are planes f - 3 .. f
     const bool fast = warp_full && f >= 3 && f < Lz;
     bool got = mbar_wait_bounded(bar_n, par_n);
-    // the heatbath deviates take the whole warp through the same path
+    // a warp makes the heatbath deviates and stage 0 whole or not at all
     if (!A_OR || !B_OR) got = __all_sync(0xffffffffu, got);
     if (!got) {
       atomicOr(err, kErrTimeout);

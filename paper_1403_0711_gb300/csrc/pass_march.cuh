@@ -27,7 +27,7 @@ struct PassLayout {
   int c0_bytes;    // colour-0 box: (TY + 2) rows x W (over-relaxation only)
   int slot_bytes;  // both, each rounded to 128 bytes
   int new_bytes;   // one plane of new colour-0 rows: (TY + 2) x W
-  int total;       // header + 4 slots + 2 new planes
+  int total;       // header + kPassStages slots + 2 new planes
 };
 
 __host__ __device__ inline PassLayout pass_layout(int TY, int W, int es, bool orx) {
@@ -235,7 +235,7 @@ __device__ bool march_pass(const Job &a, const PhiloxKeys &K, unsigned char *sme
     // nothing to zero in either stage
     const bool fast = warp_full && (STEADY || f >= 0) && f < Lz;
     bool got = mbar_wait_bounded(bar_n, par_n);
-    // the heatbath deviates take the whole warp through the same path
+    // a warp makes the heatbath deviates and stage 0 whole or not at all
     if (!OR) got = __all_sync(0xffffffffu, got);
     if (!got) {
       atomicOr(err, kErrTimeout);

@@ -14,7 +14,7 @@ namespace tile {
 // ahead.  A barrier per plane (GROUP = 1) was the heatbath half-sweep's second
 // stall; the single-lattice kernels use 8 slots in groups of 4, the
 // many-system kernel (whose largest systems' slots would cut its occupancy)
-// 4 slots in groups of 1.  At most 8 slots: 8 mbarriers fill the header's
+// 4 slots in groups of 2.  At most 8 slots: 8 mbarriers fill the header's
 // first 64 bytes.
 constexpr int kStages = 4;
 constexpr int kLatticeStages = 8, kLatticeGroup = 4;
