@@ -121,10 +121,11 @@ int coulps_set_resident(coulps_lattice_t lat, int enable);
 /* How compound sweeps of this mix run now: out[0] = CTAs that hold a chain (0:
  * the tiled kernels), out[1] = compound sweeps in a launch (about 0.1 s of them
  * at most; 1 with the tiled kernels), out[2] = 1 if the choice is the library's
- * (coulps_set_resident).  n_sweeps = 0: the measured sweeps of
- * coulps_run; n_sweeps > 0: so many sweeps between two samples that another
- * kernel takes (off-lattice and several sets, control variates), or that many
- * sweeps of coulps_sweep.  Errors: EINVAL. */
+ * (coulps_set_resident).  n_sweeps = 0: the measured sweeps of coulps_run (a
+ * call of one or a few sweeps may still make them by the tiled kernels, with
+ * bitwise the same samples); n_sweeps > 0: so many sweeps between two samples
+ * that another kernel takes (off-lattice and several sets, control variates), or
+ * that many sweeps of coulps_sweep.  Errors: EINVAL. */
 int coulps_resident(coulps_lattice_t lat, int n_hb, int n_or, int n_sweeps, int32_t out[3]);
 
 /* Copy chain `chain`'s field to / from a host array of Lx*Ly*Lz doubles in

@@ -109,6 +109,7 @@ struct coulps_lattice {
   cudaGraphExec_t graph = nullptr;
   const void *graph_key = nullptr;
   int graph_hb = -1, graph_or = -1;
+  bool graph_few = false;  // march sweep, resident sums (resident_few)
   Tile graph_tile = {0, 0};
   // per-kernel event timing
   bool profiling = false;
@@ -584,6 +585,20 @@ Tile march_gather_tile(const coulps_lattice *L, int n_hb, int n_or) {
   return P.singles > 0 ? L->ptile : L->qtile;
 }
 
+// Whether a sampled run of n sweeps that counts as resident is too short for it:
+// a launch's load, store and last sample cost 1 us and 13.7 for each wave of
+// clusters (201 lattices, rms 4.7), a run of one or two sweeps may end sooner as
+// march sweeps with the resident kernel's sums taken from memory, which leave
+// bitwise the same samples.  Taken where clearly so (one sweep a call, us,
+// resident / this way: 40^3 x 100 1:0 56.6 / 38.0, 80^3 x 4 1:3 48.5 / 43.1,
+// 35 x 13 x 81 x 94 1:3 90.7 / 65.2).
+bool resident_few(const coulps_lattice *L, int n_hb, int n_or, int n) {
+  if (n > 8 || resident_on(L, n_hb, n_or, 1)) return false;
+  const int waves = (L->g.n_chains + L->rplan.active - 1) / L->rplan.active;
+  return 1.1 * n * march_time(L->g, n_hb, n_or) <
+         n * resident_time(L->g, L->rplan, n_hb, n_or) + 1.0 + 13.7 * waves;
+}
+
 Tile fused_gather_tile(const coulps_lattice *L, int n_hb, int n_or, int n_sweeps = 0) {
   if (resident_on(L, n_hb, n_or, n_sweeps)) return Tile{L->g.Ly, L->g.Lz};
   return march_gather_tile(L, n_hb, n_or);
@@ -797,10 +812,10 @@ int enqueue_part(coulps_lattice *L, cudaStream_t st, int n_hb, int n_or, coulps_
   return COULPS_OK;
 }
 
-// n_sweeps compound sweeps of every chain (each sampled when `fuse` is given)
-// by the resident kernel, in launches of resident_sweeps.
-int enqueue_resident(coulps_lattice *L, int n_sweeps, int n_hb, int n_or, coulps_charges *fuse) {
-  ResidentArgs a = {};
+// What the resident kernels take of a lattice, and of a charge set staged for
+// them (EINVAL if it is not).
+int resident_args(coulps_lattice *L, int n_hb, int n_or, coulps_charges *fuse, ResidentArgs &a) {
+  a = {};
   const Geometry &g = L->g;
   a.field = L->field;
   a.Lx = g.Lx; a.Ly = g.Ly; a.Lz = g.Lz; a.W = g.W; a.Wq = g.Wq;
@@ -823,12 +838,31 @@ int enqueue_resident(coulps_lattice *L, int n_sweeps, int n_hb, int n_or, coulps
     a.log = fuse->d_log;
     a.log_cap = fuse->log_cap;
   }
+  return COULPS_OK;
+}
+
+// n_sweeps compound sweeps of every chain (each sampled when `fuse` is given)
+// by the resident kernel, in launches of resident_sweeps.
+int enqueue_resident(coulps_lattice *L, int n_sweeps, int n_hb, int n_or, coulps_charges *fuse) {
+  ResidentArgs a;
+  const int st = resident_args(L, n_hb, n_or, fuse, a);
+  if (st) return st;
+  const Geometry &g = L->g;
   const int per = resident_sweeps(L, n_hb, n_or);
   for (int done = 0; done < n_sweeps; done += per) {
     a.n_sweeps = std::min(per, n_sweeps - done);
     CK(launch_resident(g, L->rplan, a, fuse ? fuse->n : 0, L->stream));
     CK(launch_advance_pass(L->d_pass, (uint32_t)a.n_sweeps * (uint32_t)(n_hb + n_or), L->stream));
   }
+  return COULPS_OK;
+}
+
+// One sample of every chain as the resident kernel takes it.
+int enqueue_resident_sample(coulps_lattice *L, coulps_charges *C) {
+  ResidentArgs a;
+  const int st = resident_args(L, 0, 0, C, a);
+  if (st) return st;
+  CK(launch_resident_sample(L->g, L->rplan, a, C->n, L->stream));
   return COULPS_OK;
 }
 
@@ -1810,19 +1844,26 @@ int coulps_run(coulps_lattice_t L, coulps_charges_t C, int n_therm, int n_meas, 
     if (!st) L->pass += (uint64_t)n_meas * P;
     return st;
   }
-  if (fused && resident_on(L, n_hb, n_or)) {
+  const bool res = fused && resident_on(L, n_hb, n_or);
+  const bool few = res && resident_few(L, n_hb, n_or, n_meas);
+  if (res && !few) {
     st = enqueue_resident(L, n_meas, n_hb, n_or, C);
     if (!st) L->pass += (uint64_t)n_meas * P;
     return st;
   }
   const bool capturable = L->stream != nullptr && !L->profiling;
+  // one measured sweep: the sample in its last kernel, or after it
+  auto one = [&]() -> int {
+    int s1 = enqueue_compound(L, n_hb, n_or, fused && !few ? C : nullptr);
+    if (s1 || (fused && !few)) return s1;
+    return few ? enqueue_resident_sample(L, C) : enqueue_measure(L, C);
+  };
   if (capturable && (L->graph_key != C || L->graph_hb != n_hb || L->graph_or != n_or ||
-                     L->graph_tile.ty != L->tile.ty || L->graph_tile.dz != L->tile.dz)) {
+                     L->graph_few != few || L->graph_tile.ty != L->tile.ty || L->graph_tile.dz != L->tile.dz)) {
     drop_graph(L);
     cudaGraph_t gr = nullptr;
     CK(cudaStreamBeginCapture(L->stream, cudaStreamCaptureModeThreadLocal));
-    int s1 = enqueue_compound(L, n_hb, n_or, fused ? C : nullptr);
-    int s2 = s1 ? s1 : (fused ? COULPS_OK : enqueue_measure(L, C));
+    const int s2 = one();
     cudaError_t e = cudaStreamEndCapture(L->stream, &gr);
     if (s2 || e != cudaSuccess) {
       cudaGetLastError();
@@ -1839,14 +1880,14 @@ int coulps_run(coulps_lattice_t L, coulps_charges_t C, int n_therm, int n_meas, 
     L->graph_key = C;
     L->graph_hb = n_hb;
     L->graph_or = n_or;
+    L->graph_few = few;
     L->graph_tile = L->tile;
   }
   for (int k = 0; k < n_meas; ++k) {
     if (capturable) {
       CK(cudaGraphLaunch(L->graph, L->stream));
     } else {
-      st = enqueue_compound(L, n_hb, n_or, fused ? C : nullptr);
-      if (!st && !fused) st = enqueue_measure(L, C);
+      st = one();
       if (st) return st;
     }
     L->pass += (uint64_t)(n_hb + n_or);

@@ -174,6 +174,9 @@ struct ResidentPlan {
 bool resident_shape(const Geometry &g, int C, ResidentPlan *p);
 // Estimated time (us) of a compound sweep of every chain.
 double resident_time(const Geometry &g, const ResidentPlan &p, int n_hb, int n_or);
+// One sample of every chain from the fields in memory, bitwise launch_resident's.
+cudaError_t launch_resident_sample(const Geometry &g, const ResidentPlan &p, ResidentArgs a,
+                                   int64_t n_q, cudaStream_t s);
 // n_q: charges of the measured set (0 without)
 cudaError_t launch_resident(const Geometry &g, const ResidentPlan &p, ResidentArgs a, int64_t n_q,
                             cudaStream_t s);

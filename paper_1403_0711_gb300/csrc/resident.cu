@@ -165,6 +165,44 @@ template <> struct Draw<1> {
   }
 };
 
+// A sample's sums, here and in resident_sample_kernel: the same order, and
+// explicit roundings, so that a contraction does not depend on the kernel.
+__device__ __forceinline__ void add_charge(double q, double phi, double &sq, double &sp) {
+  const double t = __dmul_rn(q, phi);
+  sq = __dadd_rn(sq, t);
+  sp = __fma_rn(t, t, sp);
+}
+// sums of a warp whose first `n` lanes hold something
+__device__ __forceinline__ void add_lanes(uint32_t n, double &a, double &b) {
+  for (uint32_t o = 16; o > 0; o >>= 1)
+    if (o < n) {
+      a = __dadd_rn(a, __shfl_xor_sync(0xffffffffu, a, o));
+      b = __dadd_rn(b, __shfl_xor_sync(0xffffffffu, b, o));
+    }
+}
+// the n measuring warps' sums, by a warp
+__device__ __forceinline__ void add_parts(const double *part, int n, int lane, double &Q, double &P) {
+  Q = P = 0.0;
+  for (int r = lane; r < n; r += 32) {
+    Q = __dadd_rn(Q, part[2 * r]);
+    P = __dadd_rn(P, part[2 * r + 1]);
+  }
+  add_lanes((uint32_t)n, Q, P);
+}
+// e = Q^2 - P into a chain's running sums `st` and batch sums, and the log
+__device__ __forceinline__ void record_sums(const ResidentArgs &a, int chain, double Q, double P,
+                                            double *st, double *batch) {
+  const double e = __fma_rn(Q, Q, -P);
+  const int64_t n = (int64_t)st[kStatN];
+  if (a.log != nullptr && n < a.log_cap) {
+    double *row = a.log + 3 * ((size_t)n * a.n_chains + chain);
+    row[0] = Q;
+    row[1] = P;
+    row[2] = e;
+  }
+  record_value(st, batch, e, a.err);
+}
+
 template <typename T, int V, bool SINGLE>
 __global__ void __launch_bounds__(kMaxSweepThreads + kMeasThreads, 1)
     resident_kernel(const ResidentArgs a) {
@@ -452,31 +490,11 @@ __global__ void __launch_bounds__(kMaxSweepThreads + kMeasThreads, 1)
       double Q = 0.0, P = 0.0;
       bool pending = false;
       auto sum = [&]() {
-        const int n = C * a.meas_warps;
-        Q = P = 0.0;
-        for (int r = lane; r < n; r += 32) {
-          Q += part[2 * r];
-          P += part[2 * r + 1];
-        }
-        for (int o = 16; o > 0; o >>= 1)
-          if (o < n) {
-            Q += __shfl_xor_sync(0xffffffffu, Q, o);
-            P += __shfl_xor_sync(0xffffffffu, P, o);
-          }
+        add_parts(part, C * a.meas_warps, lane, Q, P);
         pending = true;
       };
       auto record = [&]() {
-        if (lane == 0 && pending) {
-          const double e = Q * Q - P;
-          const int64_t n = (int64_t)run_st[kStatN];
-          if (a.log != nullptr && n < a.log_cap) {
-            double *row = a.log + 3 * ((size_t)n * a.n_chains + chain);
-            row[0] = Q;
-            row[1] = P;
-            row[2] = e;
-          }
-          record_value(run_st, st + kStatBatch0, e, a.err);
-        }
+        if (lane == 0 && pending) record_sums(a, chain, Q, P, run_st, st + kStatBatch0);
         pending = false;
       };
       const int at_half = n_half > 2 ? 2 : 0;
@@ -532,18 +550,13 @@ __global__ void __launch_bounds__(kMaxSweepThreads + kMeasThreads, 1)
 #pragma unroll
         for (int k = 0; k < kResEntries; ++k) {
           const uint32_t e = e0 + (uint32_t)k * stride;
-          if (e < e1 && (at[k] >> 31) == c) {
-            const double t = q[k] * (double)planes[at[k] & ~kGatherColourBit];
-            sq += t;
-            sp += t * t;
-          }
+          if (e < e1 && (at[k] >> 31) == c)
+            add_charge(q[k], (double)planes[at[k] & ~kGatherColourBit], sq, sp);
         }
         for (uint32_t e = e0 + (uint32_t)kResEntries * stride; e < e1; e += stride) {
           const uint32_t ent = a.g_ent[e];
-          if ((ent >> 31) != c) continue;
-          const double t = a.g_q[e] * (double)planes[place(ent) & ~kGatherColourBit];
-          sq += t;
-          sp += t * t;
+          if ((ent >> 31) == c)
+            add_charge(a.g_q[e], (double)planes[place(ent) & ~kGatherColourBit], sq, sp);
         }
       };
       // this warp's sums to CTA 0's shared memory (the slots of warps without
@@ -553,11 +566,7 @@ __global__ void __launch_bounds__(kMaxSweepThreads + kMeasThreads, 1)
       const uint32_t to_cta0 = C > 1 ? map_rank(to, 0u) : 0u;
       auto send = [&]() {
         if (top == 0u) return;
-        for (int o = 16; o > 0; o >>= 1)
-          if ((uint32_t)o < top) {
-            sq += __shfl_xor_sync(0xffffffffu, sq, o);
-            sp += __shfl_xor_sync(0xffffffffu, sp, o);
-          }
+        add_lanes(top, sq, sp);
         if (lane == 0) {
           if (C > 1) {
             const double vq[1] = {sq}, vp[1] = {sp};
@@ -606,6 +615,57 @@ __global__ void __launch_bounds__(kMaxSweepThreads + kMeasThreads, 1)
   if (measure && rank == 0)
     for (int i = tid; i < kStatStride; i += blockDim.x)
       a.stats[(size_t)chain * kStatStride + i] = st[i];
+}
+
+// One sample of every chain from the fields in memory, bitwise the resident
+// kernel's: its warps' charges, their order and its additions.  For runs of so
+// few sweeps that the march kernels make them sooner.  A CTA per chain, bound by
+// its chain of dependent loads and sums; with 8 warps instead of 16 the sums of 12
+// measuring warps take two rounds and a sweep 40.2 instead of 38.0 us (40^3 x 100).
+constexpr int kSampleThreads = 512;
+template <typename T>
+__global__ void __launch_bounds__(kSampleThreads) resident_sample_kernel(const ResidentArgs a) {
+  __shared__ double part[2 * kResParts];
+  const int chain = blockIdx.x, lane = threadIdx.x & 31;
+  const T *f = reinterpret_cast<const T *>(a.field) + (size_t)chain * a.chain_elems;
+  const int slots = a.cluster * a.meas_warps;
+  const uint32_t stride = 32u * (uint32_t)a.meas_warps;
+  for (int s = threadIdx.x >> 5; s < slots; s += kSampleThreads / 32) {
+    const int rank = s / a.meas_warps, w = s - rank * a.meas_warps;
+    const int z0 = (int)((int64_t)a.Lz * rank / a.cluster),
+              z1 = (int)((int64_t)a.Lz * (rank + 1) / a.cluster);
+    const uint32_t first = a.g_off[z0] + (uint32_t)(32 * w), e1 = a.g_off[z1];
+    double sq = 0.0, sp = 0.0;
+    for (uint32_t c = 0; c < 2; ++c)
+      for (uint32_t e0 = first + (uint32_t)lane; e0 < e1; e0 += 4u * stride) {
+        // four charges' loads at a time, added in order
+        double q[4], phi[4];
+        bool in[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const uint32_t e = e0 + (uint32_t)k * stride;
+          const uint32_t ent = e < e1 ? a.g_ent[e] : 0u;
+          in[k] = e < e1 && (ent >> 31) == c;
+          q[k] = in[k] ? a.g_q[e] : 0.0;
+          phi[k] = in[k] ? (double)f[(size_t)c * a.colour_elems + (ent & ~kGatherColourBit)] : 0.0;
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          if (in[k]) add_charge(q[k], phi[k], sq, sp);
+      }
+    add_lanes(e1 > first ? e1 - first : 0u, sq, sp);
+    if (lane == 0) {
+      part[2 * s] = sq;
+      part[2 * s + 1] = sp;
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    double Q, P;
+    add_parts(part, slots, lane, Q, P);
+    double *st = a.stats + (size_t)chain * kStatStride;
+    if (lane == 0) record_sums(a, chain, Q, P, st, st + kStatBatch0);
+  }
 }
 
 size_t resident_smem(const Geometry &g, int C, bool single) {
@@ -722,12 +782,27 @@ double resident_time(const Geometry &g, const ResidentPlan &p, int n_hb, int n_o
   return waves * (n_half * barrier + work);
 }
 
+// one measuring warp where each CTA has few charges
+static int measuring_warps(const ResidentPlan &p, int64_t n_q) {
+  return n_q <= 16 * (int64_t)p.cluster ? 1 : kGatherWarps;
+}
+
+cudaError_t launch_resident_sample(const Geometry &g, const ResidentPlan &p, ResidentArgs a,
+                                   int64_t n_q, cudaStream_t s) {
+  a.cluster = p.cluster;
+  a.meas_warps = measuring_warps(p, n_q);
+  if (g.precision == COULPS_F32)
+    resident_sample_kernel<float><<<g.n_chains, kSampleThreads, 0, s>>>(a);
+  else
+    resident_sample_kernel<double><<<g.n_chains, kSampleThreads, 0, s>>>(a);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_resident(const Geometry &g, const ResidentPlan &p, ResidentArgs a, int64_t n_q,
                             cudaStream_t s) {
   a.cluster = p.cluster;
   a.run = p.run;
-  // one measuring warp where each CTA has few charges
-  a.meas_warps = n_q <= 16 * (int64_t)p.cluster ? 1 : kGatherWarps;
+  a.meas_warps = measuring_warps(p, n_q);
   const bool f32 = g.precision == COULPS_F32;
   if (p.single)
     return f32 ? launch_t<float, 4, true>(g, p, a, s) : launch_t<double, 1, true>(g, p, a, s);
