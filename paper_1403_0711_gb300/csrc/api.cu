@@ -319,6 +319,32 @@ Tile fill_grid(const Geometry &g, Tile t, int target, int min_dz) {
   return t;
 }
 
+struct TileRows {  // what the rows of a tile decide
+  int threads, box_rows, per_sm;
+  size_t smem;
+  int64_t ny;
+};
+TileRows tile_rows(const Geometry &g, MarchKind kind, int ty) {
+  const bool f64 = g.precision == COULPS_F64;
+  const int qw = g.W / 4;
+  const Tile t{ty, 1};  // shared memory and threads do not depend on the planes
+  TileRows r;
+  if (kind == kMarchPair) {
+    r.threads = pair_threads(g, t); r.box_rows = 2 * ty + 14; r.smem = pair_smem_bytes(g, t, true);
+  } else if (kind == kMarchPass) {
+    r.threads = pass_threads(g, t); r.box_rows = 2 * ty + 6; r.smem = pass_smem_bytes(g, t, true);
+  } else {
+    // heatbath (FP32: two quads per thread); the other colour only
+    r.threads = ((f64 ? qw : (qw + 1) / 2) * ty + 31) / 32 * 32; r.box_rows = ty + 2;
+    r.smem = halfsweep_smem_bytes(g, t, false);
+  }
+  r.per_sm = std::max(1, std::min(std::min(65536 / (kTileCost[kind][f64 ? 1 : 0].regs * r.threads),
+                                           2048 / r.threads),
+                                  std::min((int)(228 * 1024 / (r.smem + 1024)), 32)));
+  r.ny = (g.Ly + ty - 1) / ty;
+  return r;
+}
+
 // Time of one launch over all chains (us) of a march kernel with this tile,
 // as far as the tile decides it.  CTAs run in waves of as many as an SM holds
 // (registers, shared memory, threads); a wave takes its steps (planes and
@@ -326,42 +352,29 @@ Tile fill_grid(const Geometry &g, Tile t, int target, int min_dz) {
 // SM's warps and its TMA rows, and a start; the launch is no shorter than its
 // reads (with the halo) and writes take (joined as cubes: neither hides the
 // other fully near the line).
-double tile_time(const Geometry &g, MarchKind kind, const Tile &t, int sms,
+// A time of `most` or more may come back as `most`.
+double tile_time(const Geometry &g, MarchKind kind, const TileRows &r, int dz, int sms, double most,
                  int64_t *full_waves = nullptr) {
-  const bool f64 = g.precision == COULPS_F64;
-  const TileCost &k = kTileCost[kind][f64 ? 1 : 0];
+  const TileCost &k = kTileCost[kind][g.precision == COULPS_F64 ? 1 : 0];
   const double row_bytes = (double)g.W * g.es;
-  const int qw = g.W / 4;
-  int threads, steps, planes, box_rows;
-  size_t smem;
-  if (kind == kMarchPair) {
-    threads = pair_threads(g, t); steps = t.dz + 6; planes = 8; box_rows = 2 * t.ty + 14;
-    smem = pair_smem_bytes(g, t, true);
-  } else if (kind == kMarchPass) {
-    threads = pass_threads(g, t); steps = t.dz + 2; planes = 4; box_rows = 2 * t.ty + 6;
-    smem = pass_smem_bytes(g, t, true);
-  } else {
-    // heatbath (FP32: two quads per thread); the other colour only
-    threads = ((f64 ? qw : (qw + 1) / 2) * t.ty + 31) / 32 * 32; steps = t.dz + 2; planes = 2;
-    box_rows = t.ty + 2;
-    smem = halfsweep_smem_bytes(g, t, false);
-  }
-  const int per_sm = std::max(1, std::min(std::min(65536 / (k.regs * threads), 2048 / threads),
-                                          std::min((int)(228 * 1024 / (smem + 1024)), 32)));
-  const int64_t ny = (g.Ly + t.ty - 1) / t.ty, nz = (g.Lz + t.dz - 1) / t.dz;
-  const int64_t ctas = ny * nz * g.n_chains, full = ctas / ((int64_t)sms * per_sm);
-  const int64_t rest = (ctas - full * sms * per_sm + sms - 1) / sms;
-  if (full_waves) *full_waves = full;
-  auto wave = [&](int64_t n) {
-    return steps * std::max(k.step, (double)n * std::max(threads / 32 * k.warp, box_rows * k.row)) +
-           k.wave + k.cta * (double)n;
-  };
-  const double work = (double)full * wave(per_sm) + (rest > 0 ? wave(rest) : 0.0);
+  const int planes = kind == kMarchPair ? 8 : (kind == kMarchPass ? 4 : 2);
+  const int steps = dz + (kind == kMarchPair ? 6 : 2);
+  const int64_t nz = (g.Lz + dz - 1) / dz;
   const double volume = row_bytes * g.Ly * g.Lz * g.n_chains;
   const double traffic =
-      row_bytes * box_rows * (double)(ny * g.n_chains) * (double)(g.Lz + nz * planes) +
+      row_bytes * r.box_rows * (double)(r.ny * g.n_chains) * (double)(g.Lz + nz * planes) +
       volume * (kind == kMarchHalf ? 1.0 : 2.0);
   const double mem = traffic / k.bytes;
+  if (mem + 4.0 >= most) return most;
+  const int64_t ctas = r.ny * nz * g.n_chains, full = ctas / ((int64_t)sms * r.per_sm);
+  const int64_t rest = (ctas - full * sms * r.per_sm + sms - 1) / sms;
+  if (full_waves) *full_waves = full;
+  auto wave = [&](int64_t n) {
+    return steps * std::max(k.step, (double)n * std::max(r.threads / 32 * k.warp, r.box_rows * k.row)) +
+           k.wave + k.cta * (double)n;
+  };
+  const double work = (double)full * wave(r.per_sm) + (rest > 0 ? wave(rest) : 0.0);
+  if (work + 4.0 >= most) return most;
   return std::cbrt(work * work * work + mem * mem * mem) + 4.0;
 }
 
@@ -390,37 +403,25 @@ Tile best_tile(const Geometry &g, MarchKind kind, Tile t, int sms, double clear)
   const int halo = kind == kMarchPair ? 6 : (kind == kMarchPass ? 2 : 0);
   const int ty_max = std::min(std::min(threads / qw - halo, g.Ly), 248);
   int64_t waves = 0;
-  double best = clear * tile_time(g, kind, t, sms, &waves);
+  double best = clear * tile_time(g, kind, tile_rows(g, kind, t.ty), t.dz, sms, 1e30, &waves);
   if (waves >= 5) return t;
   Tile out = t;
-  int last_ty = 0;
-  for (int ny = 1; ny <= g.Ly; ++ny) {
-    int ty = (g.Ly + ny - 1) / ny;
-    if (ty > ty_max) {
-      if ((g.Ly + ny) / (ny + 1) > ty_max) continue;
-      ty = ty_max;  // the most rows that fit, ahead of the first even division
-    }
-    if (ty < 2 || ty == last_ty) continue;
-    last_ty = ty;
-    int last_dz = 0;
-    for (int nz = 1; nz <= g.Lz; ++nz) {
-      int dz = (g.Lz + nz - 1) / nz;
-      if (kind == kMarchHalf) {
-        if (nz > 4) break;
-        dz = 4 * nz;
-      }
-      if (dz < 4) break;
-      if (dz == last_dz || dz > g.Lz) continue;
-      last_dz = dz;
-      const Tile c{ty, dz};
-      const size_t smem = kind == kMarchPair   ? pair_smem_bytes(g, c, true)
-                          : kind == kMarchPass ? pass_smem_bytes(g, c, true)
-                                               : halfsweep_smem_bytes(g, c, true);
-      if (smem > 227 * 1024) continue;
-      const double e = tile_time(g, kind, c, sms);
+  // the next smaller even division of n
+  auto next = [](int n, int part) {
+    const int k = (n + part - 2) / (part - 1);
+    return (n + k - 1) / k;
+  };
+  for (int ty = ty_max; ty >= 2; ty = next(g.Ly, ty)) {
+    const TileRows r = tile_rows(g, kind, ty);
+    const size_t smem = kind == kMarchHalf ? halfsweep_smem_bytes(g, Tile{ty, 1}, true) : r.smem;
+    if (smem > 227 * 1024) continue;
+    for (int dz = kind == kMarchHalf ? 4 : g.Lz; dz >= 4 && dz <= g.Lz;
+         dz = kind == kMarchHalf ? dz + 4 : next(g.Lz, dz)) {
+      if (kind == kMarchHalf && dz > 16) break;
+      const double e = tile_time(g, kind, r, dz, sms, best);
       if (e < best) {
         best = e;
-        out = c;
+        out = Tile{ty, dz};
       }
     }
   }
@@ -431,13 +432,31 @@ Tile best_tile(const Geometry &g, MarchKind kind, Tile t, int sms, double clear)
 // sweep of 1 heatbath : 3 over-relaxation passes; {cluster = 0} if the chain
 // fits no cluster.
 ResidentPlan resident_plan(const Geometry &g) {
-  ResidentPlan best;
-  double t_best = 0.0;
+  // The number of clusters that the GPU holds is a query of the driver each: the
+  // sizes in the order of their times with the most clusters that SMs and shared
+  // memory allow, as far as these stay below the best time found.
+  struct Candidate {
+    double least;
+    ResidentPlan p;
+  };
+  Candidate c[kMaxCluster];
+  int n = 0;
+  const int sms = device_sms();
   for (int C = 1; C <= kMaxCluster && C <= g.Lz; ++C) {
     ResidentPlan p;
     if (!resident_shape(g, C, &p)) continue;
+    p.active = std::max(1, sms * resident_per_sm(p) / C);
+    c[n].p = p;
+    c[n++].least = resident_time(g, p, 1, 3);
+  }
+  std::stable_sort(c, c + n, [](const Candidate &x, const Candidate &y) { return x.least < y.least; });
+  ResidentPlan best;
+  double t_best = 0.0;
+  for (int i = 0; i < n && (best.cluster == 0 || c[i].least <= t_best); ++i) {
+    ResidentPlan &p = c[i].p;
+    if (!resident_active(g, &p)) continue;
     const double t = resident_time(g, p, 1, 3);
-    if (best.cluster == 0 || t < t_best) {
+    if (best.cluster == 0 || t < t_best || (t == t_best && p.cluster < best.cluster)) {
       t_best = t;
       best = p;
     }

@@ -170,8 +170,12 @@ struct ResidentPlan {
   size_t smem = 0;
   double steps = 0.0;  // steps of a thread per half-sweep
 };
-// The plan with clusters of C CTAs; false if the chain does not fit them.
+// The plan with clusters of C CTAs, without `active`; false if the chain does not
+// fit them.
 bool resident_shape(const Geometry &g, int C, ResidentPlan *p);
+int resident_per_sm(const ResidentPlan &p);  // CTAs of an SM at most
+// Asks the driver for `active`; false if the GPU cannot hold one cluster.
+bool resident_active(const Geometry &g, ResidentPlan *p);
 // Estimated time (us) of a compound sweep of every chain.
 double resident_time(const Geometry &g, const ResidentPlan &p, int n_hb, int n_or);
 // One sample of every chain from the fields in memory, bitwise launch_resident's.

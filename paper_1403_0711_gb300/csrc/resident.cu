@@ -755,6 +755,15 @@ bool resident_shape(const Geometry &g, int C, ResidentPlan *p) {
       p->run = r;
     }
   }
+  return true;
+}
+
+int resident_per_sm(const ResidentPlan &p) {
+  return std::min(2048 / resident_block(p), (int)(228 * 1024 / (p.smem + 1024)));
+}
+
+bool resident_active(const Geometry &g, ResidentPlan *p) {
+  const bool f32 = g.precision == COULPS_F32;
   if (p->single)
     p->active = f32 ? active_clusters_t<float, 4, true>(*p) : active_clusters_t<double, 1, true>(*p);
   else
