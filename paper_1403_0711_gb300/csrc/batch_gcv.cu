@@ -11,8 +11,8 @@
 //
 // Work per sample, all systems at once: the v . phi sums over fixed-size
 // chunks of the batch's field array (one CTA per chunk, chunks never cross a
-// system), warps of up to 16 charges (8 in FP64) for q phi and q^2 phi w
-// (charge_local.cuh), and one CTA per system adding its chunks and charges in a
+// system), warps of up to 16 charges (8 in FP64), or of one where that is the
+// better way, for q phi and q^2 phi w (charge_local.cuh), and one CTA per system adding its chunks and charges in a
 // fixed order.  The SOR solve is the lattice solver's (sor.cu), so a system's h
 // is the one coulps_gcv_create makes for the same box and charges.
 #include <algorithm>
@@ -228,6 +228,29 @@ __global__ void __launch_bounds__(32 * kBgcvWarps, 4)
   }
 }
 
+// the same by a warp per charge (direct_sum)
+template <typename T>
+__global__ void __launch_bounds__(32 * kBgcvWarps)
+    bgcv_charge_direct_kernel(const T *__restrict__ field, const BgcvSystem *__restrict__ sys,
+                              const int4 *__restrict__ qsite, const double *__restrict__ q,
+                              int64_t n_q, const float *__restrict__ kt, int R,
+                              double *__restrict__ out) {
+  const int lane = threadIdx.x & 31;
+  const int64_t warps = (int64_t)gridDim.x * kBgcvWarps;
+  for (int64_t i = (int64_t)blockIdx.x * kBgcvWarps + (threadIdx.x >> 5); i < n_q; i += warps) {
+    const int4 r = __ldg(qsite + i);
+    const double qi = __ldg(q + i);
+    const BgcvSystem S = sys[r.w];
+    const LocalBox<T> b{field + S.field_off, (size_t)S.colour_elems, S.Lx, S.Ly, S.Lz, S.W};
+    const double p = (double)box_phi(b, r.x, r.y, r.z);
+    const double w = direct_sum(b, r.x, r.y, r.z, R, kt, lane);
+    if (lane == 0) {
+      out[2 * i] = qi * p;
+      out[2 * i + 1] = qi * qi * p * w;
+    }
+  }
+}
+
 // R = 0: out[2 i] = q_i phi(r_i), out[2 i + 1] = 0 (thread per charge)
 template <typename T>
 __global__ void bgcv_charge0_kernel(const T *__restrict__ field, const BgcvSystem *__restrict__ sys,
@@ -328,11 +351,28 @@ void drop_graph(coulps_batch_gcv *G) {
 
 // q phi and the local P term of every charge: persistent warps (8 per block,
 // 8 blocks per SM)
+// Whether a warp takes one charge for itself, as in the lattice's evaluation
+// (gcv_direct in gcv.cu).  Evaluation hot / cold, us, neighbourhoods against direct:
+// 64 systems of 32 .. 80 with 20 charges each, R = 1 36 / 49 against 31 / 44, with
+// 1500 91 / 104 against 99 / 108; 200 of 20 x 24 x 30 with 1500, R = 4 1345 / 1355
+// against 1410 / 1420, FP64 4040 / 4084 against 3280 / 3290.
+bool bgcv_direct(const coulps_batch_gcv *G) {
+  if (G->B->precision == COULPS_F64 && G->R >= 3) return true;
+  return G->n_q < ((int64_t)20000 << G->R);
+}
+
 template <typename T>
 cudaError_t launch_charge(coulps_batch_gcv *G, const T *field, cudaStream_t st) {
   if (G->R == 0) {
     bgcv_charge0_kernel<T><<<(int)((G->n_q + 255) / 256), 256, 0, st>>>(
         field, G->d_sys, G->d_qsite, G->d_q, G->n_q, G->d_qpart);
+    return cudaGetLastError();
+  }
+  if (bgcv_direct(G)) {
+    const int blocks = (int)std::min<int64_t>((G->n_q + kBgcvWarps - 1) / kBgcvWarps,
+                                              (int64_t)G->sms * 8);
+    bgcv_charge_direct_kernel<T><<<blocks, 32 * kBgcvWarps, 0, st>>>(
+        field, G->d_sys, G->d_qsite, G->d_q, G->n_q, G->d_k, G->R, G->d_qpart);
     return cudaGetLastError();
   }
   const int m = 2 * G->R + 1, n_pts = m * m * (m + 6);

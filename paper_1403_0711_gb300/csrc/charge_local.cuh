@@ -25,6 +25,37 @@ struct LocalBox {
   int Lx, Ly, Lz, W;
 };
 
+// phi at a site, 0 outside the box
+template <typename T>
+__device__ __forceinline__ T box_phi(const LocalBox<T> &b, int x, int y, int z) {
+  if ((unsigned)x >= (unsigned)b.Lx || (unsigned)y >= (unsigned)b.Ly || (unsigned)z >= (unsigned)b.Lz)
+    return T(0);
+  return b.f[((x + y + z) & 1 ? b.ce : (size_t)0) + ((size_t)z * b.Ly + y) * b.W + (x >> 1)];
+}
+
+// w of the charge at (x, y, z) in every lane, by a warp for itself: lane t takes the
+// points t, t + 32, .. of the cube and loads each with its six neighbours.  No shared
+// memory and no charge waits for another: for few charges, and for FP64 and cubes so
+// large that their neighbourhoods leave an SM few warps.
+template <typename T>
+__device__ __forceinline__ double direct_sum(const LocalBox<T> &b, int x, int y, int z, int R,
+                                             const float *kt, int lane) {
+  const int m = 2 * R + 1, m3 = m * m * m;
+  T w = T(0);
+  for (int t = lane; t < m3; t += 32) {
+    const int xx = x + t % m - R, yy = y + (t / m) % m - R, zz = z + t / (m * m) - R;
+    if ((unsigned)xx >= (unsigned)b.Lx || (unsigned)yy >= (unsigned)b.Ly ||
+        (unsigned)zz >= (unsigned)b.Lz)
+      continue;
+    const T Ap = T(6) * box_phi(b, xx, yy, zz) - box_phi(b, xx - 1, yy, zz) -
+                 box_phi(b, xx + 1, yy, zz) - box_phi(b, xx, yy - 1, zz) -
+                 box_phi(b, xx, yy + 1, zz) - box_phi(b, xx, yy, zz - 1) -
+                 box_phi(b, xx, yy, zz + 1);
+    w += (T)__ldg(kt + t) * Ap;
+  }
+  return warp_sum((double)w);
+}
+
 // Shared memory of a CTA of `warps` warps with at most `charges` charges a warp:
 // per warp the neighbourhoods of two charges ((2R + 3)^3 each) and the lanes'
 // shares [charge][33], then the cube's points (offsets in such a neighbourhood),

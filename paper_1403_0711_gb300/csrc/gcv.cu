@@ -172,7 +172,8 @@ __global__ void gcv_v_kernel(const float *__restrict__ h32, Geometry g, float *_
 // load, and those, not DRAM, were the time; through shared memory by bulk
 // copies 113 us, its barriers and v's latency in the way).
 //
-// Local term: charge_local.cuh, up to kEvalCharges charges of a chain a warp.
+// Local term: charge_local.cuh, up to kEvalCharges charges of a chain a warp, or a
+// warp a charge (gcv_direct).
 //
 // Measured, evaluation of 128^3 x 64 chains, 4096 charges (cold L2, the finish
 // kernel included): R = 1 313 -> 243 us, R = 0 144 -> 116.  v . phi is near its
@@ -315,23 +316,59 @@ __device__ __forceinline__ void eval_local(const Geometry &g, const EvalArgs &A,
   }
 }
 
+// The local term by a warp per charge (direct_sum).
 template <typename T>
-__global__ void __launch_bounds__(kGcvThreads, 4)
+__device__ __forceinline__ void eval_direct(const Geometry &g, const EvalArgs &A, int chain, int pb) {
+  const T *f = reinterpret_cast<const T *>(A.field) + (size_t)chain * g.chain_elems;
+  const LocalBox<T> box{f, g.colour_elems, g.Lx, g.Ly, g.Lz, g.W};
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int64_t i = (int64_t)pb * kEvalWarps + wid;
+  double contrib = 0.0;
+  if (i < A.n_q) {
+    const uint32_t e = A.idx[i], ce = (uint32_t)g.colour_elems;
+    const int c = e >= ce ? 1 : 0;
+    const uint32_t r = e - (c ? ce : 0u), row = r / (uint32_t)g.W;
+    const int z = (int)(row / (uint32_t)g.Ly), y = (int)(row - (uint32_t)z * (uint32_t)g.Ly),
+              x = 2 * (int)(r - row * (uint32_t)g.W) + ((c + y + z) & 1);
+    const double qi = A.q[i];
+    contrib = qi * qi * (double)f[e] * direct_sum(box, x, y, z, A.R, A.kt, lane);
+  }
+  __shared__ double red[kEvalWarps];
+  if (lane == 0) red[wid] = contrib;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double sum = 0.0;
+    for (int k = 0; k < kEvalWarps; ++k) sum += red[k];
+    A.ppart[(size_t)chain * A.nblk_p + pb] = sum;
+  }
+}
+
+// (direct: five CTAs per SM, 48 registers; with four FP64 96^3 x 16, 200 charges,
+// R = 2 takes 100 instead of 88 us, 128^3 x 2, R = 4 59 instead of 47)
+template <typename T, bool DIRECT>
+__global__ void __launch_bounds__(kGcvThreads, DIRECT ? 5 : 4)
     gcv_eval_kernel(const Geometry g, const EvalArgs A) {
   extern __shared__ __align__(128) unsigned char smem[];
   const int pb = (int)blockIdx.x - A.nblk;
   if (pb < 0)
     eval_dot<T>(g, A, blockIdx.y);
+  else if (DIRECT)
+    eval_direct<T>(g, A, blockIdx.y, pb);
   else
     eval_local<T>(g, A, blockIdx.y, pb, smem);
 }
 
 template <typename T>
-cudaError_t launch_eval(const Geometry &g, const EvalArgs &A, cudaStream_t s) {
-  const size_t smem = A.nblk_p > 0 ? local_bytes<T>(kEvalWarps, kEvalCharges<T>, A.R, A.n_pts) : (size_t)0;
-  const cudaError_t e = raise_smem((const void *)gcv_eval_kernel<T>, smem);
+cudaError_t launch_eval(const Geometry &g, const EvalArgs &A, bool direct, cudaStream_t s) {
+  const dim3 grid(A.nblk + A.nblk_p, g.n_chains);
+  if (direct || A.nblk_p == 0) {
+    gcv_eval_kernel<T, true><<<grid, kGcvThreads, 0, s>>>(g, A);
+    return cudaGetLastError();
+  }
+  const size_t smem = local_bytes<T>(kEvalWarps, kEvalCharges<T>, A.R, A.n_pts);
+  const cudaError_t e = raise_smem((const void *)gcv_eval_kernel<T, false>, smem);
   if (e != cudaSuccess) return e;
-  gcv_eval_kernel<T><<<dim3(A.nblk + A.nblk_p, g.n_chains), kGcvThreads, smem, s>>>(g, A);
+  gcv_eval_kernel<T, false><<<grid, kGcvThreads, smem, s>>>(g, A);
   return cudaGetLastError();
 }
 
@@ -415,6 +452,20 @@ cudaError_t gcv_solve(const Geometry &g, int64_t n_q, const int32_t *sites, cons
   return cudaGetLastError();
 }
 
+// Whether a warp takes one charge for itself (eval_direct).  What the shared
+// neighbourhoods save, accesses to L1, counts only where there are charges enough to
+// fill the GPU, and their shared memory leaves an SM few warps from R = 4 (FP32) or 2
+// (FP64) on, also for v . phi.  Evaluation hot / cold, us, neighbourhoods against
+// direct: 64^3 x 4, 200 charges, R = 2 14.5 / 19.1 against 12.4 / 16.0; 128^3 x 64,
+// 1000 charges, R = 1 133 / 143 against 145 / 152, R = 4 604 / 612 against 388 / 393;
+// FP64 96^3 x 16, 1000 charges, R = 4 409 / 416 against 258 / 261, R = 1, 4096 charges
+// 126 / 135 against 158 / 160.
+static bool gcv_direct(const Geometry &g, int R, int64_t n_q) {
+  const int64_t n = n_q * g.n_chains;
+  if (g.precision == COULPS_F32) return R >= 4 || n < ((int64_t)12000 << R);
+  return R >= 2 || n < 10000;
+}
+
 cudaError_t gcv_eval(const Geometry &g, const void *field, const float *v_layout,
                      const uint32_t *idx, const double *q, int64_t n_q, double *partials,
                      int nblk, const double *c0, const float *kt, int R, double cP,
@@ -434,17 +485,18 @@ cudaError_t gcv_eval(const Geometry &g, const void *field, const float *v_layout
   A.per = 1;
   const int m = 2 * R + 1;
   A.n_pts = m * m * (m + 6);
+  const bool direct = R > 0 && gcv_direct(g, R, n_q);
   if (R > 0 && n_q > 0) {
-    // as many charges a warp as leave 32 warps for each of 152 SMs (evaluation of
+    // neighbourhoods: as many charges a warp as leave 32 warps for each of 152 SMs (evaluation of
     // 128^3 x 4 chains, 4096 charges, 16 / 32 / 64 warps: 39.6 / 37.5 / 47.7 us; 40^3 x
     // 64, 500 charges 39.6 / 43.7 / 47.7)
     const int most = g.precision == COULPS_F32 ? kEvalCharges<float> : kEvalCharges<double>;
-    while (2 * A.per <= most && n_q * g.n_chains / (2 * A.per) >= 32 * 152) A.per *= 2;
+    while (!direct && 2 * A.per <= most && n_q * g.n_chains / (2 * A.per) >= 32 * 152) A.per *= 2;
     const int per_block = A.per * (kGcvThreads / 32);
     A.nblk_p = (int)((n_q + per_block - 1) / per_block);
   }
-  const cudaError_t e = g.precision == COULPS_F32 ? launch_eval<float>(g, A, s)
-                                                  : launch_eval<double>(g, A, s);
+  const cudaError_t e = g.precision == COULPS_F32 ? launch_eval<float>(g, A, direct, s)
+                                                  : launch_eval<double>(g, A, direct, s);
   if (e != cudaSuccess) return e;
   gcv_finish_kernel<<<(g.n_chains + 7) / 8, 256, 0, s>>>(partials, nblk, ppart, A.nblk_p,
                                                         g.n_chains, c0, A.nblk_p > 0 ? cP : 0.0,
