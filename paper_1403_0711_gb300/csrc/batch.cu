@@ -143,8 +143,7 @@ struct BatchHalf {
 template <typename T, bool OR, bool GATHER, int V>
 // (Compound sweeps of the 256 systems named at batch_choose_tiles, seed 7 / 3.  FP32,
 // two quads per thread: at most 80 registers, six CTAs of 128 threads per SM; it
-// takes 106 unbounded, which made 600 instead of 588 us (seed 3) with the largest
-// tiles and makes 590 / 530 instead of 595 / 532 with the chosen ones.  One quad: at
+// takes 106 unbounded, which makes 593 / 534 instead of 582 / 523.  One quad: at
 // most 64, or the heatbath's gather form takes 96 and a sweep of heatbath passes
 // only 278 / 247 instead of 265 / 234)
 __global__ void __launch_bounds__(kBatchThreads, sizeof(T) == 8 ? 1 : (V == 2 ? 3 : 4))
@@ -489,7 +488,8 @@ Tile rule_tile(const BatchSystem &S, MarchKind kind, const TileRule &r, int wide
 // tile takes its steps times the largest of a step's latency, the issue time of
 // its and its neighbours' warps and their TMA rows, and a start (tile fetch,
 // ring fill); the CTAs share the tiles evenly, and the longest tile is the least.
-double batch_time(const coulps_batch *B, MarchKind kind, const std::vector<Tile> &tiles, int sms) {
+double batch_time(const coulps_batch *B, MarchKind kind, const std::vector<Tile> &tiles, int sms,
+                  double *waves = nullptr) {
   const bool f64 = B->precision == COULPS_F64;
   const TileCost &c = kTileCost[kind][f64 ? 1 : 0];
   const int regs = f64 ? (kind == kMarchPair ? 208 : 120) : (kind == kMarchPair ? 128 : 80);
@@ -526,6 +526,7 @@ double batch_time(const coulps_batch *B, MarchKind kind, const std::vector<Tile>
       1, std::min(std::min(65536 / (regs * threads), 2048 / threads),
                   std::min((int)(228 * 1024 / (smem + 1152)), 32)));
   const double slots = (double)sms * per_sm;
+  if (waves) *waves = n / slots;
   const double others = std::max(0.0, std::min((double)per_sm, n / sms) - 1.0);
   const double warps_av = warp_steps / steps, rows_av = row_steps / steps;
   double sum = 0.0, longest = 0.0, mean = 0.0;
@@ -550,11 +551,10 @@ double batch_time(const coulps_batch *B, MarchKind kind, const std::vector<Tile>
 // SMs idle in a batch of few systems and CTAs waiting for the last, largest tiles
 // in one of more.  Measured compound sweep 1:3, largest tiles against chosen ones,
 // us: 256 cubes of 32 .. 96, 95.7M sites (inputs.batch_systems(256, 7)) 621 against
-// 596, 84.0M sites (seed 3) 561 against 532; 64 of 32 .. 80 160 against 123, 20 of
+// 582, 84.0M sites (seed 3) 561 against 523; 64 of 32 .. 80 160 against 123, 20 of
 // 37 .. 90 177 against 68, 8 of 50 .. 90 163 against 60; FP64 64 systems 2967 (with
-// the deviates by erfcinv) against 1044; heatbath only 264 against 265 and 234
-// against 234 of the 256.  Batches below 2^19 sites (a launch is its latency) keep
-// the largest tiles.
+// the deviates by erfcinv) against 1044.  Batches below 2^19 sites (a launch is its
+// latency) keep the largest tiles.
 void batch_choose_tiles(coulps_batch *B) {
   int dev = 0, sms = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
@@ -581,6 +581,15 @@ void batch_choose_tiles(coulps_batch *B) {
     const int widest = kind == kMarchPair ? pair_max : 256;
     double clear = 0.95;
     if (kind == kMarchHalf) {
+      // FP32 half-sweeps of a wave of CTAs and more keep the largest tiles: smaller
+      // ones take more halo rows and fuller warps lose lanes.  Heatbath sweeps /
+      // measured sweeps 1:3, smaller against largest tiles, of 70 random batches: at
+      // most 1.05 / 1.01 below one wave (down to 0.58 / 0.73), 0.92 .. 1.15 /
+      // 0.97 .. 1.06 from there on (256 systems, 95.7M sites, 258 / 590 against 242 /
+      // 575 us).
+      double waves = 0.0;
+      batch_time(B, kMarchHalf, tiles, sms, &waves);
+      if (B->precision == COULPS_F32 && waves >= 1.0) continue;
       // smaller than the largest tiles in any case (heatbath only, 500 systems of
       // 40, 56: 201 -> 190 us, 100 of 64^3 86.2 -> 83.7)
       for (size_t s = 0; s < tiles.size(); ++s)
