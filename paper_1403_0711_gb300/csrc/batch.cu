@@ -815,6 +815,12 @@ int batch_layout(coulps_batch *B) {
     cudaGetLastError();
     pper_sm = 1;
   }
+  // FP64 tiles that would all be resident at once, four and more on some SMs: two
+  // CTAs per SM, which take them in turn and even out (the FP64 unit is the bound;
+  // 500 systems of 12 .. 25, two passes 368 -> 216 us, 1:3 833 -> 588; with three
+  // CTAs per SM 24 systems of 59 .. 81 lose, 318 -> 395)
+  if (!f32k && (int)B->pitems.size() > 3 * sms && (int)B->pitems.size() <= sms * pper_sm)
+    pper_sm = 2;
   B->pgrid = std::max(1, std::min((int)B->pitems.size(), sms * pper_sm));
   // pair CTAs: one per SM (512 threads of over 100 registers each)
   if (pairs) {

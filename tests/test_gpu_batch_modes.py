@@ -58,3 +58,24 @@ def test_mode_is_what_runs(cl, prec, dims, default):
         s, f = run(prepare)
         assert np.abs(s - ref[0]).max() <= 1e-13 * np.abs(ref[0]).max()
         assert all(np.array_equal(x, y) for x, y in zip(f, ref[1]))
+
+
+def test_many_small_fp64_systems(cl):
+    """One pass tile per system, about four to an SM: their CTAs take them in turn."""
+    import torch
+    from paper_1403_0711_gb300 import inputs
+    rng = np.random.default_rng(4)
+    dims = [tuple(int(v) for v in rng.choice([12, 17, 25], 3)) for _ in range(500)]
+    charges = [inputs.uniform_q(d, 9, seed=k % 5) for k, d in enumerate(dims)]
+    out = []
+    for mode in (0, 1):
+        b = cl.Batch(dims, precision=cl.F64, seed=3, stream=torch.cuda.Stream())
+        b.set_fused(mode)
+        b.set_charges(charges, log_capacity=8)
+        b.sweep(1, 1, 0)
+        b.run(1, 3, 0, 2)
+        b.run(0, 2, 1, 3)
+        out.append((b.samples(), [b.field(k) for k in range(0, 500, 83)]))
+        b.close()
+    assert np.abs(out[0][0] - out[1][0]).max() <= 1e-13 * np.abs(out[0][0]).max()
+    assert all(np.array_equal(x, y) for x, y in zip(out[0][1], out[1][1]))
